@@ -62,8 +62,8 @@ lq_status alloc_field(lq_ctx* c, Field& f, SStore s) {
   if (f.data) return LQ_OK;
   f.store = s;
   LQ_CUDA(c, cudaMalloc(&f.data, spinor_bytes(s, c->geo.V)));
-  if (s == SStore::F16 || s == SStore::BF16 || s == SStore::I16)
-    LQ_CUDA(c, cudaMalloc(&f.norm, sizeof(float) * c->geo.V));
+  if (s == SStore::F16 || s == SStore::BF16 || s == SStore::I16 || s == SStore::F64)
+    LQ_CUDA(c, cudaMalloc(&f.norm, sizeof(float) * c->geo.V));     // norms; FP64: exponent words
   return LQ_OK;
 }
 
@@ -84,6 +84,29 @@ lq_status require_gauge(lq_ctx* c, int prec) {
     c->gauge_lo_valid[prec] = true;
   }
   return LQ_OK;
+}
+
+// The fixed-point links of the FP64 operator, current with the FP64 links.
+lq_status require_fix(lq_ctx* c) {
+  LQ_TRY(require_gauge(c, LQ_F64));
+  if (!c->gauge_fix) LQ_CUDA(c, cudaMalloc(&c->gauge_fix, gauge_bytes(GStore::F64_18, c->geo.V)));
+  if (!c->fix_bad) LQ_CUDA(c, cudaMalloc(&c->fix_bad, sizeof(int)));
+  if (!c->gauge_fix_valid) {
+    launch_fix_gauge(c->geo, c->gauge64, c->gauge_fix, c->fix_bad, c->stream);
+    LQ_CUDA(c, cudaGetLastError());
+    c->gauge_fix_valid = true;
+  }
+  return LQ_OK;
+}
+// The links an application of the operator in `prec` reads.
+lq_status require_links(lq_ctx* c, int prec) { return prec == LQ_F64 ? require_fix(c) : require_gauge(c, prec); }
+
+// out = M in or M^dag in with fields in the storage of prec (links current)
+void apply_M_any(lq_ctx* c, int prec, const Field& in, const Field& out, double kappa, bool dagger) {
+  if (prec == LQ_F64) apply_M64(c, in.ref(), out.ref(), kappa, dagger, c->stream);
+  else
+    apply_M_prec(c->geo, prec, c->gauge_lo[prec], in.ref(), out.ref(), kappa, dagger, c->stream, c->pair_sites,
+                 c->staged, c->df_prefetch);
 }
 
 lq_status check_prec(lq_ctx* c, int prec) {
@@ -201,6 +224,7 @@ double reliable_delta2(int inner) {
 lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int inner, int reliable_every,
                          double* hist_dev, int hist_len, lq_solve_stats* sout) {
   LQ_TRY(require_gauge(c, inner));
+  LQ_TRY(require_fix(c));
   LQ_TRY(ensure_solver_fields(c, inner));
   const Geom& g = c->geo;
   const bool mixed = inner != LQ_F64;
@@ -406,6 +430,7 @@ lq_status deliver_mom(lq_ctx* c, const double* soa, double* out) {
 
 void gauge_changed(lq_ctx* c) {
   for (int p = 0; p < kNumPrec; ++p) c->gauge_lo_valid[p] = false;
+  c->gauge_fix_valid = false;
 }
 
 // Device time of the phases of a trajectory: CUDA event pairs on the work
@@ -455,7 +480,7 @@ lq_status md_force_step(lq_ctx* c, const lq_hmc_params* hp, double eps, lq_traj_
   res->kernel_launches += s.kernel_launches + 3;
   if (st != LQ_OK) return st;
   tm.begin(PhaseTimer::kFermion);
-  apply_M_prec(c->geo, LQ_F64, c->gauge64, c->x64.ref(), c->y64.ref(), hp->kappa, false, c->stream);
+  apply_M64(c, c->x64.ref(), c->y64.ref(), hp->kappa, false, c->stream);
   launch_fermion_force(c->geo, c->gauge64, c->x64.ref(), c->y64.ref(), c->mom, hp->kappa, eps, true, c->stream);
   tm.end(PhaseTimer::kFermion);
   LQ_CUDA(c, cudaGetLastError());
@@ -489,7 +514,8 @@ lq_status trajectory_after_heatbath(lq_ctx* c, const lq_hmc_params* hp, double u
   // phi = M^dag chi; keep the start momenta and links
   LQ_CUDA(c, cudaMemcpyAsync(c->mom0, c->mom, sizeof(double) * 32 * (size_t)g.V, cudaMemcpyDeviceToDevice,
                              c->stream));
-  apply_M_prec(g, LQ_F64, c->gauge64, c->chi64.ref(), c->phi64.ref(), hp->kappa, true, c->stream);
+  LQ_TRY(require_fix(c));
+  apply_M64(c, c->chi64.ref(), c->phi64.ref(), hp->kappa, true, c->stream);
   LQ_CUDA(c, cudaMemcpyAsync(c->gauge_old, c->gauge64, gauge_bytes(GStore::F64_18, g.V), cudaMemcpyDeviceToDevice,
                              c->stream));
   r.kernel_launches += heatbath_launches + 1;
@@ -603,7 +629,7 @@ lq_status lq_create(lq_ctx** out, const int dims[4], int t_antiperiodic, void* c
   chk(cudaMalloc(&c->gauge64, gauge_bytes(GStore::F64_18, (int)V)), "cudaMalloc gauge");
   chk(cudaMalloc(&c->stage_in, spin), "cudaMalloc stage");
   chk(cudaMalloc(&c->stage_out, spin), "cudaMalloc stage");
-  c->rs.max_blocks = (int)((V + 63) / 64) + 1;
+  c->rs.max_blocks = (int)((V + 15) / 16) + 1;       // the smallest blocks of any reducing kernel hold 16 sites
   chk(cudaMalloc(&c->rs.partials, sizeof(double) * 4 * c->rs.max_blocks), "cudaMalloc partials");
   chk(cudaMalloc(&c->rs.ticket, sizeof(unsigned int) * 4), "cudaMalloc ticket");
   if (st == LQ_OK) chk(cudaMemset(c->rs.ticket, 0, sizeof(unsigned int) * 4), "cudaMemset");
@@ -629,6 +655,8 @@ lq_status lq_destroy(lq_ctx* c) {
   for (cudaEvent_t e : c->phase_ev)
     if (e) cudaEventDestroy(e);
   if (c->gauge64) cudaFree(c->gauge64);
+  if (c->gauge_fix) cudaFree(c->gauge_fix);
+  if (c->fix_bad) cudaFree(c->fix_bad);
   for (int p = 0; p < kNumPrec; ++p)
     if (c->gauge_lo[p]) cudaFree(c->gauge_lo[p]);
   if (c->stage_in) cudaFree(c->stage_in);
@@ -710,7 +738,7 @@ lq_status lq_gauge_set(lq_ctx* c, const double* U) {
   }
   launch_pack_gauge64(c->geo, src, c->gauge64, c->stream);
   LQ_CUDA(c, cudaGetLastError());
-  for (int p = 0; p < kNumPrec; ++p) c->gauge_lo_valid[p] = false;
+  gauge_changed(c);
   c->gauge_set = true;
   if (!is_device_ptr(U)) LQ_CUDA(c, cudaStreamSynchronize(c->stream));   // the host buffer may be reused at once
   return LQ_OK;
@@ -744,7 +772,7 @@ lq_status lq_gauge_get(lq_ctx* c, double* U) {
 lq_status lq_apply_M(lq_ctx* c, double* out, const double* in, double kappa, int dagger, int prec) {
   if (!c) return LQ_ERR_ARG;
   LQ_TRY(check_prec(c, prec));
-  LQ_TRY(require_gauge(c, prec));
+  LQ_TRY(require_links(c, prec));
   if (in == out) return fail(c, LQ_ERR_ARG, "in and out must not overlap");
   const SStore s = spinor_store_of(prec);
   Field& fin = (prec == LQ_F64) ? c->phi64 : c->p_lo[(int)s];
@@ -754,9 +782,7 @@ lq_status lq_apply_M(lq_ctx* c, double* out, const double* in, double kappa, int
   const double* din = nullptr;
   LQ_TRY(stage_spinor_in(c, in, &din));
   launch_pack_spinor(c->geo, din, s, fin.ref(), c->stream);
-  const void* gauge = prec == LQ_F64 ? c->gauge64 : c->gauge_lo[prec];
-  apply_M_prec(c->geo, prec, gauge, fin.ref(), fout.ref(), kappa, dagger != 0, c->stream, c->pair_sites, c->staged,
-               c->df_prefetch);
+  apply_M_any(c, prec, fin, fout, kappa, dagger != 0);
   LQ_CUDA(c, cudaGetLastError());
   return deliver_spinor(c, fout, out);
 }
@@ -764,7 +790,7 @@ lq_status lq_apply_M(lq_ctx* c, double* out, const double* in, double kappa, int
 lq_status lq_apply_MdagM(lq_ctx* c, double* out, const double* in, double kappa, int prec) {
   if (!c) return LQ_ERR_ARG;
   LQ_TRY(check_prec(c, prec));
-  LQ_TRY(require_gauge(c, prec));
+  LQ_TRY(require_links(c, prec));
   if (in == out) return fail(c, LQ_ERR_ARG, "in and out must not overlap");
   const SStore s = spinor_store_of(prec);
   Field& fin = (prec == LQ_F64) ? c->phi64 : c->p_lo[(int)s];
@@ -776,11 +802,8 @@ lq_status lq_apply_MdagM(lq_ctx* c, double* out, const double* in, double kappa,
   const double* din = nullptr;
   LQ_TRY(stage_spinor_in(c, in, &din));
   launch_pack_spinor(c->geo, din, s, fin.ref(), c->stream);
-  const void* gauge = prec == LQ_F64 ? c->gauge64 : c->gauge_lo[prec];
-  apply_M_prec(c->geo, prec, gauge, fin.ref(), fmid.ref(), kappa, false, c->stream, c->pair_sites, c->staged,
-               c->df_prefetch);
-  apply_M_prec(c->geo, prec, gauge, fmid.ref(), fout.ref(), kappa, true, c->stream, c->pair_sites, c->staged,
-               c->df_prefetch);
+  apply_M_any(c, prec, fin, fmid, kappa, false);
+  apply_M_any(c, prec, fmid, fout, kappa, true);
   LQ_CUDA(c, cudaGetLastError());
   return deliver_spinor(c, fout, out);
 }
@@ -839,7 +862,7 @@ lq_status lq_time_dslash(lq_ctx* c, const double* in, double kappa, int dagger, 
   if (!c) return LQ_ERR_ARG;
   if (!ms || n <= 0) return fail(c, LQ_ERR_ARG, "need n > 0 and an output pointer");
   LQ_TRY(check_prec(c, prec));
-  LQ_TRY(require_gauge(c, prec));
+  LQ_TRY(require_links(c, prec));
   const SStore s = spinor_store_of(prec);
   Field& fin = (prec == LQ_F64) ? c->phi64 : c->p_lo[(int)s];
   Field& fout = (prec == LQ_F64) ? c->tmp64 : c->t_lo[(int)s];
@@ -848,23 +871,20 @@ lq_status lq_time_dslash(lq_ctx* c, const double* in, double kappa, int dagger, 
   const double* din = nullptr;
   LQ_TRY(stage_spinor_in(c, in, &din));
   launch_pack_spinor(c->geo, din, s, fin.ref(), c->stream);
-  const void* gauge = prec == LQ_F64 ? c->gauge64 : c->gauge_lo[prec];
   const size_t flush_bytes = (size_t)256 << 20;
   void* flush = nullptr;
   if (flush_l2) LQ_CUDA(c, cudaMallocAsync(&flush, flush_bytes, c->stream));
   cudaEvent_t e0, e1;
   LQ_CUDA(c, cudaEventCreate(&e0));
   LQ_CUDA(c, cudaEventCreate(&e1));
-  apply_M_prec(c->geo, prec, gauge, fin.ref(), fout.ref(), kappa, dagger != 0, c->stream, c->pair_sites, c->staged,
-               c->df_prefetch);   // warm-up
+  apply_M_any(c, prec, fin, fout, kappa, dagger != 0);   // warm-up
   double total = 0.0;
   lq_status st = LQ_OK;
   if (flush_l2) {
     for (int i = 0; i < n && st == LQ_OK; ++i) {
       cudaMemsetAsync(flush, i & 0xff, flush_bytes, c->stream);
       cudaEventRecord(e0, c->stream);
-      apply_M_prec(c->geo, prec, gauge, fin.ref(), fout.ref(), kappa, dagger != 0, c->stream, c->pair_sites, c->staged,
-               c->df_prefetch);
+      apply_M_any(c, prec, fin, fout, kappa, dagger != 0);
       cudaEventRecord(e1, c->stream);
       st = cuda_check(c, cudaEventSynchronize(e1), "cudaEventSynchronize");
       float t = 0.f;
@@ -874,8 +894,7 @@ lq_status lq_time_dslash(lq_ctx* c, const double* in, double kappa, int dagger, 
   } else {
     cudaEventRecord(e0, c->stream);
     for (int i = 0; i < n; ++i)
-      apply_M_prec(c->geo, prec, gauge, fin.ref(), fout.ref(), kappa, dagger != 0, c->stream, c->pair_sites, c->staged,
-               c->df_prefetch);
+      apply_M_any(c, prec, fin, fout, kappa, dagger != 0);
     cudaEventRecord(e1, c->stream);
     st = cuda_check(c, cudaEventSynchronize(e1), "cudaEventSynchronize");
     float t = 0.f;
@@ -929,7 +948,8 @@ lq_status lq_fermion_force(lq_ctx* c, double* F, const double* X, double kappa) 
   const double* dX = nullptr;
   LQ_TRY(stage_spinor_in(c, X, &dX));
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
-  apply_M_prec(c->geo, LQ_F64, c->gauge64, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
+  LQ_TRY(require_fix(c));
+  apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
   launch_fermion_force(c->geo, c->gauge64, c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
   LQ_CUDA(c, cudaGetLastError());
   return deliver_mom(c, c->force, F);
@@ -944,7 +964,8 @@ lq_status lq_fermion_grad(lq_ctx* c, double* G, const double* X, double kappa) {
   const double* dX = nullptr;
   LQ_TRY(stage_spinor_in(c, X, &dX));
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
-  apply_M_prec(c->geo, LQ_F64, c->gauge64, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
+  LQ_TRY(require_fix(c));
+  apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
   const size_t bytes = sizeof(double) * 72 * (size_t)c->geo.V;
   if (is_device_ptr(G)) {
     launch_fermion_grad(c->geo, c->x64.ref(), c->y64.ref(), G, kappa, c->stream);
@@ -1137,7 +1158,8 @@ lq_status lq_time_fermion_force(lq_ctx* c, const double* X, double kappa, int n,
   const double* dX = nullptr;
   LQ_TRY(stage_spinor_in(c, X, &dX));
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
-  apply_M_prec(c->geo, LQ_F64, c->gauge64, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
+  LQ_TRY(require_fix(c));
+  apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
   launch_fermion_force(c->geo, c->gauge64, c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -1160,7 +1182,7 @@ lq_status lq_time_cg_kernel(lq_ctx* c, const double* in, double kappa, int which
   if (!c) return LQ_ERR_ARG;
   if (!ms || n <= 0 || which < 0 || which > 3) return fail(c, LQ_ERR_ARG, "need 0 <= which <= 3, n > 0, ms");
   LQ_TRY(check_inner(c, prec));
-  LQ_TRY(require_gauge(c, LQ_F64));
+  LQ_TRY(require_links(c, LQ_F64));
   LQ_TRY(require_gauge(c, prec));
   LQ_TRY(ensure_solver_fields(c, prec));
   const Geom& g = c->geo;

@@ -3,6 +3,7 @@
 #include "lq_internal.h"
 #include "lq_staged.cuh"
 #include "lq_dfsplit.cuh"
+#include "lq_fix64.cuh"
 
 namespace lq {
 
@@ -22,6 +23,17 @@ static void apply_one(const Geom& g, const void* gauge, SpinorRef in, SpinorRef 
   else launch_dslash<T, G, S, false>(g, GaugeRef{gauge}, in, kappa, epi, none, stream);
 }
 
+FixGauge fix_gauge_of(const lq_ctx* c) {
+  return FixGauge{static_cast<const int4*>(c->gauge_fix), static_cast<const double2*>(c->gauge64), c->fix_bad};
+}
+
+void apply_M64(const lq_ctx* c, SpinorRef in, SpinorRef out, double kappa, bool dagger, cudaStream_t stream) {
+  FixEpiStore epi{out};
+  ReduceScratch none{nullptr, nullptr, 0};
+  if (dagger) launch_dslash_fix<true>(c->geo, fix_gauge_of(c), in, kappa, epi, none, stream);
+  else launch_dslash_fix<false>(c->geo, fix_gauge_of(c), in, kappa, epi, none, stream);
+}
+
 void apply_M_prec(const Geom& g, int prec, const void* gauge, SpinorRef in, SpinorRef out, double kappa,
                   bool dagger, cudaStream_t stream, bool pair, bool staged, bool df_prefetch) {
   if (pair && prec == LQ_I16_12 && pair_geometry(g)) {
@@ -29,7 +41,6 @@ void apply_M_prec(const Geom& g, int prec, const void* gauge, SpinorRef in, Spin
     return;
   }
   switch (prec) {
-    case LQ_F64: apply_one<double, GStore::F64_18, SStore::F64>(g, gauge, in, out, kappa, dagger, stream); break;
     case LQ_F32: apply_one<float, GStore::F32_18, SStore::F32>(g, gauge, in, out, kappa, dagger, stream, staged); break;
     case LQ_F32_12: apply_one<float, GStore::F32_12, SStore::F32>(g, gauge, in, out, kappa, dagger, stream, staged); break;
     case LQ_F16_12: apply_one<float, GStore::F16_12, SStore::F16>(g, gauge, in, out, kappa, dagger, stream, staged); break;

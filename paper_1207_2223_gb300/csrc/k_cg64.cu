@@ -4,57 +4,50 @@
 //   k2  r -= alpha M^dag t, x += alpha p, rr = |r|^2, beta
 //   k3  p = r + beta p
 // and the FP64 true residual r = phi - M^dag (M x) used to stop the solve
-// and, for mixed-precision solves, as the reliable update.
+// and, for mixed-precision solves, as the reliable update.  The operator is
+// the fixed-point one of lq_fix64.cuh.
 #include "lq_internal.h"
+#include "lq_fix64.cuh"
 
 namespace lq {
 
 void cg64_step(lq_ctx* c, int which, double kappa, cudaStream_t stream) {
-  const Geom& g = c->geo;
-  GaugeRef U{c->gauge64};
+  const FixGauge U = fix_gauge_of(c);
   if (which == 1) {
-    EpiCG1<SStore::F64> e1{c->t64.ref(), c->state};
-    launch_dslash<double, GStore::F64_18, SStore::F64, false>(g, U, c->p64.ref(), kappa, e1, c->rs, stream);
+    FixEpiCG1 e1{{c->t64.ref(), c->state}};
+    launch_dslash_fix<false>(c->geo, U, c->p64.ref(), kappa, e1, c->rs, stream);
   } else {
-    EpiCG2<SStore::F64, SStore::F64, SStore::F64> e2{c->r64.ref(), c->x64.ref(), c->p64.ref(), c->state};
-    launch_dslash<double, GStore::F64_18, SStore::F64, true>(g, U, c->t64.ref(), kappa, e2, c->rs, stream);
+    FixEpiCG2 e2{{c->r64.ref(), c->x64.ref(), c->p64.ref(), c->state}};
+    launch_dslash_fix<true>(c->geo, U, c->t64.ref(), kappa, e2, c->rs, stream);
   }
 }
 
 void cg64_iteration(lq_ctx* c, double kappa, cudaStream_t stream) {
-  const Geom& g = c->geo;
-  GaugeRef U{c->gauge64};
-  EpiCG1<SStore::F64> e1{c->t64.ref(), c->state};
-  launch_dslash<double, GStore::F64_18, SStore::F64, false>(g, U, c->p64.ref(), kappa, e1, c->rs, stream);
-  EpiCG2<SStore::F64, SStore::F64, SStore::F64> e2{c->r64.ref(), c->x64.ref(), c->p64.ref(), c->state};
-  launch_dslash<double, GStore::F64_18, SStore::F64, true>(g, U, c->t64.ref(), kappa, e2, c->rs, stream);
-  launch_xpay_p(g, SStore::F64, c->r64.ref(), c->p64.ref(), c->state, false, stream);
+  cg64_step(c, 1, kappa, stream);
+  cg64_step(c, 2, kappa, stream);
+  launch_xpay_p(c->geo, SStore::F64, c->r64.ref(), c->p64.ref(), c->state, false, stream);
 }
 
-template <SStore SLO>
-static void residual_lo(lq_ctx* c, double kappa, SpinorRef rlo, cudaStream_t stream) {
-  EpiResidual<SLO, true> e{c->phi64.ref(), c->r64.ref(), rlo, c->state};
-  launch_dslash<double, GStore::F64_18, SStore::F64, true>(c->geo, GaugeRef{c->gauge64}, c->tmp64.ref(), kappa, e,
-                                                           c->rs, stream);
+template <SStore SLO, bool STORE_LO>
+static void residual(lq_ctx* c, double kappa, SpinorRef rlo, cudaStream_t stream) {
+  FixEpiResidual<SLO, STORE_LO> e{c->phi64.ref(), c->r64.ref(), rlo, FinSolver{c->state}};
+  launch_dslash_fix<true>(c->geo, fix_gauge_of(c), c->tmp64.ref(), kappa, e, c->rs, stream);
 }
 
 void cg64_true_residual(lq_ctx* c, double kappa, int store_lo_prec, cudaStream_t stream) {
-  const Geom& g = c->geo;
-  GaugeRef U{c->gauge64};
-  EpiStore<SStore::F64> e0{c->tmp64.ref()};
-  launch_dslash<double, GStore::F64_18, SStore::F64, false>(g, U, c->x64.ref(), kappa, e0, c->rs, stream);
+  FixEpiStore e0{c->tmp64.ref()};
+  launch_dslash_fix<false>(c->geo, fix_gauge_of(c), c->x64.ref(), kappa, e0, c->rs, stream);
   if (store_lo_prec == LQ_F64) {
-    EpiResidual<SStore::F64, false> e{c->phi64.ref(), c->r64.ref(), SpinorRef{nullptr, nullptr}, c->state};
-    launch_dslash<double, GStore::F64_18, SStore::F64, true>(g, U, c->tmp64.ref(), kappa, e, c->rs, stream);
+    residual<SStore::F64, false>(c, kappa, SpinorRef{nullptr, nullptr}, stream);
     return;
   }
   const SStore slo = spinor_store_of(store_lo_prec);
   SpinorRef rlo = c->r_lo[(int)slo].ref();
   switch (slo) {
-    case SStore::F32: residual_lo<SStore::F32>(c, kappa, rlo, stream); break;
-    case SStore::F16: residual_lo<SStore::F16>(c, kappa, rlo, stream); break;
-    case SStore::BF16: residual_lo<SStore::BF16>(c, kappa, rlo, stream); break;
-    case SStore::I16: residual_lo<SStore::I16>(c, kappa, rlo, stream); break;
+    case SStore::F32: residual<SStore::F32, true>(c, kappa, rlo, stream); break;
+    case SStore::F16: residual<SStore::F16, true>(c, kappa, rlo, stream); break;
+    case SStore::BF16: residual<SStore::BF16, true>(c, kappa, rlo, stream); break;
+    case SStore::I16: residual<SStore::I16, true>(c, kappa, rlo, stream); break;
     default: break;
   }
 }

@@ -46,9 +46,13 @@ __global__ void __launch_bounds__(kBS) momenta_kernel(int V, uint32_t seed, uint
 
 // One thread per site: the 12 complex components of chi into the FP64 spinor
 // field (double2 [12][V]) and, when canon != null, the canonical [V][4][3] complex.
-__global__ void __launch_bounds__(kBS) chi_kernel(int V, uint32_t seed, uint32_t traj, double2* soa, double2* canon) {
+// ex, when not null: the exponent word of each site (the operator reads it with the field).
+__global__ void __launch_bounds__(kBS) chi_kernel(int V, uint32_t seed, uint32_t traj, double2* soa, int* ex,
+                                                  double2* canon) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= V) return;
+  ExpRange range;
+  cplx<double> spin[3] = {};
   for (int k = 0; k < 12; ++k) {
     const rng::Words w = rng::philox4x32_10((uint32_t)s, traj, (uint32_t)k, 0u, seed, kStreamChi);
     double z0, z1;
@@ -56,7 +60,12 @@ __global__ void __launch_bounds__(kBS) chi_kernel(int V, uint32_t seed, uint32_t
     const double2 v = make_double2(rng::mul(z0, rng::kSqrtHalf), rng::mul(z1, rng::kSqrtHalf));
     if (soa) soa[(size_t)k * V + s] = v;
     if (canon) canon[(size_t)s * 12 + k] = v;
+    spin[0] = spin[1];
+    spin[1] = spin[2];
+    spin[2] = {v.x, v.y};
+    if (k % 3 == 2) range.spin(spin);
   }
+  if (ex) ex[s] = range.word();
 }
 
 __global__ void __launch_bounds__(kBS) philox_kernel(int n, const uint32_t* in, uint32_t* out) {
@@ -88,7 +97,8 @@ void launch_heatbath_momenta(const Geom& g, uint64_t seed, uint64_t traj, double
 
 void launch_heatbath_chi(const Geom& g, uint64_t seed, uint64_t traj, SpinorRef soa, double* canon, cudaStream_t st) {
   chi_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g.V, (uint32_t)seed, (uint32_t)traj,
-                                                 static_cast<double2*>(soa.p), reinterpret_cast<double2*>(canon));
+                                                 static_cast<double2*>(soa.p), reinterpret_cast<int*>(soa.norm),
+                                                 reinterpret_cast<double2*>(canon));
 }
 
 double metropolis_uniform(uint64_t seed, uint64_t traj) {

@@ -2,6 +2,7 @@
 // C interface ([site][mu][3][3] links, [site][spin][colour] spinors) and the
 // internal site-major structure-of-arrays formats of lq_device.cuh.
 #include "lq_internal.h"
+#include "lq_fix64.cuh"
 
 namespace lq {
 
@@ -13,6 +14,13 @@ int resident_grid(const void* kernel, int block) {
   if (sms <= 0) sms = 1;
   if (per_sm <= 0) per_sm = 1;
   return sms * per_sm;
+}
+
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 0 ? sms : 1;
 }
 
 size_t spinor_bytes(SStore s, int V) {
@@ -118,6 +126,31 @@ __global__ void convert_gauge_kernel(int V, const double2* __restrict__ soa64, v
   }
 }
 
+// FP64 links as fixed point for the operator (lq_fix64.cuh), one thread per link.  *bad is
+// set when a row or a column of a link is longer than 1 by more than 1e-3 (or not finite):
+// the bounds that keep the fixed-point sums in range assume unitary links.
+__global__ void __launch_bounds__(256) fix_gauge_kernel(int V, const double2* __restrict__ soa64, int4* __restrict__ out,
+                                                        int* __restrict__ bad) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= 4 * V) return;
+  const int mu = idx / V, s = idx - mu * V;
+  const double2* p = soa64 + (size_t)mu * 9 * V + s;
+  int4* o = out + (size_t)mu * 9 * V + s;
+  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const double2 u = p[(size_t)k * V];
+    const float a = (float)u.x, b = (float)u.y, n = a * a + b * b;
+    row[k / 3] += n;
+    col[k % 3] += n;
+    o[(size_t)k * V] = fix_link(u);
+  }
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 1.001f && col[k] <= 1.001f;
+  if (!ok) *bad = 1;
+}
+
 template <SStore S>
 __global__ void __launch_bounds__(kSpinTile) pack_spinor_kernel(int V, const double2* __restrict__ canon,
                                                                 SpinorRef out) {
@@ -161,6 +194,11 @@ static constexpr int kBS = 256;
 void launch_pack_gauge64(const Geom& g, const double* canon, void* soa, cudaStream_t st) {
   pack_gauge64_kernel<<<grid_for(g.V, kGaugeTile), 256, 0, st>>>(g.V, reinterpret_cast<const double2*>(canon),
                                                                   static_cast<double2*>(soa));
+}
+void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* bad, cudaStream_t st) {
+  cudaMemsetAsync(bad, 0, sizeof(int), st);
+  fix_gauge_kernel<<<grid_for(4 * g.V, 256), 256, 0, st>>>(g.V, static_cast<const double2*>(soa64),
+                                                            static_cast<int4*>(fix), bad);
 }
 void launch_unpack_gauge64(const Geom& g, const void* soa, double* canon, cudaStream_t st) {
   unpack_gauge64_kernel<<<grid_for(g.V, kGaugeTile), 256, 0, st>>>(g.V, static_cast<const double2*>(soa),

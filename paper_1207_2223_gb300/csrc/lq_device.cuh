@@ -100,7 +100,7 @@ template <> __device__ __forceinline__ df64 to_df<df64>(df64 v) { return v; }
 
 struct SpinorRef {           // device view of one spinor field
   void* p;                   // chunk array
-  float* norm;               // per-site norm (F16 / BF16 only)
+  float* norm;               // per-site norm (16-bit formats); FP64: exponent words (int), may be null
 };
 struct GaugeRef {
   const void* p;
@@ -237,6 +237,32 @@ __device__ __forceinline__ T load_spinor_raw(const SpinorRef& f, int V, int s, c
   }
 }
 
+// Exponent word of a site of an FP64 field: what the fixed-point operator (lq_fix64.cuh)
+// has to know of a neighbour before it reads it.  Bits 0-10: the largest biased exponent of
+// the site's components (0 for a zero site); kFixSlow: the site needs FP64 arithmetic
+// (non-finite values, values below 2^-953, or a spin more than 2^6 below the largest, whose
+// last bits one scale for the site would cost).
+constexpr int kFixMinExp = 70;
+constexpr int kFixSlow = 1 << 16;
+struct ExpRange {
+  int mx = 0, mn = 0x7fffffff, lo = 0;     // largest and smallest spin (high words), all low words or-ed
+  __device__ __forceinline__ void spin(const cplx<double> v[3]) {
+    int m = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      m = max(m, max(__double2hiint(v[c].re) & 0x7fffffff, __double2hiint(v[c].im) & 0x7fffffff));
+      lo |= __double2loint(v[c].re) | __double2loint(v[c].im);
+    }
+    mx = max(mx, m);
+    mn = min(mn, m);
+  }
+  __device__ __forceinline__ int word() const {
+    const int E = mx >> 20, e = mn >> 20;
+    if (mx == 0 && lo == 0) return 0;
+    return E | (E < kFixMinExp || E == 0x7ff || e < E - 6 ? kFixSlow : 0);
+  }
+};
+
 template <SStore S, typename T>
 __device__ __forceinline__ void store_spinor(const SpinorRef& f, int V, int s, const cplx<T> v[12]) {
   if constexpr (S == SStore::DF64) {
@@ -250,6 +276,17 @@ __device__ __forceinline__ void store_spinor(const SpinorRef& f, int V, int s, c
     double2* p = static_cast<double2*>(f.p);
 #pragma unroll
     for (int c = 0; c < 12; ++c) p[(size_t)c * V + s] = make_double2((double)v[c].re, (double)v[c].im);
+    if (f.norm) {
+      ExpRange r;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        cplx<double> w[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) w[c] = {(double)v[3 * k + c].re, (double)v[3 * k + c].im};
+        r.spin(w);
+      }
+      reinterpret_cast<int*>(f.norm)[s] = r.word();
+    }
   } else if constexpr (S == SStore::F32) {
     float4* p = static_cast<float4*>(f.p);
 #pragma unroll

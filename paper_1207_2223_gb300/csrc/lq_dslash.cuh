@@ -316,6 +316,7 @@ inline int grid_for(int V, int bs) { return (V + bs - 1) / bs; }
 
 // Resident blocks of one kernel on the current device (queried once per kernel).
 int resident_grid(const void* kernel, int block);
+int sm_count();                        // SMs of the current device
 
 // A lattice with fewer full blocks (one site per thread) than half a wave leaves SMs idle;
 // it runs in blocks of half the size, which spread over twice as many SMs (measured: 8^4

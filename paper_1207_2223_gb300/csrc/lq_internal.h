@@ -76,6 +76,9 @@ struct lq_ctx {
   void* gauge_lo[lq::kNumPrec] = {};
   bool gauge_lo_valid[lq::kNumPrec] = {};
   bool gauge_set = false;
+  void* gauge_fix = nullptr;             // fixed-point links of the FP64 operator (lq_fix64.cuh), built lazily
+  int* fix_bad = nullptr;                // device flag: some link is not unitary
+  bool gauge_fix_valid = false;
 
   // canonical-layout staging buffers (device)
   double* stage_in = nullptr;            // V * 24 doubles
@@ -137,6 +140,7 @@ void destroy_batch_work(void* w);
 // ---- layout (k_layout.cu)
 void launch_pack_gauge64(const Geom& g, const double* canon, void* soa, cudaStream_t st);
 void launch_unpack_gauge64(const Geom& g, const void* soa, double* canon, cudaStream_t st);
+void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* bad, cudaStream_t st);
 void launch_convert_gauge(const Geom& g, const void* soa64, GStore dst, void* out, cudaStream_t st);
 void launch_pack_spinor(const Geom& g, const double* canon, SStore s, SpinorRef out, cudaStream_t st);
 void launch_unpack_spinor(const Geom& g, SStore s, SpinorRef in, double* canon, cudaStream_t st);
@@ -160,6 +164,9 @@ void launch_inner_restart(const Geom& g, SpinorRef src64, SStore s, SpinorRef x,
                           cudaStream_t stream);
 
 // ---- Wilson operator applications (k_apply.cu): out = M in or M^dag in
+// FP64, by the fixed-point operator (the context's fixed-point links must be current)
+void apply_M64(const lq_ctx* c, SpinorRef in, SpinorRef out, double kappa, bool dagger, cudaStream_t stream);
+// the other precisions
 // (pair: the two-site packed stencil where it applies, 16-bit fixed point)
 // (staged: the stencil that shares x and y links inside a block through shared memory,
 // FP32-arithmetic formats)

@@ -1,0 +1,88 @@
+"""The fixed-point FP64 operator (csrc/lq_fix64.cuh): the forms its rules send to different paths."""
+import numpy as np
+import pytest
+
+from oracle.wilson import apply_M
+from synth import Lattice, gauge_exp_iA, source
+from tests.gpu_common import require_gpu, dev, host, torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lq():
+    return require_gpu()
+
+
+def _apply(lq, dims, U, psi, dagger, t_anti=True):
+    ctx = lq.lq_create(dims, t_anti)
+    try:
+        lq.lq_gauge_set(ctx, dev(U))
+        out = torch.empty(psi.shape, dtype=torch.complex128, device="cuda")
+        lq.lq_apply_M(ctx, out, dev(psi), 0.15, dagger, lq.LQ_F64)
+        return host(out)
+    finally:
+        lq.lq_destroy(ctx)
+
+
+def _fields(dims, kind):
+    """Spinors (and links) that reach one rule each."""
+    lat = Lattice(dims)
+    U, psi = gauge_exp_iA(lat, 0.3, 6), source(lat, 6)
+    rng = np.random.default_rng(6)
+    if kind == "site_range":            # neighbours of very different size: one exponent for eight of them
+        psi = psi * np.exp(rng.normal(0, 12, (lat.V, 1, 1)))
+    elif kind == "spin_range":          # spins more than 2^6 apart: FP64 arithmetic
+        psi[::3, 1] *= 1e-7
+    elif kind == "point":               # one non-zero component
+        psi = np.zeros_like(psi)
+        psi[lat.V // 2, 2, 1] = 1.0 - 2.0j
+    elif kind == "tiny":                # below the smallest exponent the fixed-point path takes
+        psi = psi * 2.0 ** -1000
+    elif kind == "huge":
+        psi = psi * 2.0 ** 1000
+    elif kind == "ones":                # limb edges: links of exactly 1, powers of two
+        U = np.tile(np.eye(3, dtype=np.complex128), (lat.V, 4, 1, 1))
+        psi = np.sign(psi.real) + 1j * np.sign(psi.imag)
+    elif kind == "not_unitary":         # general matrices: FP64 arithmetic at every site
+        U = U * (1.5 + 0.1 * rng.normal(size=(lat.V, 4, 1, 1)))
+    return U, psi
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7), (16, 12, 12, 18)])
+@pytest.mark.parametrize("kind", ["gauss", "site_range", "spin_range", "point", "tiny", "huge", "ones", "not_unitary"])
+@pytest.mark.parametrize("dagger", [False, True])
+def test_matches_oracle_element_by_element(lq, dims, kind, dagger):
+    """(16, 12, 12, 18) has more blocks than SMs (the capped kernel), the others fewer.  Bound per
+    element: 8 hops, each rounding FP64 products and sums of the components one site reads, at most
+    64 units of 2^-53 of the largest of them (the fixed-point path keeps 2^-56 of it), times the
+    largest link element."""
+    U, psi = _fields(dims, kind)
+    scale = 1.0
+    if kind in ("tiny", "huge"):        # the oracle's own sums at a scale without underflow
+        scale = 2.0 ** (-1000 if kind == "tiny" else 1000)
+    ref = apply_M(U, psi / scale, dims, 0.15, True, dagger)
+    got = _apply(lq, dims, U, psi, dagger) / scale
+    lat = Lattice(dims)
+    a = np.abs(psi / scale).max(axis=(1, 2)).reshape(dims[::-1])
+    near = a.copy()
+    for ax in range(4):
+        near = np.maximum(near, np.maximum(np.roll(a, 1, ax), np.roll(a, -1, ax)))
+    tol = 64 * 2.0 ** -53 * max(1.0, np.abs(U).max()) * near.reshape(lat.V, 1, 1)
+    assert np.all(np.abs(got - ref) <= tol)
+    assert np.all(got[ref == 0] == 0)
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_non_finite_values_reach_their_neighbours_only(lq, value):
+    dims = (4, 6, 4, 4)
+    lat = Lattice(dims)
+    U, psi = gauge_exp_iA(lat, 0.3, 6), source(lat, 6)
+    s = 77
+    psi[s, 0, 0] = value
+    got = _apply(lq, dims, U, psi, False)
+    finite = np.isfinite(got).all(axis=(1, 2))
+    x = lat.coords()
+    d = np.abs(x - x[s])
+    d = np.minimum(d, np.array(dims) - d).sum(axis=1)
+    assert np.array_equal(finite, d > 1)
