@@ -8,9 +8,8 @@ is solved from x0 = 0 to an FP64 true relative residual of 1e-10.
 
 One step = one mixed-precision solve (inner precision --inner, default FP16
 storage with 12-real links and per-site FP32 norms, FP32 arithmetic, reliable
-updates every 50 iterations: the intermediate ones in double-float arithmetic,
-the last recomputed and certified in FP64; the all-FP64-update solve is
-reported beside it).  Printed as one JSON line:
+updates every 50 iterations, each the FP64 true residual).  Printed as one
+JSON line:
   value         solves per second over all ranks (device-timed, data resident)
   e2e           the same through the C interface with pinned host buffers
                 (gauge field and source copied in, solution copied out, every step)
@@ -617,9 +616,6 @@ def run_kernel_only(args):
     if args.kernel_only == "batch":
         import numpy as np
         R = 12
-        # the profiled passes are the inner-format iterations; FP64 reliable updates keep the
-        # device footprint small (no double-float fields)
-        lq.lq_set_option(ctx, lq.LQ_OPT_DF64_UPDATES, 0)
         phis = torch.from_numpy(np.stack([source(lat, SEED, i) for i in range(R)])).cuda()
         x = torch.zeros_like(phis)
         t0 = time.perf_counter()
@@ -700,19 +696,6 @@ def run_ours(args):
             others[name] = {"seconds": q0.elapsed_time(q1) / 1e3, "iterations": sto["iterations"],
                             "reliable_updates": sto["reliable_updates"], "escalations": sto["escalations"]}
 
-        # the same mixed solve with every reliable update in FP64 (the default does the
-        # intermediate ones in double-float arithmetic and certifies the last in FP64)
-        lq.lq_set_option(ctx, lq.LQ_OPT_DF64_UPDATES, 0)
-        solve(inner)
-        t0 = torch.cuda.Event(enable_timing=True)
-        t1 = torch.cuda.Event(enable_timing=True)
-        t0.record(stream)
-        st_fp64ru = solve(inner)
-        t1.record(stream)
-        torch.cuda.synchronize(dev)
-        mixed_fp64ru_s = t0.elapsed_time(t1) / 1e3
-        lq.lq_set_option(ctx, lq.LQ_OPT_DF64_UPDATES, 1)
-
         # plain FP64 CG on the same source: the comparison of the metric
         t0 = torch.cuda.Event(enable_timing=True)
         t1 = torch.cuda.Event(enable_timing=True)
@@ -732,11 +715,11 @@ def run_ours(args):
             gbs = DSLASH_BYTES[name] * V / (ms * 1e-3) / 1e9
             dsl[name] = {"ms": round(ms, 5), "GB/s": round(gbs, 1), "frac_hbm": round(gbs / hbm, 4),
                          "GFLOP/s": round(DSLASH_FLOPS * V / (ms * 1e-3) / 1e9, 1)}
-        # the FP64 operator is bound by the FP64 pipe: its roofline is the measured FP64
-        # fused multiply-add rate of this GPU (FP32 rate for comparison)
+        # the FP64 operator runs on the integer pipe (lq_fix64.cuh): its rate beside the measured
+        # FP64 fused multiply-add rate of this GPU, which bounds FP64 arithmetic (frac above 1)
         fma = {"f64_tflops": lq.lq_time_fma_peak(ctx, lq.LQ_F64), "f32_tflops": lq.lq_time_fma_peak(ctx, lq.LQ_F32)}
         d64 = dsl["f64"]
-        fp64_roofline = {"kernel": "dslash_kernel<f64> (M)", "bound": "alu",
+        fp64_roofline = {"kernel": "dslash_fix_kernel (M, FP64 fields)", "bound": "alu",
                          "achieved": round(d64["GFLOP/s"] / 1e3, 4), "peak": round(fma["f64_tflops"], 4),
                          "unit": "TFLOP/s", "frac": round(d64["GFLOP/s"] / 1e3 / fma["f64_tflops"], 4),
                          "peak_kind": "measured (lq_time_fma_peak: FP64 fused multiply-add chains)",
@@ -854,15 +837,11 @@ def run_ours(args):
             "data": "synthetic",
             "config": {"workload": WORKLOAD, "dims": list(DIMS), "kappa": KAPPA, "sigma": SIGMA, "seed": SEED,
                        "tol": TOL, "inner": args.inner, "reliable_every": RELIABLE,
-                       "reliable_updates": "intermediate in double-float (FP32 pipe, ~48 bits), the last "
-                                           "recomputed and certified in FP64",
+                       "reliable_updates": "FP64 true residual (fixed-point FP64 operator)",
                        "l2": "working set larger than L2 (gauge %d MB + spinors), no flush"
                              % (DSLASH_BYTES[args.inner] * V // 3 // 2**20),
                        "parallelism": "replicas" if size > 1 else "single"},
             "time_to_solution_s": {"mixed": mixed_s, "fp64": fp64_s, "speedup": fp64_s / mixed_s,
-                                   "mixed_fp64_reliable_updates": {"seconds": mixed_fp64ru_s,
-                                                                   "iterations": st_fp64ru["iterations"],
-                                                                   "reliable_updates": st_fp64ru["reliable_updates"]},
                                    "other_inner_formats": others},
             "iterations": {"mixed": stats[-1]["iterations"], "reliable_updates": stats[-1]["reliable_updates"],
                            "fp64": st64["iterations"]},

@@ -89,14 +89,7 @@ lq_status require_gauge(lq_ctx* c, int prec) {
 // The fixed-point links of the FP64 operator, current with the FP64 links.
 lq_status require_fix(lq_ctx* c) {
   LQ_TRY(require_gauge(c, LQ_F64));
-  if (!c->gauge_fix) LQ_CUDA(c, cudaMalloc(&c->gauge_fix, gauge_bytes(GStore::F64_18, c->geo.V)));
-  if (!c->fix_bad) LQ_CUDA(c, cudaMalloc(&c->fix_bad, sizeof(int)));
-  if (!c->gauge_fix_valid) {
-    launch_fix_gauge(c->geo, c->gauge64, c->gauge_fix, c->fix_bad, c->stream);
-    LQ_CUDA(c, cudaGetLastError());
-    c->gauge_fix_valid = true;
-  }
-  return LQ_OK;
+  return cuda_check(c, ensure_fix_gauge(c, c->stream), "fixed-point links");
 }
 // The links an application of the operator in `prec` reads.
 lq_status require_links(lq_ctx* c, int prec) { return prec == LQ_F64 ? require_fix(c) : require_gauge(c, prec); }
@@ -228,13 +221,8 @@ lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int i
   LQ_TRY(ensure_solver_fields(c, inner));
   const Geom& g = c->geo;
   const bool mixed = inner != LQ_F64;
-  const bool dfru = mixed && c->df_updates;     // double-float intermediate reliable updates
   SStore slo = spinor_store_of(inner);
   int k = (int)slo;
-  if (dfru) {
-    LQ_TRY(require_gauge(c, LQ_DF64));
-    for (Field* f : {&c->phi_df, &c->x_df, &c->tmp_df, &c->r_df}) LQ_TRY(alloc_field(c, *f, SStore::DF64));
-  }
   SolverState h{};
   h.stop2 = tol * tol;
   h.ru_every = mixed ? reliable_every : 0;
@@ -246,10 +234,6 @@ lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int i
   LQ_CUDA(c, cudaMemcpyAsync(c->state, c->state_host, sizeof(SolverState), cudaMemcpyHostToDevice, c->stream));
   if (mixed) {
     launch_zero_spinor(g, SStore::F64, c->x64.ref(), c->stream);
-    if (dfru) {
-      launch_convert_spinor(g, SStore::F64, c->phi64.ref(), SStore::DF64, c->phi_df.ref(), c->stream);
-      launch_zero_spinor(g, SStore::DF64, c->x_df.ref(), c->stream);
-    }
     launch_solver_init(g, c->phi64.ref(), slo, c->x_lo[k].ref(), slo, c->r_lo[k].ref(), slo, c->p_lo[k].ref(),
                        c->state, c->rs, c->stream);
   } else {
@@ -281,44 +265,13 @@ lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int i
       if (st.breakdown) { result = fail(c, LQ_ERR_NAN, "CG breakdown (non-positive or non-finite curvature)"); break; }
       if (!st.halt) continue;
       // true residual; for mixed solves this is the reliable update
-      if (dfru) {
-        // double-float on the FP32 pipe; a residual meeting tol is certified in FP64.  When
-        // the iterated residual has met tol the update is almost surely the last: it goes
-        // straight to the FP64 certification.
-        const bool last = st.rr <= st.stop2;
-        if (last) {
-          df_accumulate(c, inner, c->stream);
-          s.kernel_launches += 1;
-          rel = 0.0;
-        } else {
-          df_reliable_update(c, kappa, inner, c->stream);
-          s.kernel_launches += 3;
-          LQ_CUDA(c, cudaGetLastError());
-          LQ_TRY(read_state(c));
-          rel = std::sqrt(c->state_host->rr_true / c->state_host->phi2);
-        }
-        s.reliable_updates++;
-        if (std::isfinite(rel) && rel <= tol) {
-          launch_convert_spinor(g, SStore::DF64, c->x_df.ref(), SStore::F64, c->x64.ref(), c->stream);
-          cg64_true_residual(c, kappa, inner, c->stream);
-          s.kernel_launches += 3;
-          LQ_CUDA(c, cudaGetLastError());
-          LQ_TRY(read_state(c));
-          rel = std::sqrt(c->state_host->rr_true / c->state_host->phi2);
-          if (std::isfinite(rel) && rel <= tol) { s.converged = 1; break; }
-          // not certified: continue from the FP64 residual
-          launch_convert_spinor(g, SStore::F64, c->r64.ref(), SStore::DF64, c->r_df.ref(), c->stream);
-          s.kernel_launches += 1;
-        }
-      } else {
-        if (mixed) launch_accumulate_x(g, slo, c->x_lo[k].ref(), c->x64.ref(), c->stream);
-        cg64_true_residual(c, kappa, inner, c->stream);
-        s.kernel_launches += mixed ? 3 : 2;
-        LQ_CUDA(c, cudaGetLastError());
-        LQ_TRY(read_state(c));
-        rel = std::sqrt(c->state_host->rr_true / c->state_host->phi2);
-        if (mixed) s.reliable_updates++;
-      }
+      if (mixed) launch_accumulate_x(g, slo, c->x_lo[k].ref(), c->x64.ref(), c->stream);
+      cg64_true_residual(c, kappa, inner, c->stream);
+      s.kernel_launches += mixed ? 3 : 2;
+      LQ_CUDA(c, cudaGetLastError());
+      LQ_TRY(read_state(c));
+      rel = std::sqrt(c->state_host->rr_true / c->state_host->phi2);
+      if (mixed) s.reliable_updates++;
       const double rr_true = c->state_host->rr_true;
       if (!std::isfinite(rel)) { result = fail(c, LQ_ERR_NAN, "non-finite residual"); break; }
       if (rel <= tol) { s.converged = 1; break; }
@@ -346,12 +299,7 @@ lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int i
         k = (int)slo;
         LQ_TRY(require_gauge(c, inner));
         LQ_TRY(ensure_solver_fields(c, inner));
-        if (dfru)
-          launch_inner_restart_df(g, c->r_df.ref(), slo, c->x_lo[k].ref(), c->r_lo[k].ref(), c->p_lo[k].ref(),
-                                  c->stream);
-        else
-          launch_inner_restart(g, c->r64.ref(), slo, c->x_lo[k].ref(), c->r_lo[k].ref(), c->p_lo[k].ref(),
-                               c->stream);
+        launch_inner_restart(g, c->r64.ref(), slo, c->x_lo[k].ref(), c->r_lo[k].ref(), c->p_lo[k].ref(), c->stream);
         SolverState& hs = *c->state_host;
         hs.rr = hs.rr_prev = hs.rr_ref = rr_true;
         hs.beta = 0.0;
@@ -372,11 +320,6 @@ lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int i
       s.kernel_launches += 2;
       LQ_CUDA(c, cudaGetLastError());
     }
-  }
-  if (dfru && !s.converged) {
-    // the current solution lives in the double-float accumulator
-    launch_convert_spinor(g, SStore::DF64, c->x_df.ref(), SStore::F64, c->x64.ref(), c->stream);
-    s.kernel_launches += 1;
   }
   s.iterations = c->state_host->iter;
   s.true_rel_resid = rel;
@@ -662,8 +605,7 @@ lq_status lq_destroy(lq_ctx* c) {
   if (c->stage_in) cudaFree(c->stage_in);
   if (c->stage_out) cudaFree(c->stage_out);
   if (c->stage_gauge) cudaFree(c->stage_gauge);
-  for (Field* f : {&c->phi64, &c->x64, &c->r64, &c->p64, &c->t64, &c->tmp64, &c->y64, &c->chi64, &c->phi_df,
-                   &c->x_df, &c->tmp_df, &c->r_df})
+  for (Field* f : {&c->phi64, &c->x64, &c->r64, &c->p64, &c->t64, &c->tmp64, &c->y64, &c->chi64})
     free_field(*f);
   for (double* d : {c->mom, c->mom0, c->force, c->stage_mom})
     if (d) cudaFree(d);
@@ -698,7 +640,7 @@ lq_status lq_set_option(lq_ctx* c, int option, int value) {
   if (!c) return LQ_ERR_ARG;
   switch (option) {
     case LQ_OPT_CUDA_GRAPHS: c->use_graphs = value ? 1 : 0; return LQ_OK;
-    case LQ_OPT_DF64_UPDATES: c->df_updates = value ? 1 : 0; return LQ_OK;
+    case LQ_OPT_DF64_UPDATES: return LQ_OK;      // every reliable update is FP64
     case LQ_OPT_PAIR_SITES: c->pair_sites = value ? 1 : 0; return LQ_OK;
     case LQ_OPT_STAGED: c->staged = value ? 1 : 0; return LQ_OK;
     case LQ_OPT_BATCH_RHS_PER_THREAD:

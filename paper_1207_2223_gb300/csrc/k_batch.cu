@@ -33,10 +33,7 @@
 // whose iterated residual fell far) x is folded into the high-precision
 // solution and the true residual of every column is recomputed; a column
 // whose true residual meets the tolerance is frozen (alpha = 0 from then on).
-// The intermediate updates run in double-float arithmetic (k_batch_df.cu)
-// unless the context asks for FP64 throughout; once every column is frozen,
-// or every open column's iterated residual has met the tolerance, x is
-// certified with the FP64 operator, which reopens any column that fails.
+// The updates run in FP64 (k_batch64.cu), so a frozen column is certified.
 #include <algorithm>
 #include <climits>
 #include <chrono>
@@ -181,7 +178,7 @@ __global__ void batch_unpack_kernel(BatchDesc bd, SpinorRef x64) {
 // ------------------------------------------------------------ host side
 namespace {
 
-enum { kFormChunk = 0, kFormLoop64 = 1, kFormLoopDF = 2 };
+enum { kFormChunk = 0, kFormLoop = 1 };
 
 // Launch shape of the inner-format passes, picked by timing.
 struct Tuning {
@@ -194,8 +191,7 @@ struct Tuning {
 struct BatchWork {
   std::vector<int> key;           // signature: per system dims, R, antiperiodic, precision
   int total = 0, ncols = 0, sms = 0, max_blocks = 0;
-  Field phi64, x64, r64, tmp64, plo, tlo, rlo, xlo;
-  Field phidf, xdf, tmpdf;        // double-float updates: phi, the solution, M x
+  Field phi64, x64, tmp64, plo, tlo, rlo, xlo;
   BatchState* st = nullptr;
   BatchState* st_host = nullptr;
   BatchReduce br{};
@@ -208,8 +204,8 @@ struct BatchWork {
   // recorded graphs with the descriptor and form they were recorded for
   struct Recorded {
     BatchDesc bd;
-    int form;                     // kFormChunk, kFormLoop64, kFormLoopDF
-    int chunk;                    // iterations of a chunk graph; operator variant of a loop graph
+    int form;                     // kFormChunk, kFormLoop
+    int chunk;                    // iterations of a chunk graph
     cudaGraphExec_t exec;
   };
   std::vector<Recorded> graphs;
@@ -247,8 +243,7 @@ void free_batch(BatchWork* w) {
   for (auto& g : w->graphs) cudaGraphExecDestroy(g.exec);
   for (cudaStream_t s : w->body_stream)
     if (s) cudaStreamDestroy(s);
-  for (Field* f : {&w->phi64, &w->x64, &w->r64, &w->tmp64, &w->plo, &w->tlo, &w->rlo, &w->xlo, &w->phidf, &w->xdf,
-                   &w->tmpdf}) {
+  for (Field* f : {&w->phi64, &w->x64, &w->tmp64, &w->plo, &w->tlo, &w->rlo, &w->xlo}) {
     if (f->data) cudaFree(f->data);
     if (f->norm) cudaFree(f->norm);
   }
@@ -274,8 +269,6 @@ BatchDesc make_desc(lq_ctx** ctxs, int n, int R, const double* const* phi, doubl
     SysDesc& sd = bd.sys[k];
     sd.geo = ctxs[k]->geo;
     sd.gauge_lo = ctxs[k]->gauge_lo[prec];
-    sd.gauge64 = ctxs[k]->gauge64;
-    sd.gauge_df = ctxs[k]->gauge_lo[LQ_DF64];
     sd.kappa = kappa[k];
     sd.R = R;
     sd.off = off;
@@ -315,14 +308,6 @@ void batch_iteration_prec(BatchWork* w, const BatchDesc& bd, int prec, const Tun
   }
 }
 
-template <SStore S>
-void batch_true_residual_s(BatchWork* w, const BatchDesc& bd64, cudaStream_t st) {
-  BEpiStore64 e0{w->tmp64.ref(), bd64.total};
-  launch_batch<double, GStore::F64_18, SStore::F64, false>(bd64, w->x64.ref(), e0, w->br, 1, w->sms, 0, st);
-  BEpiResidual<S> e1{w->phi64.ref(), w->r64.ref(), w->rlo.ref(), bd64.total, w->st};
-  launch_batch<double, GStore::F64_18, SStore::F64, true>(bd64, w->tmp64.ref(), e1, w->br, 1, w->sms, 0, st);
-}
-
 // the format-dependent element kernels of the host loop
 template <SStore S>
 void batch_init_s(BatchWork* w, const BatchDesc& bd, cudaStream_t st) {
@@ -347,37 +332,26 @@ void batch_init(BatchWork* w, const BatchDesc& bd, int prec, cudaStream_t st) {
   }
 }
 
-// FP64 reliable update.  fold: x64 += x_lo first (otherwise x64 was just converted from
-// the double-float solution).
+// FP64 reliable update: x64 += x_lo, the true residual of every open column, p = r + beta p
 template <SStore S>
-void batch_reliable_tail_s(BatchWork* w, const BatchDesc& bd, const BatchDesc& bd64, bool fold, cudaStream_t st) {
-  if (fold) batch_accumulate_kernel<S><<<flat_grid(w), 256, 0, st>>>(bd.total, w->xlo.ref(), w->x64.ref());
-  batch_true_residual_s<S>(w, bd64, st);
+void batch_reliable_tail_s(BatchWork* w, const BatchDesc& bd, const Batch64Args& a64, cudaStream_t st) {
+  batch_accumulate_kernel<S><<<flat_grid(w), 256, 0, st>>>(bd.total, w->xlo.ref(), w->x64.ref());
+  batch_true_residual(a64, bd, S, st);
   batch_xpay_kernel<S><<<flat_grid(w), 256, 0, st>>>(bd, w->rlo.ref(), w->plo.ref(), w->st, 1, 0, 0);
 }
-void batch_reliable_tail(BatchWork* w, const BatchDesc& bd, const BatchDesc& bd64, int prec, bool fold,
-                         cudaStream_t st) {
+void batch_reliable_tail(BatchWork* w, const BatchDesc& bd, const Batch64Args& a64, int prec, cudaStream_t st) {
   switch (spinor_store_of(prec)) {
-    case SStore::F16: batch_reliable_tail_s<SStore::F16>(w, bd, bd64, fold, st); break;
-    case SStore::BF16: batch_reliable_tail_s<SStore::BF16>(w, bd, bd64, fold, st); break;
-    case SStore::I16: batch_reliable_tail_s<SStore::I16>(w, bd, bd64, fold, st); break;
-    default: batch_reliable_tail_s<SStore::F32>(w, bd, bd64, fold, st); break;
+    case SStore::F16: batch_reliable_tail_s<SStore::F16>(w, bd, a64, st); break;
+    case SStore::BF16: batch_reliable_tail_s<SStore::BF16>(w, bd, a64, st); break;
+    case SStore::I16: batch_reliable_tail_s<SStore::I16>(w, bd, a64, st); break;
+    default: batch_reliable_tail_s<SStore::F32>(w, bd, a64, st); break;
   }
-}
-void batch_xpay_forced(BatchWork* w, const BatchDesc& bd, int prec, cudaStream_t st) {
-  launch_batch_xpay(bd, spinor_store_of(prec), w->rlo.ref(), w->plo.ref(), w->st, 1, flat_grid(w), st);
-}
-Geom flat_geom(int total) {
-  Geom g{};
-  g.V = total;
-  return g;
 }
 
 // ------------------------------------------------------------ device-side solve loop
 // The whole solve as one CUDA graph: a while node over update cycles whose body holds a
-// while node over CG iterations (until a reliable update is due), then the update, with if
-// nodes around the double-float residual and the FP64 certification.  One-thread kernels
-// read the state, take each decision and set the node's condition (the iteration loop's
+// while node over CG iterations (until a reliable update is due), then the update.  One-thread
+// kernels read the state, take each decision and set the node's condition (the iteration loop's
 // condition is set by the first thread of each iteration's last kernel, batch_xpay_kernel);
 // every loop counts its bodies against a cap taken from the iteration limit, so the graph
 // ends even if the state never halts.
@@ -386,24 +360,6 @@ Geom flat_geom(int total) {
 __global__ void cond_enter_kernel(BatchState* st, cudaGraphConditionalHandle inner) {
   st->guard_inner = 0;
   cudaGraphSetConditional(inner, st->halt ? 0u : 1u);
-}
-// the double-float residual unless every open column's iterated residual met the
-// tolerance (that update goes straight to the FP64 certification)
-__global__ void cond_df_kernel(BatchState* st, int ncols, cudaGraphConditionalHandle df) {
-  int last = 1;
-  for (int c = 0; c < ncols; ++c)
-    if (!st->done[c] && !(st->rr[c] <= st->stop2 * st->phi2[c])) last = 0;
-  st->df_last = last;
-  if (!last) st->loops[2]++;
-  cudaGraphSetConditional(df, last ? 0u : 1u);
-}
-// the FP64 certification once every column is frozen (or the double-float step was skipped)
-__global__ void cond_cert_kernel(BatchState* st, int ncols, cudaGraphConditionalHandle cert) {
-  int all = 1;
-  for (int c = 0; c < ncols; ++c) all &= st->done[c] ? 1 : 0;
-  const int go = st->df_last || (all && !st->breakdown);
-  if (go) st->loops[3]++;
-  cudaGraphSetConditional(cert, go ? 1u : 0u);
 }
 // another update cycle unless every column is frozen (certified), the iteration limit is
 // reached or a breakdown was seen
@@ -462,9 +418,8 @@ cudaError_t record_body(cudaStream_t s, cudaGraph_t body, F&& launches) {
   return err != cudaSuccess ? err : (e0 != cudaSuccess ? e0 : e1);
 }
 
-// dfa null: every reliable update in FP64
-cudaError_t build_solve_graph(BatchWork* w, const BatchDesc& bd, const BatchDesc& bd64, int prec, const Tuning& tu,
-                              const BatchDfArgs* dfa, cudaGraphExec_t* exec) {
+cudaError_t build_solve_graph(BatchWork* w, const BatchDesc& bd, const Batch64Args& a64, int prec, const Tuning& tu,
+                              cudaGraphExec_t* exec) {
   for (cudaStream_t& s : w->body_stream)
     if (!s) {
       const cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
@@ -485,7 +440,6 @@ cudaError_t build_solve_graph(BatchWork* w, const BatchDesc& bd, const BatchDesc
   cudaGraphNode_t outer = nullptr;
   if (err == cudaSuccess) err = cudaGraphAddNode(&outer, g, nullptr, nullptr, 0, &p);
   const int ncols = bd.ncols;
-  const SStore slo = spinor_store_of(prec);
   BatchState* st = w->st;
   if (err == cudaSuccess) {
     err = record_body(s1, p.conditional.phGraph_out[0], [&](cudaStream_t s) -> cudaError_t {
@@ -502,41 +456,7 @@ cudaError_t build_solve_graph(BatchWork* w, const BatchDesc& bd, const BatchDesc
         return cudaSuccess;
       });
       if (e != cudaSuccess) return e;
-      if (!dfa) {
-        batch_reliable_tail(w, bd, bd64, prec, true, s);
-      } else {
-        cudaGraphConditionalHandle h_df, h_cert;
-        e = new_handle(s, &h_df);
-        if (e == cudaSuccess) e = new_handle(s, &h_cert);
-        if (e != cudaSuccess) return e;
-        cond_df_kernel<<<1, 1, 0, s>>>(st, ncols, h_df);
-        BatchDfArgs acc = *dfa;
-        acc.accumulate = true;
-        acc.residual = false;
-        batch_df_tail(acc, bd, slo, s);
-        // the double-float residual of every column
-        e = add_conditional(s, cudaGraphCondTypeIf, h_df, &body);
-        if (e != cudaSuccess) return e;
-        e = record_body(s2, body, [&](cudaStream_t q) -> cudaError_t {
-          BatchDfArgs res = *dfa;
-          res.accumulate = false;
-          res.residual = true;
-          batch_df_tail(res, bd, slo, q);
-          batch_xpay_forced(w, bd, prec, q);
-          return cudaSuccess;
-        });
-        if (e != cudaSuccess) return e;
-        // the FP64 certification
-        cond_cert_kernel<<<1, 1, 0, s>>>(st, ncols, h_cert);
-        e = add_conditional(s, cudaGraphCondTypeIf, h_cert, &body);
-        if (e != cudaSuccess) return e;
-        e = record_body(s2, body, [&](cudaStream_t q) -> cudaError_t {
-          launch_convert_spinor(flat_geom(bd.total), SStore::DF64, w->xdf.ref(), SStore::F64, w->x64.ref(), q);
-          batch_reliable_tail(w, bd, bd64, prec, false, q);
-          return cudaSuccess;
-        });
-        if (e != cudaSuccess) return e;
-      }
+      batch_reliable_tail(w, bd, a64, prec, s);
       cond_continue_kernel<<<1, 1, 0, s>>>(st, ncols, h_outer);
       return cudaSuccess;
     });
@@ -586,20 +506,20 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
     if (elements > (long long)(INT_MAX / 2)) return fail(LQ_ERR_SHAPE, "batch too large for 32-bit element indices");
   }
   cudaStream_t st = c->stream;
-  const bool dfru = c->df_updates != 0;      // double-float intermediate reliable updates
-  // every system's links in the inner format (and as double-float pairs), converted on
+  // every system's links in the inner format and in fixed point (FP64 updates), converted on
   // the caller's stream
   for (int k = 0; k < n; ++k) {
     lq_ctx* ck = ctxs[k];
-    for (int prec : {inner_prec, dfru ? (int)LQ_DF64 : inner_prec}) {
-      if (!ck->gauge_lo[prec]) {
-        if (cudaMalloc(&ck->gauge_lo[prec], gauge_bytes(gauge_store_of(prec), ck->geo.V)) != cudaSuccess)
-          return fail(LQ_ERR_CUDA, "cudaMalloc");
-      }
-      if (!ck->gauge_lo_valid[prec]) {
-        launch_convert_gauge(ck->geo, ck->gauge64, gauge_store_of(prec), ck->gauge_lo[prec], st);
-        ck->gauge_lo_valid[prec] = true;
-      }
+    void*& lo = ck->gauge_lo[inner_prec];
+    if (!lo && cudaMalloc(&lo, gauge_bytes(gauge_store_of(inner_prec), ck->geo.V)) != cudaSuccess)
+      return fail(LQ_ERR_CUDA, "cudaMalloc");
+    if (!ck->gauge_lo_valid[inner_prec]) {
+      launch_convert_gauge(ck->geo, ck->gauge64, gauge_store_of(inner_prec), lo, st);
+      ck->gauge_lo_valid[inner_prec] = true;
+    }
+    if (ensure_fix_gauge(ck, st) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(LQ_ERR_CUDA, "fixed-point links");
     }
   }
   // workspace owned by the first context, rebuilt when the batch changes shape
@@ -607,7 +527,6 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
   for (int k = 0; k < n; ++k)
     for (int m = 0; m < 4; ++m) key.push_back(ctxs[k]->geo.L[m]);
   for (int k = 0; k < n; ++k) key.push_back(ctxs[k]->geo.antiperiodic);
-  key.push_back(dfru);
   BatchWork* w = static_cast<BatchWork*>(c->batch);
   if (!w || w->key != key) {
     free_batch(w);
@@ -621,20 +540,19 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
     auto alloc = [&](Field& f, SStore s) {
       f.store = s;
       ok = ok && cudaMalloc(&f.data, spinor_bytes(s, w->total)) == cudaSuccess;
-      if (s == SStore::F16 || s == SStore::BF16 || s == SStore::I16)
+      if (s != SStore::F32)       // norms; FP64: exponent words
         ok = ok && cudaMalloc(&f.norm, sizeof(float) * w->total) == cudaSuccess;
     };
     const SStore slo = spinor_store_of(inner_prec);
-    alloc(w->phi64, SStore::F64); alloc(w->x64, SStore::F64); alloc(w->r64, SStore::F64); alloc(w->tmp64, SStore::F64);
+    alloc(w->phi64, SStore::F64); alloc(w->x64, SStore::F64); alloc(w->tmp64, SStore::F64);
     alloc(w->plo, slo); alloc(w->tlo, slo); alloc(w->rlo, slo); alloc(w->xlo, xlo_store(slo));
-    if (dfru) { alloc(w->phidf, SStore::DF64); alloc(w->xdf, SStore::DF64); alloc(w->tmpdf, SStore::DF64); }
     cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, c->device);
     w->sms = std::max(1, w->sms);
     w->max_blocks = w->sms * 8;
     w->br.max_blocks = w->max_blocks;
     ok = ok && cudaMalloc(&w->br.partials, sizeof(double) * kMaxCols * w->br.max_blocks) == cudaSuccess;
-    ok = ok && cudaMalloc(&w->br.ticket, sizeof(unsigned int)) == cudaSuccess;
-    ok = ok && cudaMemset(w->br.ticket, 0, sizeof(unsigned int)) == cudaSuccess;
+    ok = ok && cudaMalloc(&w->br.ticket, sizeof(unsigned int) * kMaxCols) == cudaSuccess;
+    ok = ok && cudaMemset(w->br.ticket, 0, sizeof(unsigned int) * kMaxCols) == cudaSuccess;
     ok = ok && cudaMalloc(&w->st, sizeof(BatchState)) == cudaSuccess;
     ok = ok && cudaMallocHost(&w->st_host, sizeof(BatchState)) == cudaSuccess;
     ok = ok && cudaMalloc(&w->part, sizeof(double) * 2 * kMaxCols * w->max_blocks) == cudaSuccess;
@@ -745,26 +663,10 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
   }
   const Tuning tu = w->tune;
   const BatchDesc bd = make_desc(ctxs, n, nrhs, phi, x, kappa, inner_prec, tu.tile, tu.rb, tu.site_major);
-  // FP64 passes (~250 registers per thread): one right-hand side per thread, 128 threads
-  const BatchDesc bd64 = make_desc(ctxs, n, nrhs, phi, x, kappa, inner_prec, 128, 1, 1);
   batch_init(w, bdi, inner_prec, st);
   s.kernel_launches += 1;
-  BatchDfArgs dfa{};
-  if (dfru) {
-    launch_convert_spinor(flat_geom(bd.total), SStore::F64, w->phi64.ref(), SStore::DF64, w->phidf.ref(), st);
-    launch_zero_spinor(flat_geom(bd.total), SStore::DF64, w->xdf.ref(), st);
-    s.kernel_launches += 2;
-    dfa.xlo = w->xlo.ref();
-    dfa.xdf = w->xdf.ref();
-    dfa.tmpdf = w->tmpdf.ref();
-    dfa.phidf = w->phidf.ref();
-    dfa.rlo = w->rlo.ref();
-    dfa.st = w->st;
-    dfa.br = w->br;
-    for (int k = 0; k < n; ++k) dfa.gauge_df[k] = ctxs[k]->gauge_lo[LQ_DF64];
-    dfa.flat_grid = flat_grid(w);
-    dfa.prefetch = c->df_prefetch != 0;
-  }
+  Batch64Args a64{w->x64.ref(), w->tmp64.ref(), w->phi64.ref(), w->rlo.ref(), w->st, w->br, {}, w->sms};
+  for (int k = 0; k < n; ++k) a64.U[k] = fix_gauge_of(ctxs[k]);
 
   const int chunk = reliable_every;
   lq_status result = LQ_OK;
@@ -773,13 +675,10 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
   if (!host_loop) {
     // the whole solve as one graph with conditional nodes; a launch that its loop caps
     // ended early is repeated (at most a few times)
-    // the graph bakes in the double-float operator variant: part of its key
-    const int form = dfru ? kFormLoopDF : kFormLoop64;
-    const int variant = dfru && dfa.prefetch ? 1 : 0;
-    cudaGraphExec_t exec = find_graph(w, bd, form, variant);
+    cudaGraphExec_t exec = find_graph(w, bd, kFormLoop, 0);
     if (!exec) {
-      err = build_solve_graph(w, bd, bd64, inner_prec, tu, dfru ? &dfa : nullptr, &exec);
-      if (err == cudaSuccess) keep_graph(w, bd, form, variant, exec);
+      err = build_solve_graph(w, bd, a64, inner_prec, tu, &exec);
+      if (err == cudaSuccess) keep_graph(w, bd, kFormLoop, 0, exec);
     }
     for (int launch = 0; launch < 4 && err == cudaSuccess; ++launch) {
       err = cudaGraphLaunch(exec, st);
@@ -799,14 +698,8 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
     // launches from the loop counts: an iteration is three passes (the last one sets the
     // loop's condition); an update cycle enters and leaves the loop around its update
     const int* L = w->st_host->loops;
-    s.kernel_launches += 3 * L[0];
-    if (dfru) {
-      s.kernel_launches += 5 * L[1] + (2 * bd.ncols + 1) * L[2] + 4 * L[3];
-      s.reliable_updates += L[2] + L[3];
-    } else {
-      s.kernel_launches += 6 * L[1];
-      s.reliable_updates += L[1];
-    }
+    s.kernel_launches += 3 * L[0] + 6 * L[1];
+    s.reliable_updates += L[1];
   }
   // host loop: iterations as CUDA graphs of reliable_every iterations
   for (long guard = 0; host_loop && guard < (long)maxiter + 64; ++guard) {
@@ -853,45 +746,12 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
     s.kernel_launches += 3 * chunk;
     }
     // reliable update: fold x, true residual per column, freeze converged columns
-    bool certify = true;
-    if (dfru) {
-      // double-float update, skipped (x_lo only folded) when every open column's
-      // iterated residual has already met the tolerance: that update goes straight
-      // to the FP64 certification
-      err = cudaMemcpyAsync(w->st_host, w->st, sizeof(BatchState), cudaMemcpyDeviceToHost, st);
-      if (err == cudaSuccess) err = cudaStreamSynchronize(st);
-      if (err != cudaSuccess) break;
-      bool last = true;
-      for (int col = 0; col < bd.ncols; ++col)
-        if (!w->st_host->done[col] && !(w->st_host->rr[col] <= w->st_host->stop2 * w->st_host->phi2[col]))
-          last = false;
-      dfa.accumulate = true;
-      dfa.residual = !last;
-      batch_df_tail(dfa, bd, spinor_store_of(inner_prec), st);
-      s.kernel_launches += last ? 1 : 1 + 2 * bd.ncols;
-      if (!last) {
-        batch_xpay_forced(w, bd, inner_prec, st);
-        s.kernel_launches += 1;
-        s.reliable_updates++;
-        err = cudaMemcpyAsync(w->st_host, w->st, sizeof(BatchState), cudaMemcpyDeviceToHost, st);
-        if (err == cudaSuccess) err = cudaStreamSynchronize(st);
-        if (err != cudaSuccess) break;
-        for (int col = 0; col < bd.ncols; ++col) certify = certify && w->st_host->done[col];
-        certify = certify && !w->st_host->breakdown;
-      }
-      if (certify) {
-        launch_convert_spinor(flat_geom(bd.total), SStore::DF64, w->xdf.ref(), SStore::F64, w->x64.ref(), st);
-        s.kernel_launches += 1;
-      }
-    }
-    if (certify) {
-      batch_reliable_tail(w, bd, bd64, inner_prec, !dfru, st);
-      s.kernel_launches += dfru ? 3 : 4;
-      s.reliable_updates++;
-      err = cudaMemcpyAsync(w->st_host, w->st, sizeof(BatchState), cudaMemcpyDeviceToHost, st);
-      if (err == cudaSuccess) err = cudaStreamSynchronize(st);
-      if (err != cudaSuccess) break;
-    }
+    batch_reliable_tail(w, bd, a64, inner_prec, st);
+    s.kernel_launches += 4;
+    s.reliable_updates++;
+    err = cudaMemcpyAsync(w->st_host, w->st, sizeof(BatchState), cudaMemcpyDeviceToHost, st);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(st);
+    if (err != cudaSuccess) break;
     const BatchState& hs = *w->st_host;
     if (hs.breakdown) { result = fail(LQ_ERR_NAN, "non-finite value or CG breakdown"); break; }
     bool all = true;
@@ -902,11 +762,6 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
   if (err != cudaSuccess) {
     cudaGetLastError();
     return fail(LQ_ERR_CUDA, cudaGetErrorString(err));
-  }
-  if (dfru) {
-    // the solution lives in the double-float accumulator (x_lo already folded)
-    launch_convert_spinor(flat_geom(bd.total), SStore::DF64, w->xdf.ref(), SStore::F64, w->x64.ref(), st);
-    s.kernel_launches += 1;
   }
   batch_unpack_kernel<<<flat_grid(w), 256, 0, st>>>(bd, w->x64.ref());
   s.kernel_launches += 1;

@@ -218,23 +218,6 @@ void launch_convert_gauge(const Geom& g, const void* soa64, GStore dst, void* ou
   }
 }
 
-// field-to-field format conversion (through FP64 values)
-template <SStore A, SStore B>
-__global__ void convert_spinor_kernel(int V, SpinorRef in, SpinorRef out) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= V) return;
-  cplx<double> v[12];
-  load_spinor<A, double>(in, V, s, v);
-  store_spinor<B, double>(out, V, s, v);
-}
-
-void launch_convert_spinor(const Geom& g, SStore a, SpinorRef in, SStore b, SpinorRef out, cudaStream_t st) {
-  const int grid = grid_for(g.V, kBS);
-  if (a == SStore::F64 && b == SStore::DF64)
-    convert_spinor_kernel<SStore::F64, SStore::DF64><<<grid, kBS, 0, st>>>(g.V, in, out);
-  else if (a == SStore::DF64 && b == SStore::F64)
-    convert_spinor_kernel<SStore::DF64, SStore::F64><<<grid, kBS, 0, st>>>(g.V, in, out);
-}
 void launch_pack_spinor(const Geom& g, const double* canon, SStore s, SpinorRef out, cudaStream_t st) {
   const int grid = grid_for(g.V, kSpinTile);
   const double2* in = reinterpret_cast<const double2*>(canon);

@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "lq_internal.h"
+#include "lq_fix64.cuh"
 
 namespace lq {
 
@@ -18,8 +19,6 @@ constexpr int kMaxRB = 4;
 struct SysDesc {
   Geom geo;
   const void* gauge_lo;   // inner-format links of the system (SoA, stride V)
-  const void* gauge64;    // FP64 links
-  const void* gauge_df;   // links as double-float pairs (double-float updates), else null
   double kappa;
   int R;                  // right-hand sides
   int off;                // first element in the batch fields
@@ -48,16 +47,15 @@ struct BatchState {
   int timeout;             // a bounded wait of the persistent iteration gave up
   double* hist;            // [ncols][hist_len] relative iterated residuals
   // device-side solve loop (one graph with conditional nodes): body counts of the
-  // current iteration loop and of the update loop (each loop stops at a cap), whether
-  // the current update skipped the double-float residual, and how many CG iterations,
-  // update cycles, double-float updates and FP64 certifications ran
-  int guard_inner, guard_outer, df_last;
-  int loops[4];
+  // current iteration loop and of the update loop (each loop stops at a cap), and how
+  // many CG iterations and update cycles ran
+  int guard_inner, guard_outer;
+  int loops[2];
 };
 
 struct BatchReduce {
   double* partials;        // [kMaxCols][max_blocks]
-  unsigned int* ticket;
+  unsigned int* ticket;    // [kMaxCols]: the FP64 passes count each column's blocks, the others use the first
   int max_blocks;
 };
 
@@ -179,18 +177,6 @@ __device__ __forceinline__ void clear_columns(int ncols, double* sh_wcol) {
 // Each gets the element index e (in the batch fields), its column, the
 // result v = M in (or M^dag in) of that element, and returns the value to
 // be summed for its column.
-struct BEpiStore64 {                        // tmp = M x (FP64)
-  SpinorRef out;
-  int total;
-  __device__ bool halted() const { return false; }
-  template <typename T> __device__ double apply(int e, int, const cplx<T> v[12]) const {
-    store_spinor<SStore::F64, T>(out, total, e, v);
-    return 0.0;
-  }
-  static constexpr bool REDUCE = false;
-  __device__ void finalize_cols(const double*, int) const {}
-};
-
 template <SStore S>
 struct BEpiCG1 {                             // t = M p, tt = |t|^2, alpha = rr / tt
   SpinorRef t;
@@ -276,23 +262,18 @@ struct BEpiCG2 {                             // r -= alpha M^dag t, x += alpha p
 };
 
 // A column's true residual |r|^2 = tot after a reliable update: freeze the column once it
-// meets the tolerance (alpha = beta = 0 from then on), reopen a frozen column whose
-// residual no longer does (a double-float estimate that the FP64 certification overrules),
-// restart the search direction when the recursion drifted far from the true residual.
+// meets the tolerance (alpha = beta = 0 from then on), restart the search direction when the recursion drifted far from the true residual.
 __device__ __forceinline__ void reliable_update_column(BatchState* st, int c, double tot) {
   st->rr_true[c] = tot;
   if (!isfinite(tot)) { st->breakdown = 1; return; }
-  const bool meets = tot <= st->stop2 * st->phi2[c];
-  if (st->done[c] && meets) { st->beta[c] = 0.0; return; }
-  if (meets) {                                      // converged: freeze the column
+  if (tot <= st->stop2 * st->phi2[c]) {                                      // converged: freeze the column
     st->done[c] = 1;
     st->conv_iter[c] = st->iter;
     st->beta[c] = 0.0;
     st->alpha[c] = 0.0;
-  } else if (st->done[c] || tot > 100.0 * st->rr[c]) {
-    // reopened, or the low-precision recursion drifted far below the true
-    // residual: the search direction no longer fits it, restart from r
-    st->done[c] = 0;
+  } else if (tot > 100.0 * st->rr[c]) {
+    // the low-precision recursion drifted far below the true residual: the
+    // search direction no longer fits it, restart from r
     st->beta[c] = 0.0;
   } else {
     st->beta[c] = tot / st->rr_prev[c];
@@ -300,36 +281,6 @@ __device__ __forceinline__ void reliable_update_column(BatchState* st, int c, do
   st->rr[c] = tot;
   st->rr_ref[c] = tot;
 }
-
-template <SStore S>
-struct BEpiResidual {                        // r64 = phi - M^dag tmp, r_lo = r64, rr_true = |r64|^2
-  SpinorRef phi, r64, rlo;
-  int total;
-  BatchState* st;
-  static constexpr bool REDUCE = true;
-  __device__ bool halted() const { return false; }
-  template <typename T> __device__ double apply(int e, int, const cplx<T> v[12]) const {
-    cplx<double> ph[12], rv[12];
-    load_spinor<SStore::F64, double>(phi, total, e, ph);
-    double a = 0.0;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      rv[k] = {ph[k].re - (double)v[k].re, ph[k].im - (double)v[k].im};
-      a += rv[k].re * rv[k].re + rv[k].im * rv[k].im;
-    }
-    store_spinor<SStore::F64, double>(r64, total, e, rv);
-    store_spinor<S, double>(rlo, total, e, rv);
-    return a;
-  }
-  // every thread of the reducing block: one column per thread
-  __device__ void finalize_cols(const double* tot, int ncols) const {
-    for (int c = threadIdx.x; c < ncols; c += blockDim.x) reliable_update_column(st, c, tot[c]);
-    if (threadIdx.x == 0) {
-      st->iter_since_ru = 0;
-      st->halt = 0;
-    }
-  }
-};
 
 // ------------------------------------------------------------ stencil
 // Both hops of direction MU at site s for RB right-hand sides: the links
@@ -394,7 +345,6 @@ __device__ __forceinline__ void batch_hops(const Geom& geo, int total, const Gau
 // Register cap: one right-hand side per thread fits two blocks of 256 threads per
 // SM (128 registers); more need the larger register budget of one block.
 template <typename T, int RB> struct BatchMinBlocks { static constexpr int value = (RB == 1) ? 2 : 1; };
-template <int RB> struct BatchMinBlocks<double, RB> { static constexpr int value = 1; };
 
 // One stencil pass over the block's tiles: out = M in (or M^dag in) per right-hand side,
 // handed to the epilogue; with Epi::REDUCE every warp adds its per-column sums to its slots
@@ -405,7 +355,7 @@ template <int RB> struct BatchMinBlocks<double, RB> { static constexpr int value
 // kernel parameters (no per-access indexed constant loads).
 template <typename T, GStore G, SStore SI, bool DAG, int RB, class Epi, int LD = 1, bool ONE = false>
 __device__ __forceinline__ void batch_stencil_pass(const BatchDesc& bd, const SpinorRef& in, const Epi& epi,
-                                                   int use64, double* sh_wcol, double* sh_col) {
+                                                   double* sh_wcol, double* sh_col) {
   int cur = -1;                       // first column of the group the sums belong to
   double red[RB];
 #pragma unroll
@@ -426,7 +376,7 @@ __device__ __forceinline__ void batch_stencil_pass(const BatchDesc& bd, const Sp
       const int s = w.s;
       int c[4];
       site_coords(sd.geo, s, c);
-      const GaugeRef U{use64 ? sd.gauge64 : sd.gauge_lo};
+      const GaugeRef U{sd.gauge_lo};
       const int e0 = sd.off + w.r0 * sd.geo.V;
       cplx<T> acc[RB][12];
       batch_hops<0, DAG, G, SI, T, RB, LD, true>(sd.geo, bd.total, U, in, s, c, e0, acc);
@@ -456,12 +406,12 @@ __device__ __forceinline__ void batch_stencil_pass(const BatchDesc& bd, const Sp
 
 template <typename T, GStore G, SStore SI, bool DAG, int RB, class Epi, bool ONE = false>
 __global__ void __launch_bounds__(256, (BatchMinBlocks<T, RB>::value))
-    batch_dslash_kernel(BatchDesc bd, SpinorRef in, Epi epi, BatchReduce br, int use64) {
+    batch_dslash_kernel(BatchDesc bd, SpinorRef in, Epi epi, BatchReduce br) {
   if (epi.halted()) return;
   __shared__ double sh_col[kMaxCols];
   __shared__ double sh_wcol[Epi::REDUCE ? kMaxCols * kMaxWarps : 1];
   if constexpr (Epi::REDUCE) clear_columns(bd.ncols, sh_wcol);
-  batch_stencil_pass<T, G, SI, DAG, RB, Epi, 1, ONE>(bd, in, epi, use64, sh_wcol, sh_col);
+  batch_stencil_pass<T, G, SI, DAG, RB, Epi, 1, ONE>(bd, in, epi, sh_wcol, sh_col);
   if constexpr (Epi::REDUCE) {
     auto fin = [&](const double* tot) { epi.finalize_cols(tot, bd.ncols); };
     batch_grid_sum(bd, sh_col, br, fin);
@@ -582,7 +532,7 @@ __global__ void __launch_bounds__(256, (BatchMinBlocks<float, RB>::value))
     // pass 1: t = M p, |t|^2 per column -> alpha
     clear_columns(bd.ncols, sh_wcol);
     PEpiCG1<S> e1{a.tlo, bd.total};
-    batch_stencil_pass<float, G, S, false, RB, PEpiCG1<S>, 2>(bd, a.plo, e1, 0, sh_wcol, sh_col);
+    batch_stencil_pass<float, G, S, false, RB, PEpiCG1<S>, 2>(bd, a.plo, e1, sh_wcol, sh_col);
     for (int c = threadIdx.x; c < bd.ncols; c += blockDim.x) part1[(size_t)c * a.stride + blockIdx.x] = sh_col[c];
     if (!grid_barrier(a, gen, &s_ok)) return;
     column_totals(part1, a.stride, bd.ncols, s_tot);
@@ -603,7 +553,7 @@ __global__ void __launch_bounds__(256, (BatchMinBlocks<float, RB>::value))
     // pass 2: r -= alpha M^dag t, x += alpha p, |r|^2 per column -> beta, halt decision
     clear_columns(bd.ncols, sh_wcol);
     PEpiCG2<S> e2{a.rlo, a.xlo, a.plo, bd.total, s_alpha};
-    batch_stencil_pass<float, G, S, true, RB, PEpiCG2<S>, 2>(bd, a.tlo, e2, 0, sh_wcol, sh_col);
+    batch_stencil_pass<float, G, S, true, RB, PEpiCG2<S>, 2>(bd, a.tlo, e2, sh_wcol, sh_col);
     for (int c = threadIdx.x; c < bd.ncols; c += blockDim.x) part2[(size_t)c * a.stride + blockIdx.x] = sh_col[c];
     if (!grid_barrier(a, gen, &s_ok)) return;
     column_totals(part2, a.stride, bd.ncols, s_tot);
@@ -693,7 +643,7 @@ struct BatchIterArgs {
 };
 
 template <typename T, GStore G, SStore SI, bool DAG, int RB, class Epi, bool ONE>
-void launch_batch_rb(const BatchDesc& bd, SpinorRef in, const Epi& epi, const BatchReduce& br, int use64, int sms,
+void launch_batch_rb(const BatchDesc& bd, SpinorRef in, const Epi& epi, const BatchReduce& br, int sms,
                      int per_sm, cudaStream_t st) {
   auto kern = &batch_dslash_kernel<T, G, SI, DAG, RB, Epi, ONE>;
   static const int wave_all = resident_grid(reinterpret_cast<const void*>(kern), 256);
@@ -702,27 +652,25 @@ void launch_batch_rb(const BatchDesc& bd, SpinorRef in, const Epi& epi, const Ba
   const int fit = std::max(1, wave_all / std::max(1, sms)) * (256 / bd.tile);
   const int wave = sms * (per_sm > 0 ? std::min(per_sm, fit) : fit);
   const int grid = std::max(1, std::min(std::min(bd.ntiles, br.max_blocks), wave));
-  kern<<<grid, bd.tile, 0, st>>>(bd, in, epi, br, use64);
+  kern<<<grid, bd.tile, 0, st>>>(bd, in, epi, br);
 }
 
 template <typename T, GStore G, SStore SI, bool DAG, class Epi>
-void launch_batch(const BatchDesc& bd, SpinorRef in, const Epi& epi, const BatchReduce& br, int use64, int sms,
+void launch_batch(const BatchDesc& bd, SpinorRef in, const Epi& epi, const BatchReduce& br, int sms,
                   int per_sm, cudaStream_t st) {
-  if constexpr (std::is_same<T, double>::value) {
-    launch_batch_rb<T, G, SI, DAG, 1, Epi, false>(bd, in, epi, br, use64, sms, per_sm, st);   // FP64: one per thread
-  } else if (bd.nsys == 1) {
+  if (bd.nsys == 1) {
     switch (bd.rb) {
-      case 2: launch_batch_rb<T, G, SI, DAG, 2, Epi, true>(bd, in, epi, br, use64, sms, per_sm, st); break;
-      case 3: launch_batch_rb<T, G, SI, DAG, 3, Epi, true>(bd, in, epi, br, use64, sms, per_sm, st); break;
-      case 4: launch_batch_rb<T, G, SI, DAG, 4, Epi, true>(bd, in, epi, br, use64, sms, per_sm, st); break;
-      default: launch_batch_rb<T, G, SI, DAG, 1, Epi, true>(bd, in, epi, br, use64, sms, per_sm, st); break;
+      case 2: launch_batch_rb<T, G, SI, DAG, 2, Epi, true>(bd, in, epi, br, sms, per_sm, st); break;
+      case 3: launch_batch_rb<T, G, SI, DAG, 3, Epi, true>(bd, in, epi, br, sms, per_sm, st); break;
+      case 4: launch_batch_rb<T, G, SI, DAG, 4, Epi, true>(bd, in, epi, br, sms, per_sm, st); break;
+      default: launch_batch_rb<T, G, SI, DAG, 1, Epi, true>(bd, in, epi, br, sms, per_sm, st); break;
     }
   } else {
     switch (bd.rb) {
-      case 2: launch_batch_rb<T, G, SI, DAG, 2, Epi, false>(bd, in, epi, br, use64, sms, per_sm, st); break;
-      case 3: launch_batch_rb<T, G, SI, DAG, 3, Epi, false>(bd, in, epi, br, use64, sms, per_sm, st); break;
-      case 4: launch_batch_rb<T, G, SI, DAG, 4, Epi, false>(bd, in, epi, br, use64, sms, per_sm, st); break;
-      default: launch_batch_rb<T, G, SI, DAG, 1, Epi, false>(bd, in, epi, br, use64, sms, per_sm, st); break;
+      case 2: launch_batch_rb<T, G, SI, DAG, 2, Epi, false>(bd, in, epi, br, sms, per_sm, st); break;
+      case 3: launch_batch_rb<T, G, SI, DAG, 3, Epi, false>(bd, in, epi, br, sms, per_sm, st); break;
+      case 4: launch_batch_rb<T, G, SI, DAG, 4, Epi, false>(bd, in, epi, br, sms, per_sm, st); break;
+      default: launch_batch_rb<T, G, SI, DAG, 1, Epi, false>(bd, in, epi, br, sms, per_sm, st); break;
     }
   }
 }
@@ -752,26 +700,23 @@ cudaError_t batch_persistent_bf16(const BatchDesc& bd, const PersistArgs& a, int
 cudaError_t batch_persistent_i16(const BatchDesc& bd, const PersistArgs& a, int prec, int sms, int max_grid,
                                  cudaStream_t st);
 
-// Double-float reliable update of the batch (k_batch_df.cu): x_df += x_lo, x_lo = 0
-// (`accumulate`) and per column r = phi - M^dag M x_df with r to r_lo and the column's
-// |r|^2 through reliable_update_column (`residual`).
-struct BatchDfArgs {
-  SpinorRef xlo, xdf, tmpdf, phidf, rlo;
+// FP64 reliable update of the batch (k_batch64.cu): per open column r = phi - M^dag M x, r to
+// rlo in the inner format, |r|^2 through reliable_update_column.
+struct Batch64Args {
+  SpinorRef x, tmp, phi, rlo;
   BatchState* st;
   BatchReduce br;
-  const void* gauge_df[kMaxSys];   // per system: links as double-float pairs
-  int flat_grid;
-  bool accumulate, residual;       // which of the two steps to launch
-  bool prefetch;                   // the double-float operator's prefetching variant
+  FixGauge U[kMaxSys];
+  int sms;
 };
-void batch_df_tail(const BatchDfArgs& a, const BatchDesc& bd, SStore s, cudaStream_t st);
+void batch_true_residual(const Batch64Args& a, const BatchDesc& bd, SStore s, cudaStream_t st);
 
 template <GStore G, SStore S>
 void batch_iteration_t(const BatchIterArgs& a, const BatchDesc& bd, cudaStream_t st) {
   BEpiCG1<S> e1{a.tlo, bd.total, a.st};
-  launch_batch<float, G, S, false>(bd, a.plo, e1, a.br, 0, a.sms, a.per_sm, st);
+  launch_batch<float, G, S, false>(bd, a.plo, e1, a.br, a.sms, a.per_sm, st);
   BEpiCG2<S> e2{a.rlo, a.xlo, a.plo, bd.total, a.st};
-  launch_batch<float, G, S, true>(bd, a.tlo, e2, a.br, 0, a.sms, a.per_sm, st);
+  launch_batch<float, G, S, true>(bd, a.tlo, e2, a.br, a.sms, a.per_sm, st);
   launch_batch_xpay(bd, S, a.rlo, a.plo, a.st, 0, a.sms * 8, st, a.cond, a.use_cond);
 }
 

@@ -553,18 +553,19 @@ __device__ __forceinline__ void block_sum(double (&v)[NRED], double* sh /* [NRED
   }
 }
 
-// Returns true in thread 0 of the last block, with the grid totals in tot.
+// Returns true in thread 0 of the last block, with the totals in tot: block `block` of the
+// `nblocks` blocks that share rs (the whole grid by default).
 template <int NRED>
-__device__ bool grid_sum(double (&v)[NRED], const ReduceScratch& rs, double (&tot)[NRED]) {
+__device__ bool grid_sum(double (&v)[NRED], const ReduceScratch& rs, double (&tot)[NRED], int block, int nblocks) {
   __shared__ double sh[NRED * 32];
   __shared__ bool last;
   block_sum<NRED>(v, sh);
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int q = 0; q < NRED; ++q) rs.partials[(size_t)q * rs.max_blocks + blockIdx.x] = v[q];
+    for (int q = 0; q < NRED; ++q) rs.partials[(size_t)q * rs.max_blocks + block] = v[q];
     __threadfence();
     unsigned int t = atomicAdd(rs.ticket, 1u);
-    last = (t == gridDim.x - 1);
+    last = (t == (unsigned)nblocks - 1);
   }
   __syncthreads();
   if (!last) return false;
@@ -573,7 +574,7 @@ __device__ bool grid_sum(double (&v)[NRED], const ReduceScratch& rs, double (&to
 #pragma unroll
   for (int q = 0; q < NRED; ++q) {
     double x = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
+    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
       x += __ldcg(rs.partials + (size_t)q * rs.max_blocks + b);
     w[q] = x;
   }
@@ -586,6 +587,11 @@ __device__ bool grid_sum(double (&v)[NRED], const ReduceScratch& rs, double (&to
     return true;
   }
   return false;
+}
+
+template <int NRED>
+__device__ __forceinline__ bool grid_sum(double (&v)[NRED], const ReduceScratch& rs, double (&tot)[NRED]) {
+  return grid_sum<NRED>(v, rs, tot, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // ------------------------------------------------------------ geometry

@@ -1,6 +1,6 @@
 // Double-float Wilson operator with two threads per site (the operator of
-// Sec. 3 kernel 1 in ~48-bit double-float arithmetic on the FP32 pipe, used
-// for the intermediate true residuals of mixed-precision CG).
+// Sec. 3 kernel 1 in ~48-bit double-float arithmetic on the FP32 pipe): the
+// LQ_DF64 precision of lq_apply_M and lq_apply_MdagM.
 //
 // Double-float values double the registers of every quantity, and the long
 // dependent chains of the compensated sums need many warps in flight.  The
@@ -195,51 +195,6 @@ struct DFEpiStore {
     }
   }
   __device__ void finalize(double (&)[1]) const {}
-};
-
-// |r|^2 of a single solve goes to its state
-struct DFFinSolver {
-  SolverState* st;
-  __device__ void operator()(double rr) const { st->rr_true = rr; }
-};
-
-// r = phi - M^dag tmp (double-float), r_lo = r in the inner format, |r|^2 to the
-// finaliser; RDF: r is also stored as a double-float field (rdf)
-template <SStore SLO, class Fin = DFFinSolver, bool RDF = true>
-struct DFEpiResidual {
-  static constexpr bool REDUCE = true;
-  SpinorRef phi, rdf, rlo;
-  Fin fin;
-  __device__ void apply(int V, int s, int half, bool active, const cplx<df64> v[6], double (&red)[1]) const {
-    const float4* ph = static_cast<const float4*>(phi.p);
-    float4* rp = static_cast<float4*>(rdf.p);
-    cplx<float> mine[6];
-    float a = 0.f;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const int comp = (k < 3) ? 3 * half + k : 3 * (half + 2) + (k - 3);
-      const cplx<df64> f = ldf(ph, (size_t)comp * V + s);
-      const cplx<df64> r = {f.re - v[k].re, f.im - v[k].im};
-      if (RDF && active) rp[(size_t)comp * V + s] = make_float4(r.re.hi, r.re.lo, r.im.hi, r.im.lo);
-      mine[k] = {(float)r.re, (float)r.im};
-      a = fmaf(mine[k].re, mine[k].re, a);
-      a = fmaf(mine[k].im, mine[k].im, a);
-    }
-    // the inner-format copy needs all 12 components of the site (per-site norm): lane 0 gathers
-    cplx<float> full[12];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const cplx<float> o = {__shfl_xor_sync(0xffffffffu, mine[k].re, 1), __shfl_xor_sync(0xffffffffu, mine[k].im, 1)};
-      // lane 0 holds spins 0, 2; the partner spins 1, 3
-      const int ca = (k < 3) ? k : 6 + (k - 3);        // own components (lane 0 view)
-      const int cb = (k < 3) ? 3 + k : 9 + (k - 3);    // partner's components
-      full[ca] = mine[k];
-      full[cb] = o;
-    }
-    if (active && half == 0) store_spinor<SLO, float>(rlo, V, s, full);
-    if (active) red[0] += (double)a;
-  }
-  __device__ void finalize(double (&tot)[1]) const { fin(tot[0]); }
 };
 
 // ------------------------------------------------------------ prefetching variant

@@ -244,24 +244,21 @@ __device__ __noinline__ void split_site64(Geom geo, const double2* psi, int sstr
 // Component of element k of a lane's six (spin half, then spin half + 2, colour fastest).
 __device__ __forceinline__ int fix_comp(int half, int k) { return k < 3 ? 3 * half + k : 3 * (half + 2) + (k - 3); }
 
+// Applies M (or M^dag) at the sites of pair `first`, first + stride, ... of one lattice.
 // Spinor fields are [chunk][element] with chunk stride `sstride` (V for a single lattice, the
 // batch's element count for one column of a batch) and the lattice's sites at elements
 // off .. off + V - 1; `in.norm` holds the sites' exponent words.  The epilogue gets the
-// element index.  MINB: resident blocks per SM asked for (register cap).
-template <bool DAG, class Epi, int MINB>
-__global__ void __launch_bounds__(kFixBlock, MINB)
-    dslash_fix_kernel(Geom geo, FixGauge U, SpinorRef in, int sstride, int off, double kappa, Epi epi,
-                      ReduceScratch rs) {
-  if (epi.halted()) return;
+// element index.
+template <bool DAG, class Epi>
+__device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, const SpinorRef& in, int sstride, int off,
+                                          double kappa, const Epi& epi, int first, int stride, double (&red)[1]) {
   constexpr int SF = DAG ? +1 : -1;
   const double2* psi = static_cast<const double2*>(in.p) + off;
   const int* word = reinterpret_cast<const int*>(in.norm) + off;
   const bool bad = __ldg(U.bad) != 0;
-  double red[1] = {0.0};
   const int half = threadIdx.x & 1, ls = -half;
   const int Vr = (geo.V + 15) & ~15;                     // whole warps iterate together
-  const int stride = (gridDim.x * blockDim.x) >> 1;
-  for (int s0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 1; s0 < Vr; s0 += stride) {
+  for (int s0 = first; s0 < Vr; s0 += stride) {
     const bool active = s0 < geo.V;
     const int s = active ? s0 : 0;
     int c[4];
@@ -314,6 +311,16 @@ __global__ void __launch_bounds__(kFixBlock, MINB)
     }
     epi.apply(sstride, off + s, half, active, v, red);
   }
+}
+
+// MINB: resident blocks per SM asked for (register cap).
+template <bool DAG, class Epi, int MINB>
+__global__ void __launch_bounds__(kFixBlock, MINB)
+    dslash_fix_kernel(Geom geo, FixGauge U, SpinorRef in, double kappa, Epi epi, ReduceScratch rs) {
+  if (epi.halted()) return;
+  double red[1] = {0.0};
+  fix_sites<DAG, Epi>(geo, U, in, geo.V, 0, kappa, epi, (blockIdx.x * blockDim.x + threadIdx.x) >> 1,
+                      (gridDim.x * blockDim.x) >> 1, red);
   if constexpr (Epi::REDUCE) {
     double tot[1];
     if (grid_sum<1>(red, rs, tot)) epi.finalize(tot);
@@ -405,8 +412,8 @@ struct FinSolver {
 };
 
 // True residual: v = M^dag (M x) -> r = phi - v, |r|^2 to the finaliser; STORE_LO: r also in
-// the inner format (reliable update)
-template <SStore SLO, bool STORE_LO, class Fin = FinSolver>
+// the inner format (reliable update); STORE_R: r itself
+template <SStore SLO, bool STORE_LO, class Fin = FinSolver, bool STORE_R = true>
 struct FixEpiResidual {
   static constexpr bool REDUCE = true;
   SpinorRef phi, r, r_lo;
@@ -417,7 +424,7 @@ struct FixEpiResidual {
     load6(phi, V, e, half, ph);
 #pragma unroll
     for (int k = 0; k < 6; ++k) rv[k] = ph[k] - v[k];
-    store6(r, V, e, half, active, rv);
+    if constexpr (STORE_R) store6(r, V, e, half, active, rv);
     if constexpr (STORE_LO) {
       // the inner-format copy needs all 12 components of the site (per-site norm): lane 0 gathers
       cplx<float> full[12];
@@ -435,7 +442,7 @@ struct FixEpiResidual {
   __device__ void finalize(double (&tot)[1]) const { fin(tot[0]); }
 };
 
-// sstride < 0: a single lattice (chunk stride V, sites at elements 0 .. V - 1).  Blocks of 256
+// Blocks of 256
 // threads (128 sites), two per SM; measured slower: 64-site blocks at the same occupancy (286
 // against 241 us at 24^3 x 32: fewer of the x and y neighbours are in the block's own lines),
 // three blocks of 80 registers (344, spills), blocks of 4 x 4 x 4 x 2 sites (304: shorter runs per
@@ -443,18 +450,17 @@ struct FixEpiResidual {
 // cap (its warps are alone on their schedulers: 8^4 14.4 -> 10.3 us).
 template <bool DAG, class Epi>
 inline void launch_dslash_fix(const Geom& geo, const FixGauge& U, SpinorRef in, double kappa, const Epi& epi,
-                              const ReduceScratch& rs, cudaStream_t stream, int sstride = -1, int off = 0) {
-  const int st = sstride < 0 ? geo.V : sstride;
+                              const ReduceScratch& rs, cudaStream_t stream) {
   static const int sms = sm_count();
   const int blocks = grid_for(2 * geo.V, kFixBlock);
   if (blocks <= sms) {
     int bs = kFixBlock;
     while (bs > 32 && grid_for(2 * geo.V, bs) < sms) bs >>= 1;
-    dslash_fix_kernel<DAG, Epi, 1><<<grid_for(2 * geo.V, bs), bs, 0, stream>>>(geo, U, in, st, off, kappa, epi, rs);
+    dslash_fix_kernel<DAG, Epi, 1><<<grid_for(2 * geo.V, bs), bs, 0, stream>>>(geo, U, in, kappa, epi, rs);
     return;
   }
   static const int wave = resident_grid(reinterpret_cast<const void*>(&dslash_fix_kernel<DAG, Epi, 2>), kFixBlock);
-  dslash_fix_kernel<DAG, Epi, 2><<<std::min(blocks, wave), kFixBlock, 0, stream>>>(geo, U, in, st, off, kappa, epi, rs);
+  dslash_fix_kernel<DAG, Epi, 2><<<std::min(blocks, wave), kFixBlock, 0, stream>>>(geo, U, in, kappa, epi, rs);
 }
 
 }  // namespace lq

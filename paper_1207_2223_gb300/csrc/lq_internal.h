@@ -89,8 +89,6 @@ struct lq_ctx {
   lq::Field phi64, x64, r64, p64, t64, tmp64;
   // low-precision solver fields, one set per storage format (indexed by SStore)
   lq::Field r_lo[lq::kNumSStore], p_lo[lq::kNumSStore], t_lo[lq::kNumSStore], x_lo[lq::kNumSStore];
-  // double-float reliable updates: phi, the accumulated solution, M x, the residual
-  lq::Field phi_df, x_df, tmp_df, r_df;
 
   // molecular dynamics: momenta / forces double [32][V], the start momenta,
   // the force buffer, the gauge field at the start of a trajectory, Y = M X
@@ -112,7 +110,6 @@ struct lq_ctx {
   std::map<std::tuple<int, int, int, double>, lq::GraphEntry> graphs;
   void* batch = nullptr;                 // workspace of lq_solve_batch (k_batch.cu)
   int use_graphs = 1;                    // CG iterations as CUDA graphs (lq_set_option)
-  int df_updates = 1;                    // double-float intermediate reliable updates (lq_set_option)
   int pair_sites = 0;                    // two-site packed stencil for 16-bit storage (lq_set_option)
   int staged = 0;                        // links shared in-block through shared memory (lq_set_option)
   int batch_rb = 0;                      // batched solves: right-hand sides per thread (0: autotuned)
@@ -141,11 +138,11 @@ void destroy_batch_work(void* w);
 void launch_pack_gauge64(const Geom& g, const double* canon, void* soa, cudaStream_t st);
 void launch_unpack_gauge64(const Geom& g, const void* soa, double* canon, cudaStream_t st);
 void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* bad, cudaStream_t st);
+// the context's fixed-point links, built on `st` unless they are current
+cudaError_t ensure_fix_gauge(lq_ctx* c, cudaStream_t st);
 void launch_convert_gauge(const Geom& g, const void* soa64, GStore dst, void* out, cudaStream_t st);
 void launch_pack_spinor(const Geom& g, const double* canon, SStore s, SpinorRef out, cudaStream_t st);
 void launch_unpack_spinor(const Geom& g, SStore s, SpinorRef in, double* canon, cudaStream_t st);
-// FP64 <-> double-float field conversion
-void launch_convert_spinor(const Geom& g, SStore a, SpinorRef in, SStore b, SpinorRef out, cudaStream_t st);
 
 // ---- BLAS-1 (k_blas.cu)
 // phi2 = |phi|^2 -> state; x = 0; r = phi; p = phi (each in its own format)
@@ -185,15 +182,6 @@ void pair_cg2(lq_ctx* c, const void* gauge, double kappa, cudaStream_t stream); 
 // ---- FP64 CG pieces (k_cg64.cu)
 void cg64_iteration(lq_ctx* c, double kappa, cudaStream_t stream);
 void cg64_true_residual(lq_ctx* c, double kappa, int store_lo_prec, cudaStream_t stream);
-
-// ---- double-float reliable update (k_cgdf.cu): x_df += x_lo; r = phi_df - M^dag M x_df
-// stored as r_df and in the inner format r_lo[prec]; |r|^2 -> state->rr_true
-void df_reliable_update(lq_ctx* c, double kappa, int inner_prec, cudaStream_t stream);
-// x_df += x_lo; x_lo = 0 (no residual)
-void df_accumulate(lq_ctx* c, int inner_prec, cudaStream_t stream);
-// x = 0, r = p = src in format s, from a double-float residual
-void launch_inner_restart_df(const Geom& g, SpinorRef src, SStore s, SpinorRef x, SpinorRef r, SpinorRef p,
-                             cudaStream_t stream);
 
 // ---- low-precision CG iteration (k_cglo.cu)
 void cglo_iteration(lq_ctx* c, int prec, double kappa, cudaStream_t stream);
