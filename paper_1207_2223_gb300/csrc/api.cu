@@ -411,7 +411,8 @@ struct PhaseTimer {
 // p -= eps (F_gauge + F_fermion) at the current links; one solve for X = (M^dag M)^{-1} phi
 lq_status md_force_step(lq_ctx* c, const lq_hmc_params* hp, double eps, lq_traj_result* res, PhaseTimer& tm) {
   tm.begin(PhaseTimer::kGauge);
-  launch_gauge_force(c->geo, c->gauge64, c->mom, hp->beta, eps, true, c->stream);
+  LQ_TRY(require_fix(c));
+  launch_gauge_force(c->geo, fix_gauge_of(c), c->mom, hp->beta, eps, true, c->stream);
   tm.end(PhaseTimer::kGauge);
   lq_solve_stats s{};
   tm.begin(PhaseTimer::kSolve);
@@ -494,7 +495,7 @@ lq_status trajectory_after_heatbath(lq_ctx* c, const lq_hmc_params* hp, double u
   // Delta H from per-site differences
   launch_fermion_action_diff(g, c->phi64.ref(), c->x64.ref(), c->chi64.ref(), c->rs, c->dscalar + 0, c->stream);
   launch_kinetic_diff(g, c->mom, c->mom0, c->rs, c->dscalar + 1, c->stream);
-  launch_plaquette(g, c->gauge_old, c->gauge64, c->rs, c->dscalar + 2, c->stream);
+  launch_plaquette_diff(g, c->gauge_old, c->gauge64, c->rs, c->dscalar + 2, c->stream);
   r.kernel_launches += 3;
   LQ_CUDA(c, cudaGetLastError());
   LQ_TRY(read_scalars(c));
@@ -515,7 +516,8 @@ lq_status trajectory_after_heatbath(lq_ctx* c, const lq_hmc_params* hp, double u
                                cudaMemcpyDeviceToDevice, c->stream));
     gauge_changed(c);
   }
-  launch_plaquette(g, c->gauge64, nullptr, c->rs, c->dscalar + 4, c->stream);
+  LQ_TRY(require_fix(c));
+  launch_plaquette(g, fix_gauge_of(c), c->rs, c->dscalar + 4, c->stream);
   r.kernel_launches += 1;
   LQ_TRY(read_scalars(c));
   r.plaquette = c->dscalar_host[4] / (18.0 * g.V);
@@ -855,8 +857,8 @@ lq_status lq_time_dslash(lq_ctx* c, const double* in, double kappa, int dagger, 
 lq_status lq_plaquette(lq_ctx* c, double* plaq) {
   if (!c) return LQ_ERR_ARG;
   if (!plaq) return fail(c, LQ_ERR_ARG, "null output");
-  LQ_TRY(require_gauge(c, LQ_F64));
-  launch_plaquette(c->geo, c->gauge64, nullptr, c->rs, c->dscalar, c->stream);
+  LQ_TRY(require_fix(c));
+  launch_plaquette(c->geo, fix_gauge_of(c), c->rs, c->dscalar, c->stream);
   LQ_CUDA(c, cudaGetLastError());
   LQ_TRY(read_scalars(c));
   *plaq = c->dscalar_host[0] / (18.0 * c->geo.V);
@@ -866,8 +868,8 @@ lq_status lq_plaquette(lq_ctx* c, double* plaq) {
 lq_status lq_gauge_action(lq_ctx* c, double beta, double* S) {
   if (!c) return LQ_ERR_ARG;
   if (!S) return fail(c, LQ_ERR_ARG, "null output");
-  LQ_TRY(require_gauge(c, LQ_F64));
-  launch_plaquette(c->geo, c->gauge64, nullptr, c->rs, c->dscalar, c->stream);
+  LQ_TRY(require_fix(c));
+  launch_plaquette(c->geo, fix_gauge_of(c), c->rs, c->dscalar, c->stream);
   LQ_CUDA(c, cudaGetLastError());
   LQ_TRY(read_scalars(c));
   *S = beta * (6.0 * c->geo.V - c->dscalar_host[0] / 3.0);
@@ -876,9 +878,9 @@ lq_status lq_gauge_action(lq_ctx* c, double beta, double* S) {
 
 lq_status lq_gauge_force(lq_ctx* c, double* F, double beta) {
   if (!c) return LQ_ERR_ARG;
-  LQ_TRY(require_gauge(c, LQ_F64));
+  LQ_TRY(require_fix(c));
   LQ_TRY(ensure_md_fields(c));
-  launch_gauge_force(c->geo, c->gauge64, c->force, beta, 0.0, false, c->stream);
+  launch_gauge_force(c->geo, fix_gauge_of(c), c->force, beta, 0.0, false, c->stream);
   LQ_CUDA(c, cudaGetLastError());
   return deliver_mom(c, c->force, F);
 }

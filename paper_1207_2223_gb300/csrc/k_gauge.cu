@@ -1,12 +1,15 @@
 // Gauge-side kernels of the molecular dynamics (paper Sec. 3, kernels 2 and 4;
 // Eq. 5): plaquettes and the Wilson gauge action, the gauge force fused with
 // the momentum update, the link update U <- exp(i eps p) U with
-// reunitarisation, and the kinetic-energy difference.  All FP64.
+// reunitarisation, and the kinetic-energy difference.  All FP64; plaquettes and
+// staples multiply links in fixed point (lq_fixsu3.cuh), and in FP64 arithmetic
+// when some link is not unitary.
 //
 // Momenta and forces are stored site-major as double [32][V], entry
 // (4 mu + ... ) -> index (8 mu + a) * V + site, for su(3) coefficient a.
 #include "lq_internal.h"
 #include "lq_su3.cuh"
+#include "lq_fixsu3.cuh"
 
 namespace lq {
 
@@ -30,9 +33,53 @@ __device__ __forceinline__ double site_plaquettes(const double2* g, const Geom& 
   return sum;
 }
 
-// red[0] = sum_x sum_{mu<nu} Re tr U_P (gauge a);  red[1] = same minus for gauge b (when given)
+// out[0] = sum_x sum_{mu<nu} Re tr U_P with fixed-point links: per site the two-link products of
+// both paths row by row and their scalar product, summed exactly in units of 2^-58.  24^3 x 32: 1.19 ms
+// in FP64 arithmetic (1400 multiply-adds per site at 2 per clock and SM), 0.31 ms here.
+__global__ void __launch_bounds__(kFixBlock, 2) plaquette_fix_kernel(Geom geo, const int4* __restrict__ g,
+                                                                     const int* __restrict__ bad, ReduceScratch rs,
+                                                                     double* out) {
+  if (__ldg(bad)) return;                              // plaquette_kernel computes it
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  double red[1] = {0.0};
+  if (s < geo.V) {
+    int c[4];
+    site_coords(geo, s, c);
+    long long sum = 0;
+#pragma unroll 1
+    for (int mu = 0; mu < 3; ++mu) {
+      const int xm = nbr_fwd(geo, s, c, mu);
+#pragma unroll 1
+      for (int nu = mu + 1; nu < 4; ++nu) {
+        const int xn = nbr_fwd(geo, s, c, nu);
+        const Fix3 p = load_fix3(g, geo.V, nu, xm), q = load_fix3(g, geo.V, mu, xn);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          long long a[3][2], b[3][2];
+          fix_vecmat<false>(fix_row(g, geo.V, mu, s, i), p, a);
+          fix_vecmat<false>(fix_row(g, geo.V, nu, s, i), q, b);
+          const FixRow x = fix_split(a), y = fix_split(b);
+          long long h = 0, m = 1 << 30;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            fix_mac(h, m, x.re[k].x, x.re[k].y, y.re[k]);
+            fix_mac(h, m, x.im[k].x, x.im[k].y, y.im[k]);
+          }
+          sum += h + (m >> 31);
+        }
+      }
+    }
+    red[0] = (double)sum * 0x1p-58;
+  }
+  double tot[1];
+  if (grid_sum<1>(red, rs, tot)) out[0] = tot[0];
+}
+
+// red[0] = sum_x sum_{mu<nu} Re tr U_P (gauge a);  red[1] = same minus for gauge b (when given).
+// only_bad, when not null: runs only if it points to a non-zero flag (links that are not unitary).
 __global__ void __launch_bounds__(kBS) plaquette_kernel(Geom geo, const double2* ga, const double2* gb,
-                                                        ReduceScratch rs, double* out) {
+                                                        const int* only_bad, ReduceScratch rs, double* out) {
+  if (only_bad && !__ldg(only_bad)) return;
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   double red[2] = {0.0, 0.0};
   if (s < geo.V) {
@@ -48,9 +95,103 @@ __global__ void __launch_bounds__(kBS) plaquette_kernel(Geom geo, const double2*
 
 // F_a(x, mu) = (beta/3) Im tr(t_a U_mu(x) Sigma_mu(x)), Sigma the six staples.
 // UPDATE: p -= eps F, otherwise F is stored.
+//
+// Fixed point, one thread per link.  The rows of a staple are independent chains of two
+// row-vector products, so one plane needs two links in registers (72) and one row at a time of
+// the third; the staple sum is 18 64-bit integers.  Units: staples 2^-59, their sum 2^-58 after a
+// shift, W = U Sigma 2^-57; |Sigma| <= 6 keeps every sum in 63 bits.  1404 real products per link
+// took 770 clocks per link and SM on the FP64 pipe (24^3 x 32: 4.65 ms); 1.28 ms here, now bound by
+// load latency at 8 warps per SM (168 registers for 12 warps spill: 1.36 ms; 128: 1.51 ms).
 template <bool UPDATE>
-__global__ void __launch_bounds__(kBS) gauge_force_kernel(Geom geo, const double2* g, double* f, double beta,
-                                                          double eps) {
+__global__ void __launch_bounds__(128, 2) gauge_force_fix_kernel(Geom geo, const int4* __restrict__ g,
+                                                                 const int* __restrict__ bad, double* f, double beta,
+                                                                 double eps) {
+  if (__ldg(bad)) return;                              // gauge_force_kernel computes it
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= 4 * geo.V) return;
+  const int mu = idx / geo.V, s = idx - mu * geo.V;
+  int c[4];
+  site_coords(geo, s, c);
+  const int xm = nbr_fwd(geo, s, c, mu);
+  int cm[4] = {c[0], c[1], c[2], c[3]};
+  cm[mu] = (c[mu] + 1) % geo.L[mu];
+  long long S[3][3][2] = {};
+#pragma unroll 1
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu == mu) continue;
+    {
+      // upper: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
+      const Fix3 b = load_fix3(g, geo.V, mu, nbr_fwd(geo, s, c, nu)), d = load_fix3(g, geo.V, nu, s);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        long long w[3][2], v[3][2];
+        fix_vecmat<true>(fix_row(g, geo.V, nu, xm, i), b, w);
+        fix_vecmat<true>(fix_split(w), d, v);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) { S[i][j][0] += v[j][0]; S[i][j][1] += v[j][1]; }
+      }
+    }
+    {
+      // lower: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
+      const int xmn = nbr_bwd(geo, s, c, nu), xpm = nbr_bwd(geo, xm, cm, nu);
+      const Fix3 b = load_fix3(g, geo.V, mu, xmn), d = load_fix3(g, geo.V, nu, xmn);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        long long w[3][2], v[3][2];
+        fix_vecmat<true>(fix_row_dag(g, geo.V, nu, xpm, i), b, w);
+        fix_vecmat<false>(fix_split(w), d, v);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) { S[i][j][0] += v[j][0]; S[i][j][1] += v[j][1]; }
+      }
+    }
+  }
+  // W = U Sigma
+  FixRow R[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      R[k].re[j] = fix_limbs(S[k][j][0] >> 1);
+      R[k].im[j] = fix_limbs(S[k][j][1] >> 1);
+    }
+  long long W[3][3][2];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const FixRow u = fix_row(g, geo.V, mu, s, i);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      long long rh = 0, rm = 1 << 30, ih = 0, im = 1 << 30;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        fix_mac(rh, rm, u.re[k].x, u.re[k].y, R[k].re[j]);
+        fix_mac(rh, rm, -u.im[k].x, -u.im[k].y, R[k].im[j]);
+        fix_mac(ih, im, u.re[k].x, u.re[k].y, R[k].im[j]);
+        fix_mac(ih, im, u.im[k].x, u.im[k].y, R[k].re[j]);
+      }
+      W[i][j][0] = rh + (rm >> 31);
+      W[i][j][1] = ih + (im >> 31);
+    }
+  }
+  // f_a = Im tr(t_a W) (im_tr_ta), the sums of matrix elements exact
+  const double r2 = 0.70710678118654752440 * 0x1p-57 * (beta / 3.0), r6 = 0.40824829046386301637 * 0x1p-57 * (beta / 3.0);
+  const double fa[8] = {r2 * (double)(W[0][1][1] + W[1][0][1]), r2 * (double)(W[0][1][0] - W[1][0][0]),
+                        r2 * (double)(W[0][0][1] - W[1][1][1]), r2 * (double)(W[0][2][1] + W[2][0][1]),
+                        r2 * (double)(W[0][2][0] - W[2][0][0]), r2 * (double)(W[1][2][1] + W[2][1][1]),
+                        r2 * (double)(W[1][2][0] - W[2][1][0]),
+                        r6 * (double)(W[0][0][1] + W[1][1][1] - 2 * W[2][2][1])};
+#pragma unroll
+  for (int a = 0; a < 8; ++a) {
+    double* q = f + ((size_t)mu * 8 + a) * geo.V + s;
+    if (UPDATE) *q -= eps * fa[a];
+    else *q = fa[a];
+  }
+}
+
+// The same in FP64 arithmetic, for links that are not unitary (*bad set).
+template <bool UPDATE>
+__global__ void __launch_bounds__(kBS) gauge_force_kernel(Geom geo, const double2* g, const int* bad, double* f,
+                                                          double beta, double eps) {
+  if (!__ldg(bad)) return;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= 4 * geo.V) return;
   const int mu = idx / geo.V, s = idx - mu * geo.V;
@@ -133,16 +274,24 @@ __global__ void __launch_bounds__(kBS) kinetic_diff_kernel(int V, const double* 
   if (grid_sum<1>(red, rs, tot)) out[0] = tot[0];
 }
 
-void launch_plaquette(const Geom& g, const void* ga, const void* gb, const ReduceScratch& rs, double* out,
-                      cudaStream_t st) {
+void launch_plaquette_diff(const Geom& g, const void* ga, const void* gb, const ReduceScratch& rs, double* out,
+                           cudaStream_t st) {
   plaquette_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g, static_cast<const double2*>(ga),
-                                                       static_cast<const double2*>(gb), rs, out);
+                                                       static_cast<const double2*>(gb), nullptr, rs, out);
 }
-void launch_gauge_force(const Geom& g, const void* gauge, double* f, double beta, double eps, bool update,
+void launch_plaquette(const Geom& g, const FixGauge& U, const ReduceScratch& rs, double* out, cudaStream_t st) {
+  plaquette_fix_kernel<<<grid_for(g.V, kFixBlock), kFixBlock, 0, st>>>(g, U.fix, U.bad, rs, out);
+  plaquette_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g, U.f64, nullptr, U.bad, rs, out);
+}
+template <bool UPDATE>
+static void gauge_force(const Geom& g, const FixGauge& U, double* f, double beta, double eps, cudaStream_t st) {
+  gauge_force_fix_kernel<UPDATE><<<grid_for(4 * g.V, 128), 128, 0, st>>>(g, U.fix, U.bad, f, beta, eps);
+  gauge_force_kernel<UPDATE><<<grid_for(4 * g.V, kBS), kBS, 0, st>>>(g, U.f64, U.bad, f, beta, eps);
+}
+void launch_gauge_force(const Geom& g, const FixGauge& U, double* f, double beta, double eps, bool update,
                         cudaStream_t st) {
-  const int grid = grid_for(4 * g.V, kBS);
-  if (update) gauge_force_kernel<true><<<grid, kBS, 0, st>>>(g, static_cast<const double2*>(gauge), f, beta, eps);
-  else gauge_force_kernel<false><<<grid, kBS, 0, st>>>(g, static_cast<const double2*>(gauge), f, beta, eps);
+  if (update) gauge_force<true>(g, U, f, beta, eps, st);
+  else gauge_force<false>(g, U, f, beta, eps, st);
 }
 void launch_link_update(const Geom& g, void* gauge, const double* p, double eps, cudaStream_t st) {
   link_update_kernel<<<grid_for(4 * g.V, kBS), kBS, 0, st>>>(g, static_cast<double2*>(gauge), p, eps);

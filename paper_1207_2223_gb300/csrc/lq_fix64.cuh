@@ -32,29 +32,29 @@
 #pragma once
 #include <algorithm>
 
-#include "lq_dslash.cuh"
+#include "lq_internal.h"
 
 namespace lq {
 
 constexpr int kFixBlock = 256;
 
-// Links of one lattice: fixed-point int4 [4][9][V] (re.hi, re.lo, im.hi, im.lo), the FP64
-// links for sites that take the FP64 path, and the flag "some link is not unitary".
-struct FixGauge {
-  const int4* fix;
-  const double2* f64;
-  const int* bad;
-};
-
-}  // namespace lq
-struct lq_ctx;
-namespace lq {
-FixGauge fix_gauge_of(const lq_ctx* c);   // k_apply.cu
-
+// round(x 2^61) of |x| < 2 as limbs (integer operations: FP64 conversions issue at 2 per clock
+// and SM; 24^3 x 32 links 166 us with them); larger or non-finite x gives some other value
+__device__ __forceinline__ int2 fix_element(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned d = 1023u - ((unsigned)hi << 1 >> 21);
+  const unsigned long long m =
+      ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(x)) << 10;
+  unsigned long long v;
+  asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(d));           // shifts beyond 63 give 0
+  v = (v >> 1) + (v & 1);
+  const long long s = hi >> 31, w = ((long long)v ^ s) - s;
+  const int lo = (int)((unsigned)w << 1) >> 1;                     // low 31 bits, signed
+  return make_int2((int)((w - lo) >> 31), lo);
+}
 __device__ __forceinline__ int4 fix_link(double2 u) {
-  const long long a = __double2ll_rn(u.x * 2305843009213693952.0), b = __double2ll_rn(u.y * 2305843009213693952.0);
-  const int al = (int)((unsigned)a << 1) >> 1, bl = (int)((unsigned)b << 1) >> 1;      // low 31 bits, signed
-  return make_int4((int)((a - al) >> 31), al, (int)((b - bl) >> 31), bl);
+  const int2 a = fix_element(u.x), b = fix_element(u.y);
+  return make_int4(a.x, a.y, b.x, b.y);
 }
 
 // Running sums of one lane: the upper spin, the lower spin handed to the partner and the

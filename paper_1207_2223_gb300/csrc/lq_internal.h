@@ -61,6 +61,15 @@ struct GraphEntry {
   cudaGraphExec_t exec = nullptr;
 };
 
+// Links of one lattice as the fixed-point kernels read them (lq_fix64.cuh): int4 [4][9][V]
+// (re.hi, re.lo, im.hi, im.lo), the FP64 links for what takes FP64 arithmetic, and the device
+// flag "some link is not unitary".
+struct FixGauge {
+  const int4* fix;
+  const double2* f64;
+  const int* bad;
+};
+
 }  // namespace lq
 
 struct lq_ctx {
@@ -140,6 +149,7 @@ void launch_unpack_gauge64(const Geom& g, const void* soa, double* canon, cudaSt
 void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* bad, cudaStream_t st);
 // the context's fixed-point links, built on `st` unless they are current
 cudaError_t ensure_fix_gauge(lq_ctx* c, cudaStream_t st);
+FixGauge fix_gauge_of(const lq_ctx* c);
 void launch_convert_gauge(const Geom& g, const void* soa64, GStore dst, void* out, cudaStream_t st);
 void launch_pack_spinor(const Geom& g, const double* canon, SStore s, SpinorRef out, cudaStream_t st);
 void launch_unpack_spinor(const Geom& g, SStore s, SpinorRef in, double* canon, cudaStream_t st);
@@ -206,9 +216,11 @@ void launch_heatbath_chi(const Geom& g, uint64_t seed, uint64_t traj, SpinorRef 
 double metropolis_uniform(uint64_t seed, uint64_t traj);
 
 // ---- gauge side (k_gauge.cu); momenta / forces are double [32][V]
-void launch_plaquette(const Geom& g, const void* ga, const void* gb, const ReduceScratch& rs, double* out,
-                      cudaStream_t st);
-void launch_gauge_force(const Geom& g, const void* gauge, double* f, double beta, double eps, bool update,
+// out[0] = sum_x sum_{mu<nu} Re tr U_P; the difference of two gauge fields, per site, goes to out[1]
+void launch_plaquette(const Geom& g, const FixGauge& U, const ReduceScratch& rs, double* out, cudaStream_t st);
+void launch_plaquette_diff(const Geom& g, const void* ga, const void* gb, const ReduceScratch& rs, double* out,
+                           cudaStream_t st);
+void launch_gauge_force(const Geom& g, const FixGauge& U, double* f, double beta, double eps, bool update,
                         cudaStream_t st);
 void launch_link_update(const Geom& g, void* gauge, const double* p, double eps, cudaStream_t st);
 void launch_pack_mom(const Geom& g, const double* canon, double* soa, cudaStream_t st);

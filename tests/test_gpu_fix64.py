@@ -86,3 +86,26 @@ def test_non_finite_values_reach_their_neighbours_only(lq, value):
     d = np.abs(x - x[s])
     d = np.minimum(d, np.array(dims) - d).sum(axis=1)
     assert np.array_equal(finite, d > 1)
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7), (2, 2, 2, 2)])
+@pytest.mark.parametrize("kind", ["gauss", "ones", "not_unitary"])
+def test_plaquette_and_gauge_force(lq, dims, kind):
+    """Staples and plaquettes in fixed point, and in FP64 arithmetic for general matrices, against
+    the oracle.  Bounds: a staple is three FP64 matrix products (at most 3 * 9 roundings of sums of
+    |U|^3), six of them times a link; 128 units of 2^-53 of (beta / 3) * 18 * max |U|^4."""
+    from oracle.gauge import gauge_force, plaquette
+    U, _ = _fields(dims, kind)
+    V = Lattice(dims).V
+    ctx = lq.lq_create(dims)
+    try:
+        lq.lq_gauge_set(ctx, dev(U))
+        F = torch.empty((V, 4, 8), dtype=torch.float64, device="cuda")
+        lq.lq_gauge_force(ctx, F, 5.6)
+        F, P = host(F), lq.lq_plaquette(ctx)
+    finally:
+        lq.lq_destroy(ctx)
+    top = max(1.0, np.abs(U).max()) ** 4
+    unit = 128 * 2.0 ** -53
+    assert np.abs(F - gauge_force(U, dims, 5.6)).max() <= unit * 5.6 / 3 * 18 * top
+    assert abs(P - plaquette(U, dims)) <= unit * 3 * top
