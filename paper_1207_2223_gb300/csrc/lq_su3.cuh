@@ -75,7 +75,6 @@ __device__ __forceinline__ void add_to(M3& a, const M3& b) {
 #pragma unroll
   for (int c = 0; c < 9; ++c) a.m[c] = a.m[c] + b.m[c];
 }
-__device__ __forceinline__ double re_trace(const M3& a) { return a.m[0].re + a.m[4].re + a.m[8].re; }
 // Re tr(a b^dag) = Re sum_ij a_ij conj(b_ij)
 __device__ __forceinline__ double re_tr_mul_dag(const M3& a, const M3& b) {
   double s = 0.0;
@@ -100,7 +99,6 @@ __device__ __forceinline__ void im_tr_ta(const M3& W, double f[8]) {
   f[7] = r6 * (W.m[0].im + W.m[4].im - 2.0 * W.m[8].im);
 }
 
-// X = i eps sum_a p_a t_a (anti-Hermitian, traceless)
 // eps P, P = sum_a p_a t_a (Hermitian, traceless)
 __device__ __forceinline__ M3 eps_algebra(const double p[8], double eps) {
   const double r2 = 0.70710678118654752440 * eps;
@@ -117,63 +115,16 @@ __device__ __forceinline__ M3 eps_algebra(const double p[8], double eps) {
   P.m[7] = {r2 * p[5], r2 * p[6]};
   return P;
 }
-// i eps P
-__device__ __forceinline__ M3 i_eps_algebra(const double p[8], double eps) {
-  const M3 P = eps_algebra(p, eps);
-  M3 X;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) X.m[c] = {-P.m[c].im, P.m[c].re};
-  return X;
-}
-
-// exp(X) by scaling and squaring: X / 2^k has Frobenius norm <= 1/4, a Taylor
-// series of 16 terms in Horner form (remainder < 0.25^17 / 17! ~ 6e-25), then
-// k squarings.
-__device__ __forceinline__ M3 expm3(const M3& X) {
-  double n2 = 0.0;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) n2 += norm2(X.m[c]);
-  int k = 0;
-  double nrm = sqrt(n2);
-  while (nrm > 0.25 && k < 60) { nrm *= 0.5; ++k; }
-  const double sc = ldexp(1.0, -k);
-  M3 A;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) A.m[c] = sc * X.m[c];
-  // Horner: E = I + A/1 (I + A/2 (I + ... (I + A/16)))
-  M3 E;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) E.m[c] = {0.0, 0.0};
-  E.m[0] = E.m[4] = E.m[8] = {1.0, 0.0};
-  for (int j = 16; j >= 1; --j) {
-    M3 T = mul(A, E);
-    const double inv = 1.0 / j;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) E.m[c] = inv * T.m[c];
-    E.m[0].re += 1.0; E.m[4].re += 1.0; E.m[8].re += 1.0;
-  }
-  for (int i = 0; i < k; ++i) E = mul(E, E);
-  return E;
-}
-
 // exp(i Q) for Hermitian traceless Q by the Cayley-Hamilton closed form of
 // Morningstar and Peardon, PRD 69 (2004) 054501: exp(iQ) = f0 + f1 Q + f2 Q^2,
 // where the f_j follow from the invariants c0 = det Q = tr(Q^3)/3 and
 // c1 = tr(Q^2)/2 through the eigenvalues 2u, -u + w, -u - w of Q.  For c0 < 0
 // the coefficients come from -Q: f_j(-c0) = (-1)^j conj(f_j(c0)).  With c0 >= 0
-// the denominator 9u^2 - w^2 is at least c1, so the form is well conditioned;
-// Q = 0 (c1 below 1e-12) goes to the Taylor series.  About a quarter of the FP64
-// work of expm3 (one matrix product and a few sines and cosines instead of ~18
-// products).
-__device__ __forceinline__ M3 expi_hermitian(const M3& Q) {
+// the denominator 9u^2 - w^2 is at least c1, so the form is well conditioned for the large Q it
+// is used for (expi_rows takes c1 <= 3/4).
+static __device__ __noinline__ M3 expi_hermitian(const M3& Q) {
   const M3 Q2 = mul(Q, Q);
   const double c1 = 0.5 * (Q2.m[0].re + Q2.m[4].re + Q2.m[8].re);
-  if (!(c1 >= 1e-12)) {
-    M3 X;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) X.m[c] = {-Q.m[c].im, Q.m[c].re};
-    return expm3(X);
-  }
   double t3 = 0.0;   // Re tr(Q Q^2)
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -215,16 +166,86 @@ __device__ __forceinline__ M3 expi_hermitian(const M3& Q) {
   return E;
 }
 
+// Hermitian traceless Q as real numbers: the diagonal and the upper triangle.
+struct H3 {
+  double d[3];
+  cplx<double> u01, u02, u12;
+};
+
+// Rows 0 and 1 of exp(i Q) U for Hermitian traceless Q = eps P (eps_algebra's elements).
+// Every power of Q is a combination of 1, Q, Q^2 with real coefficients (Cayley-Hamilton,
+// Q^3 = c1 Q + c0, c0 = det Q, c1 = tr(Q^2) / 2):
+//   Q^n = a_n + b_n Q + c_n Q^2,  a_{n+1} = c0 c_n,  b_{n+1} = a_n + c1 c_n,  c_{n+1} = b_n,
+// so the Taylor series of exp(iQ) is summed on three real numbers, five FP64 operations a term,
+// without the closed form's arc cosine, sines, square roots and divisions.  The eigenvalues are at
+// most sqrt(4 c1 / 3): 12 terms leave (1/4)^13 / 13! = 2.4e-18 for c1 <= 3/64, 18 leave
+// 1 / 19! = 8e-18 for c1 <= 3/4 (a molecular-dynamics step is below the first); larger Q
+// takes the closed form.  Only two rows of the product are formed: the third is rebuilt.
+__device__ __forceinline__ void expi_rows(const H3& q, double c1, double c0, int terms, const cplx<double> U[9],
+                                          cplx<double> r0[3], cplx<double> r1[3], const H3& q2) {
+  // (a, b, c) / n!; even powers are real (sign + -), odd powers imaginary
+  double a = 1.0, b = 0.0, c = 0.0;
+  double re[3] = {1.0, 0.0, 0.0}, im[3] = {0.0, 0.0, 0.0};
+  const double inv[19] = {0.0,      1.0,      1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,  1.0 / 7,  1.0 / 8, 1.0 / 9,
+                          1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18};
+#pragma unroll
+  for (int n = 1; n <= 18; ++n) {
+    if (n == 13 && terms <= 12) break;
+    const double cn = inv[n] * c, bn = inv[n] * b;
+    c = bn;
+    b = fma(c1, cn, inv[n] * a);
+    a = c0 * cn;
+    if (n & 1) {
+      if (n & 2) { im[0] -= a; im[1] -= b; im[2] -= c; }
+      else       { im[0] += a; im[1] += b; im[2] += c; }
+    } else {
+      if (n & 2) { re[0] -= a; re[1] -= b; re[2] -= c; }
+      else       { re[0] += a; re[1] += b; re[2] += c; }
+    }
+  }
+  // E = A + i B with A = re . (1, Q, Q^2), B = im . (1, Q, Q^2) Hermitian
+  auto comb = [](const double f[3], double x, double y) { return fma(f[2], y, f[1] * x); };
+  const double A00 = re[0] + comb(re, q.d[0], q2.d[0]), B00 = im[0] + comb(im, q.d[0], q2.d[0]);
+  const double A11 = re[0] + comb(re, q.d[1], q2.d[1]), B11 = im[0] + comb(im, q.d[1], q2.d[1]);
+  auto herm = [&](cplx<double> x, cplx<double> y, cplx<double>& up, cplx<double>& low) {
+    const double ar = comb(re, x.re, y.re), ai = comb(re, x.im, y.im), br = comb(im, x.re, y.re), bi = comb(im, x.im, y.im);
+    up = {ar - bi, ai + br};       // A_ij + i B_ij
+    low = {ar + bi, br - ai};      // conj(A_ij) + i conj(B_ij)
+  };
+  cplx<double> e01, e10, e02, e20, e12, e21;
+  herm(q.u01, q2.u01, e01, e10);
+  herm(q.u02, q2.u02, e02, e20);
+  herm(q.u12, q2.u12, e12, e21);
+  const cplx<double> e00{A00, B00}, e11{A11, B11};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    cplx<double> t = cmul(e00, U[j]);
+    t = cmadd(t, e01, U[3 + j]);
+    r0[j] = cmadd(t, e02, U[6 + j]);
+    t = cmul(e10, U[j]);
+    t = cmadd(t, e11, U[3 + j]);
+    r1[j] = cmadd(t, e12, U[6 + j]);
+  }
+}
+
+// 1 / sqrt(x); by three terms of its series next to 1, where the rows of a unitary matrix are
+// (|x - 1| < 1e-4: the next term is below 3e-17)
+__device__ __forceinline__ double inv_norm(double x) {
+  const double d = x - 1.0;
+  if (fabs(d) < 1e-4) return fma(d * fma(d, fma(d, -0.3125, 0.375), -0.5), 1.0, 1.0);
+  return 1.0 / sqrt(x);
+}
+
 // Gram-Schmidt on rows 0, 1; row 2 = conj(row0 x row1)
 __device__ __forceinline__ void reunitarise(M3& U) {
-  const double n0 = 1.0 / sqrt(norm2(U.m[0]) + norm2(U.m[1]) + norm2(U.m[2]));
+  const double n0 = inv_norm(norm2(U.m[0]) + norm2(U.m[1]) + norm2(U.m[2]));
   for (int j = 0; j < 3; ++j) U.m[j] = n0 * U.m[j];
   // <r0, r1> = sum conj(r0_j) r1_j
   cplx<double> d = cjmul(U.m[0], U.m[3]);
   d = cjmadd(d, U.m[1], U.m[4]);
   d = cjmadd(d, U.m[2], U.m[5]);
   for (int j = 0; j < 3; ++j) U.m[3 + j] = U.m[3 + j] - cmul(d, U.m[j]);
-  const double n1 = 1.0 / sqrt(norm2(U.m[3]) + norm2(U.m[4]) + norm2(U.m[5]));
+  const double n1 = inv_norm(norm2(U.m[3]) + norm2(U.m[4]) + norm2(U.m[5]));
   for (int j = 0; j < 3; ++j) U.m[3 + j] = n1 * U.m[3 + j];
   U.m[6] = conjg(cmul(U.m[1], U.m[5]) - cmul(U.m[2], U.m[4]));
   U.m[7] = conjg(cmul(U.m[2], U.m[3]) - cmul(U.m[0], U.m[5]));

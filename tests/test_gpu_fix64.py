@@ -109,3 +109,28 @@ def test_plaquette_and_gauge_force(lq, dims, kind):
     unit = 128 * 2.0 ** -53
     assert np.abs(F - gauge_force(U, dims, 5.6)).max() <= unit * 5.6 / 3 * 18 * top
     assert abs(P - plaquette(U, dims)) <= unit * 3 * top
+
+
+@pytest.mark.parametrize("eps", [1e-9, 0.02, 0.08, 0.3, 0.45, 2.0])
+def test_link_update_over_step_sizes(lq, eps):
+    """exp(i eps P) U by 12 or 18 terms of its series or by the closed form, per link by the size of
+    eps P (the steps straddle both limits), momenta of zero among them.  Bound: 64 units of 2^-53
+    (about 40 rounded sums of numbers of order 1; the closed form's sines of arguments of order eps |p|)."""
+    from oracle.su3 import link_update
+    dims = (4, 3, 2, 5)
+    lat = Lattice(dims)
+    U = gauge_exp_iA(lat, 0.3, 6)
+    p = np.random.default_rng(3).normal(size=(lat.V, 4, 8))
+    p[5] = 0.0
+    ctx = lq.lq_create(dims)
+    try:
+        lq.lq_gauge_set(ctx, dev(U))
+        lq.lq_link_update(ctx, dev(p), eps)
+        got = torch.empty(U.shape, dtype=torch.complex128, device="cuda")
+        lq.lq_gauge_get(ctx, got)
+    finally:
+        lq.lq_destroy(ctx)
+    got = host(got)
+    ref = link_update(U, p, eps)
+    assert np.abs(got - ref).max() <= 64 * 2.0 ** -53 * max(1.0, eps)
+    assert np.abs(got @ got.conj().swapaxes(-1, -2) - np.eye(3)).max() <= 16 * 2.0 ** -53
