@@ -425,7 +425,7 @@ lq_status md_force_step(lq_ctx* c, const lq_hmc_params* hp, double eps, lq_traj_
   if (st != LQ_OK) return st;
   tm.begin(PhaseTimer::kFermion);
   apply_M64(c, c->x64.ref(), c->y64.ref(), hp->kappa, false, c->stream);
-  launch_fermion_force(c->geo, c->gauge64, c->x64.ref(), c->y64.ref(), c->mom, hp->kappa, eps, true, c->stream);
+  launch_fermion_force(c->geo, fix_gauge_of(c), c->x64.ref(), c->y64.ref(), c->mom, hp->kappa, eps, true, c->stream);
   tm.end(PhaseTimer::kFermion);
   LQ_CUDA(c, cudaGetLastError());
   return LQ_OK;
@@ -894,7 +894,7 @@ lq_status lq_fermion_force(lq_ctx* c, double* F, const double* X, double kappa) 
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
   LQ_TRY(require_fix(c));
   apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
-  launch_fermion_force(c->geo, c->gauge64, c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
+  launch_fermion_force(c->geo, fix_gauge_of(c), c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
   LQ_CUDA(c, cudaGetLastError());
   return deliver_mom(c, c->force, F);
 }
@@ -1104,13 +1104,13 @@ lq_status lq_time_fermion_force(lq_ctx* c, const double* X, double kappa, int n,
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
   LQ_TRY(require_fix(c));
   apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
-  launch_fermion_force(c->geo, c->gauge64, c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
+  launch_fermion_force(c->geo, fix_gauge_of(c), c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventRecord(e0, c->stream);
   for (int i = 0; i < n; ++i)
-    launch_fermion_force(c->geo, c->gauge64, c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
+    launch_fermion_force(c->geo, fix_gauge_of(c), c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
   cudaEventRecord(e1, c->stream);
   lq_status st = cuda_check(c, cudaGetLastError(), "fermion force");
   lq_status sy = cuda_check(c, cudaEventSynchronize(e1), "cudaEventSynchronize");

@@ -228,7 +228,7 @@ void launch_unpack_mom(const Geom& g, const double* soa, double* canon, cudaStre
 void launch_kinetic_diff(const Geom& g, const double* p, const double* p0, const ReduceScratch& rs, double* out,
                          cudaStream_t st);
 // ---- fermion side (k_force.cu)
-void launch_fermion_force(const Geom& g, const void* gauge, SpinorRef X, SpinorRef Y, double* f, double kappa,
+void launch_fermion_force(const Geom& g, const FixGauge& U, SpinorRef X, SpinorRef Y, double* f, double kappa,
                           double eps, bool update, cudaStream_t st);
 void launch_fermion_grad(const Geom& g, SpinorRef X, SpinorRef Y, double* G, double kappa, cudaStream_t st);
 void launch_dot_re(const Geom& g, SpinorRef a, SpinorRef b, const ReduceScratch& rs, double* out, cudaStream_t st);

@@ -134,3 +134,38 @@ def test_link_update_over_step_sizes(lq, eps):
     ref = link_update(U, p, eps)
     assert np.abs(got - ref).max() <= 64 * 2.0 ** -53 * max(1.0, eps)
     assert np.abs(got @ got.conj().swapaxes(-1, -2) - np.eye(3)).max() <= 16 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7), (2, 2, 2, 2)])
+@pytest.mark.parametrize("kind", ["gauss", "site_range", "spin_range", "point", "huge", "not_unitary"])
+def test_fermion_force(lq, dims, kind):
+    """Force of X and Y = M X in fixed point and, where their exponents or the links do not fit, in
+    FP64.  Bound per link: two outer products of projected spinors (rounded products of U, X and Y,
+    at most 64 roundings) of the largest |X| and |Y| of its two sites, times 2 kappa max |U|."""
+    from oracle.fermion import fermion_force_from_X
+    U, X = _fields(dims, kind)
+    scale = 2.0 ** 500 if kind == "huge" else 1.0      # X^2 has to stay finite
+    X = X / (2.0 ** 500 if kind == "huge" else 1.0)
+    V = Lattice(dims).V
+    ctx = lq.lq_create(dims)
+    try:
+        lq.lq_gauge_set(ctx, dev(U))
+        F = torch.empty((V, 4, 8), dtype=torch.float64, device="cuda")
+        lq.lq_fermion_force(ctx, F, dev(X), 0.15)
+        F = host(F) / scale / scale
+    finally:
+        lq.lq_destroy(ctx)
+    X = X / scale
+    ref = fermion_force_from_X(U, X, dims, 0.15)
+    Y = apply_M(U, X, dims, 0.15)
+    grid = dims[::-1]
+    ax, ay = (np.abs(f).max(axis=(1, 2)).reshape(grid) for f in (X, Y))
+    # Y itself is rounded relative to the sites M reads
+    ny = np.maximum(ay, ax)
+    for m in range(4):
+        ny = np.maximum(ny, np.maximum(np.roll(ax, 1, m), np.roll(ax, -1, m)))
+    u = max(1.0, np.abs(U).max()) ** 2
+    for mu in range(4):
+        fwd = lambda a: np.maximum(a, np.roll(a, -1, 3 - mu))   # noqa: E731
+        tol = 2.0 ** -53 * 64 * 24 * 0.3 * u * (fwd(ax) * fwd(ny)).reshape(V, 1)
+        assert np.all(np.abs(F[:, mu] - ref[:, mu]) <= tol), mu
