@@ -6,16 +6,17 @@
 // budget set by its host program.  lq_apply_MdagM_static serves them: it
 // takes the gauge field and the spinors in the canonical layout directly
 // from device buffers the caller owns, and keeps its one intermediate
-// field (M in) in a fixed-size array compiled into this library.
+// field (M in) and the sites' exponent words in fixed-size arrays compiled into
+// this library.
 //
-// That array is a file-scope __device__ variable.  Its name, used in host
-// code, is only a host-side stand-in and not a device address, so host code
-// asks the runtime for the device address (cudaGetSymbolAddress) once per
+// The arrays are file-scope __device__ variables.  Their names, used in host
+// code, are only host-side stand-ins and not device addresses, so host code
+// asks the runtime for the device addresses (cudaGetSymbolAddress) once per
 // device, with that device current, and passes the result to the kernels.
 #include <mutex>
 #include <string>
 
-#include "lq_internal.h"
+#include "lq_fix64.cuh"
 
 namespace lq {
 
@@ -26,58 +27,115 @@ constexpr int kStaticMaxSites = 65536;
 
 static __device__ __align__(256) double2 g_static_scratch[(size_t)kStaticMaxSites * 12];
 
-// out = in - kappa * H in (dagger = 0) or in - kappa * H^dag in (dagger = 1),
-// with U, in and out all in the canonical interleaved layout of lq.h.
-template <bool DAG>
-__global__ void __launch_bounds__(256) hop_canonical_kernel(Geom geo, const double2* __restrict__ U,
-                                                            const double2* __restrict__ in,
-                                                            double2* __restrict__ out, double kappa) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= geo.V) return;
+// Site words of the input (ExpRange, with kBadLinks) and of M in.
+static __device__ int g_static_word[2][kStaticMaxSites];
+
+// Some link of the site is longer than a unitary one: its hops take FP64 arithmetic.
+constexpr int kBadLinks = 1 << 17;
+
+// The word of every site of the input and of its four links; one thread per site and link
+// direction, direction 0 also reads the spinor.  The fixed-point operator below needs both before
+// it reads a site, and canonical buffers come without them.
+__global__ void __launch_bounds__(256) static_scan_kernel(int V, const double2* __restrict__ U,
+                                                          const double2* __restrict__ in, int* __restrict__ word) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;      // four consecutive threads per site
+  const int s = idx >> 2, mu = idx & 3;
+  const bool active = s < V;
+  bool bad = false;
+  ExpRange r;
+  if (active) {
+    const double2* u = U + (size_t)idx * 9;
+    float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const double2 w = u[k];
+      const float a = (float)w.x, b = (float)w.y, n = a * a + b * b;
+      row[k / 3] += n;
+      col[k % 3] += n;
+    }
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 1.001f && col[k] <= 1.001f;
+    bad = !ok;
+    cplx<double> v[3];                                          // thread mu reads spin mu
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double2 w = in[(size_t)s * 12 + 3 * mu + k];
+      v[k] = {w.x, w.y};
+    }
+    r.spin(v);
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    r.mx = max(r.mx, __shfl_xor_sync(0xffffffffu, r.mx, o));
+    r.mn = min(r.mn, __shfl_xor_sync(0xffffffffu, r.mn, o));
+    r.lo |= __shfl_xor_sync(0xffffffffu, r.lo, o);
+    bad |= __shfl_xor_sync(0xffffffffu, (int)bad, o) != 0;
+  }
+  if (active && mu == 0) word[s] = r.word() | (bad ? kBadLinks : 0);
+}
+
+// Canonical buffers: 12 complex numbers per site, links [site][mu][3][3], converted as they are read.
+struct CanonAccess {
+  const double2* psi;
+  const double2* U;
+  __device__ __forceinline__ const double2* site(int comp, int n) const { return psi + (size_t)n * 12 + comp; }
+  __device__ __forceinline__ double2 spin(const double2* p, int k) const { return p[k]; }
+  __device__ __forceinline__ const double2* link(int mu, int s) const { return U + ((size_t)s * 4 + mu) * 9; }
+  __device__ __forceinline__ int4 element(const double2* p, int e) const { return fix_link(__ldg(p + e)); }
+  __device__ __forceinline__ double2 element64(int mu, int e, int s) const { return __ldg(link(mu, s) + e); }
+};
+
+// out = in - kappa * H in (DAG: in - kappa * H^dag in) in fixed point (lq_fix64.cuh) on canonical
+// buffers, two threads per site.  win: words of the input; wlink: the words that hold kBadLinks;
+// wout (may be null): the words of out.  8^4: one thread per site in FP64 arithmetic 65 us,
+// bound by the FP64 pipe of the 16 SMs its blocks reached; here 45 us for the whole call (132).
+template <bool DAG, int MINB>
+__global__ void __launch_bounds__(kFixBlock, MINB) hop_canonical_kernel(Geom geo, const double2* __restrict__ U,
+                                                                     const double2* in, const int* win,
+                                                                     const int* __restrict__ wlink, double2* out,
+                                                                     int* wout, double kappa) {
+  const CanonAccess acc{in, U};
+  const int half = threadIdx.x & 1;
+  const int s0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 1;
+  const bool active = s0 < geo.V;
+  const int s = active ? s0 : 0;
   int c[4];
   site_coords(geo, s, c);
-  cplx<double> acc[12];
+  int f[4], b[4], E = kFixMinExp, any = __ldg(wlink + s) & kBadLinks;
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
-  auto load_psi = [&](int n, cplx<double> p[12]) {
+  for (int m = 0; m < 4; ++m) {
+    f[m] = nbr_fwd(geo, s, c, m);
+    b[m] = nbr_bwd(geo, s, c, m);
+    const int wf = win[f[m]], wb = win[b[m]];
+    any |= (wf | wb) & kFixSlow;
+    any |= __ldg(wlink + b[m]) & kBadLinks;
+    E = max(E, max(wf & 0x7ff, wb & 0x7ff));
+  }
+  const bool slow = any != 0;
+  FixAcc a;
+  if (!slow) {
+    fix_clear(a);
+    fix_hops<DAG>(geo, acc, s, c, f, b, half, E, a);
+  } else {
+    FixAcc t64;
+    split_site64<DAG>(geo, acc, s, half, &t64);
+    a = t64;
+  }
+  cplx<double> v[6];
+  fix_finish(acc, a, s, half, slow, slow ? -kappa : -kappa * __hiloint2double((E - 56) << 20, 0), v);
+  if (active) {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) { double2 w = in[(size_t)n * 12 + k]; p[k] = {w.x, w.y}; }
-  };
-  auto load_u = [&](int n, int mu, cplx<double> u[9]) {
-#pragma unroll
-    for (int k = 0; k < 9; ++k) { double2 w = U[((size_t)n * 4 + mu) * 9 + k]; u[k] = {w.x, w.y}; }
-  };
-  auto hop = [&](auto mu_tag) {
-    constexpr int MU = decltype(mu_tag)::value;
-    constexpr int SF = DAG ? +1 : -1;
-    cplx<double> p[12], h0[3], h1[3], u[9], w0[3], w1[3];
-    const int f = nbr_fwd(geo, s, c, MU);
-    load_psi(f, p);
-    project<MU, SF>(p, h0, h1);
-    if (MU == 3 && geo.antiperiodic && c[3] == geo.L[3] - 1)
-      for (int k = 0; k < 3; ++k) { h0[k] = -h0[k]; h1[k] = -h1[k]; }
-    load_u(s, MU, u);
-    su3_mul(u, h0, w0);
-    su3_mul(u, h1, w1);
-    accumulate<MU, SF>(acc, w0, w1);
-    const int b = nbr_bwd(geo, s, c, MU);
-    load_psi(b, p);
-    project<MU, -SF>(p, h0, h1);
-    if (MU == 3 && geo.antiperiodic && c[3] == 0)
-      for (int k = 0; k < 3; ++k) { h0[k] = -h0[k]; h1[k] = -h1[k]; }
-    load_u(b, MU, u);
-    su3_dagmul(u, h0, w0);
-    su3_dagmul(u, h1, w1);
-    accumulate<MU, -SF>(acc, w0, w1);
-  };
-  hop(std::integral_constant<int, 0>{});
-  hop(std::integral_constant<int, 1>{});
-  hop(std::integral_constant<int, 2>{});
-  hop(std::integral_constant<int, 3>{});
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    const double2 w = in[(size_t)s * 12 + k];
-    out[(size_t)s * 12 + k] = make_double2(fma(-kappa, acc[k].re, w.x), fma(-kappa, acc[k].im, w.y));
+    for (int k = 0; k < 6; ++k) out[(size_t)s * 12 + fix_comp(half, k)] = make_double2(v[k].re, v[k].im);
+  }
+  if (wout) {
+    ExpRange r;
+    r.spin(v);
+    r.spin(v + 3);
+    r.mx = max(r.mx, __shfl_xor_sync(0xffffffffu, r.mx, 1));
+    r.mn = min(r.mn, __shfl_xor_sync(0xffffffffu, r.mn, 1));
+    r.lo |= __shfl_xor_sync(0xffffffffu, r.lo, 1);
+    if (active && half == 0) wout[s] = r.word();
   }
 }
 
@@ -98,13 +156,14 @@ bool static_device_ptr(const void* p) {
 constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 double2* g_static_addr[kMaxDevices] = {};
+int* g_static_word_addr[kMaxDevices] = {};
 
 // Device address of the scratch array on the current device, looked up once
 // per device (the first call on each device) and kept for the life of the
 // process.  A device reset (cudaDeviceReset, or a reset of the primary
 // context) unloads the module that holds the array, so calls after one are
 // not supported.
-cudaError_t static_scratch_address(double2** out) {
+cudaError_t static_scratch_address(double2** out, int** word) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -114,9 +173,14 @@ cudaError_t static_scratch_address(double2** out) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_static_scratch);
     if (e != cudaSuccess) return e;
+    void* q = nullptr;
+    e = cudaGetSymbolAddress(&q, g_static_word);
+    if (e != cudaSuccess) return e;
     g_static_addr[dev] = static_cast<double2*>(p);
+    g_static_word_addr[dev] = static_cast<int*>(q);
   }
   *out = g_static_addr[dev];
+  *word = g_static_word_addr[dev];
   return cudaSuccess;
 }
 
@@ -161,7 +225,8 @@ extern "C" lq_status lq_apply_MdagM_static(double* out, const double* U, const d
     return LQ_ERR_ARG;
   }
   double2* scratch = nullptr;
-  cudaError_t e = static_scratch_address(&scratch);
+  int* word = nullptr;
+  cudaError_t e = static_scratch_address(&scratch, &word);
   if (e != cudaSuccess) {
     cudaGetLastError();
     lq_set_global_error(std::string("lq_apply_MdagM_static: cudaGetSymbolAddress: ") + cudaGetErrorString(e));
@@ -174,13 +239,22 @@ extern "C" lq_status lq_apply_MdagM_static(double* out, const double* U, const d
   for (int m = 1; m < 4; ++m) geo.stride[m] = geo.stride[m - 1] * dims[m - 1];
   geo.antiperiodic = t_antiperiodic ? 1 : 0;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int bs = 256, grid = grid_for(geo.V, bs);
+  // small lattices in smaller blocks, so that every SM gets one
+  static const int sms = sm_count();
+  int bs = kFixBlock;
+  while (bs > 32 && grid_for(2 * geo.V, bs) < sms) bs >>= 1;
+  const int grid = grid_for(2 * geo.V, bs);
+  const double2 *Uc = reinterpret_cast<const double2*>(U), *ic = reinterpret_cast<const double2*>(in);
+  int *w0 = word, *w1 = word + kStaticMaxSites;
+  static_scan_kernel<<<grid_for(4 * geo.V, 128), 128, 0, st>>>(geo.V, Uc, ic, w0);
   // scratch = M in (every site written before it is read: nothing to clear)
-  hop_canonical_kernel<false><<<grid, bs, 0, st>>>(geo, reinterpret_cast<const double2*>(U),
-                                                   reinterpret_cast<const double2*>(in), scratch, kappa);
+  const bool few = grid_for(2 * geo.V, kFixBlock) <= sms;       // as launch_dslash_fix
+  if (few) hop_canonical_kernel<false, 1><<<grid, bs, 0, st>>>(geo, Uc, ic, w0, w0, scratch, w1, kappa);
+  else hop_canonical_kernel<false, 2><<<grid, bs, 0, st>>>(geo, Uc, ic, w0, w0, scratch, w1, kappa);
   // out = M^dag scratch
-  hop_canonical_kernel<true><<<grid, bs, 0, st>>>(geo, reinterpret_cast<const double2*>(U), scratch,
-                                                  reinterpret_cast<double2*>(out), kappa);
+  double2* oc = reinterpret_cast<double2*>(out);
+  if (few) hop_canonical_kernel<true, 1><<<grid, bs, 0, st>>>(geo, Uc, scratch, w1, w0, oc, nullptr, kappa);
+  else hop_canonical_kernel<true, 2><<<grid, bs, 0, st>>>(geo, Uc, scratch, w1, w0, oc, nullptr, kappa);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     lq_set_global_error(std::string("lq_apply_MdagM_static: launch: ") + cudaGetErrorString(e));

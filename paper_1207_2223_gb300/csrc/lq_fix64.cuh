@@ -31,6 +31,7 @@
 // z, t hops) and the one it hands over at the end ("give": x, y hops).
 #pragma once
 #include <algorithm>
+#include <atomic>
 
 #include "lq_internal.h"
 
@@ -102,23 +103,49 @@ __device__ __forceinline__ void fix_mac(long long& hh, long long& mm, int ah, in
 }
 __device__ __forceinline__ int2 fix_limbs(long long h) { return make_int2((int)(h >> 31), (int)h & 0x7fffffff); }
 
-// One hop of lane `half` (ls = 0 for lane 0, -1 for lane 1) in direction MU with projector
-// sign S: the link U_mu(link) (FWD) or its adjoint times the projected spinor of site n.
-// flip: 0, or -1 when the hop crosses the antiperiodic time boundary.
-template <int MU, int S, bool FWD>
-__device__ __forceinline__ void fix_hop(const double2* psi, int sstride, const int4* U, int V, int n, int link,
-                                        int half, int ls, int flip, unsigned e2, FixAcc& a) {
+// Where the operator reads: [chunk][element] fields with fixed-point links (V: the lattice's
+// volume, sstride: the chunk stride of the spinor field, psi its first element).
+struct SoaAccess {
+  const double2* psi;
+  int sstride;
+  const int4* fix;
+  const double2* f64;
+  int V;
+  // component `comp` of site n and the k-th after it; the link (mu, s) and its element e
+  __device__ __forceinline__ const double2* site(int comp, int n) const { return psi + (size_t)comp * sstride + n; }
+  __device__ __forceinline__ double2 spin(const double2* p, int k) const { return __ldg(p + (size_t)k * sstride); }
+  __device__ __forceinline__ const int4* link(int mu, int s) const { return fix + (size_t)mu * 9 * V + s; }
+  __device__ __forceinline__ int4 element(const int4* p, int e) const { return __ldg(p + (size_t)e * V); }
+  __device__ __forceinline__ double2 element64(int mu, int e, int s) const {
+    return __ldg(f64 + ((size_t)mu * 9 + e) * V + s);
+  }
+};
+
+// The lane's two spins (half and its partner in the projection of direction MU) of site n, as read.
+struct FixRaw {
+  double2 x[3], y[3];
+};
+template <int MU, class Acc>
+__device__ __forceinline__ void fix_load(const Acc& in, int n, int half, FixRaw& r) {
   const int b = (MU <= 1) ? 3 - half : 2 + half;
-  const double2* pa = psi + (size_t)(3 * half) * sstride + n;
-  const double2* pb = psi + (size_t)(3 * b) * sstride + n;
-  // h = pa + sigma q, q = i pb (x, z) or pb (y, t); sigma = S for x, t; -S, S for y; S, -S for z (lanes 0, 1)
-  constexpr int pos = S > 0 ? 0 : -1;
-  const int sg = MU == 1 ? ~(pos ^ ls) : MU == 2 ? pos ^ ls : pos;          // 0: +, -1: -
-  int2 hr[3], hi[3];                                                        // (hi, lo) limbs
+  const double2 *pa = in.site(3 * half, n), *pb = in.site(3 * b, n);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const double2 x = __ldg(pa + (size_t)c * sstride), y = __ldg(pb + (size_t)c * sstride);
-    const FixTerm xr = fix_of(x.x, e2), xi = fix_of(x.y, e2), yr = fix_of(y.x, e2), yi = fix_of(y.y, e2);
+    r.x[c] = in.spin(pa, c);
+    r.y[c] = in.spin(pb, c);
+  }
+}
+
+// Projected spinor of lane `half` (ls = 0 for lane 0, -1 for lane 1) in direction MU with projector
+// sign S as limbs.  flip: 0, or -1 when the hop crosses the antiperiodic time boundary.
+template <int MU, int S>
+__device__ __forceinline__ void fix_half(const FixRaw& r, int ls, int flip, unsigned e2, int2 (&hr)[3], int2 (&hi)[3]) {
+  // h = x + sigma q, q = i y (x, z) or y (y, t); sigma = S for x, t; -S, S for y; S, -S for z (lanes 0, 1)
+  constexpr int pos = S > 0 ? 0 : -1;
+  const int sg = MU == 1 ? ~(pos ^ ls) : MU == 2 ? pos ^ ls : pos;          // 0: +, -1: -
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const FixTerm xr = fix_of(r.x[c].x, e2), xi = fix_of(r.x[c].y, e2), yr = fix_of(r.y[c].x, e2), yi = fix_of(r.y[c].y, e2);
     if constexpr (MU == 0 || MU == 2) {
       hr[c] = fix_limbs(fix_add(xr, flip, yi, flip ^ ~sg));
       hi[c] = fix_limbs(fix_add(xi, flip, yr, flip ^ sg));
@@ -127,13 +154,18 @@ __device__ __forceinline__ void fix_hop(const double2* psi, int sstride, const i
       hi[c] = fix_limbs(fix_add(xi, flip, yi, flip ^ sg));
     }
   }
-  const int4* u0 = U + (size_t)MU * 9 * V + link;
+}
+
+// U h (FWD) or U^dag h added to the lane's sums; link(e): element e of the link as limbs.
+template <int MU, int S, bool FWD, class Link>
+__device__ __forceinline__ void fix_rows(const Link& link, const int2 (&hr)[3], const int2 (&hi)[3], int ls, FixAcc& a) {
+  constexpr int pos = S > 0 ? 0 : -1;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     long long rh = 0, rm = 1 << 30, ih = 0, im = 1 << 30;                   // middle column rounded to nearest
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const int4 u = __ldg(u0 + (size_t)(FWD ? 3 * i + j : 3 * j + i) * V);
+      const int4 u = link(FWD ? 3 * i + j : 3 * j + i);
       fix_mac(rh, rm, u.x, u.y, hr[j]);
       fix_mac(ih, im, u.x, u.y, hi[j]);
       fix_mac(rh, rm, FWD ? -u.z : u.z, FWD ? -u.w : u.w, hi[j]);
@@ -161,6 +193,18 @@ __device__ __forceinline__ void fix_hop(const double2* psi, int sstride, const i
   }
 }
 
+// One hop: the link U_mu(link) (FWD) or its adjoint times the projected spinor of site n.
+template <int MU, int S, bool FWD, class Acc>
+__device__ __forceinline__ void fix_hop(const Acc& in, int n, int link, int half, int ls, int flip, unsigned e2,
+                                        FixAcc& a) {
+  FixRaw r;
+  fix_load<MU>(in, n, half, r);
+  int2 hr[3], hi[3];
+  fix_half<MU, S>(r, ls, flip, e2, hr, hi);
+  const auto u0 = in.link(MU, link);
+  fix_rows<MU, S, FWD>([&](int e) { return in.element(u0, e); }, hr, hi, ls, a);
+}
+
 // Start of a site's sums: zero, plus one for each sum that gets one complemented term (each
 // lane: one of the two y hops, one of the two z hops).
 __device__ __forceinline__ void fix_clear(FixAcc& a) {
@@ -174,15 +218,14 @@ __device__ __forceinline__ void fix_clear(FixAcc& a) {
 }
 
 // ------------------------------------------------------------ the FP64 path of a site
-template <int MU, int S, bool FWD>
-__device__ __forceinline__ void split_hop64(const double2* psi, int sstride, const double2* U, int V, int n, int link,
-                                            int half, bool flip, double (&up)[3][2], double (&give)[3][2],
+template <int MU, int S, bool FWD, class Acc>
+__device__ __forceinline__ void split_hop64(const Acc& in, int n, int link, int half, bool flip, double (&up)[3][2], double (&give)[3][2],
                                             double (&keep)[3][2]) {
   const int b = (MU <= 1) ? 3 - half : 2 + half;
   cplx<double> h[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const double2 x = __ldg(psi + (size_t)(3 * half + c) * sstride + n), y = __ldg(psi + (size_t)(3 * b + c) * sstride + n);
+    const double2 x = in.spin(in.site(3 * half, n), c), y = in.spin(in.site(3 * b, n), c);
     const cplx<double> p{x.x, x.y}, q{y.x, y.y};
     cplx<double> t;
     if constexpr (MU == 0) t = times_i(q);
@@ -192,13 +235,12 @@ __device__ __forceinline__ void split_hop64(const double2* psi, int sstride, con
     h[c] = (S > 0) ? p + t : p - t;
     if (flip) h[c] = -h[c];
   }
-  const double2* u0 = U + (size_t)MU * 9 * V + link;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     cplx<double> w{0.0, 0.0};
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const double2 e = __ldg(u0 + (size_t)(FWD ? 3 * i + j : 3 * j + i) * V);
+      const double2 e = in.element64(MU, FWD ? 3 * i + j : 3 * j + i, link);
       w = FWD ? cmadd(w, cplx<double>{e.x, e.y}, h[j]) : cjmadd(w, cplx<double>{e.x, e.y}, h[j]);
     }
     up[i][0] += w.re;
@@ -212,24 +254,23 @@ __device__ __forceinline__ void split_hop64(const double2* psi, int sstride, con
 }
 
 // The lane's sums of site s in FP64 arithmetic, as bit patterns (out: up, give, keep).
-template <bool DAG>
-__device__ __noinline__ void split_site64(Geom geo, const double2* psi, int sstride, const double2* U, int s, int half,
-                                          FixAcc* out) {
+template <bool DAG, class Acc>
+__device__ __noinline__ void split_site64(Geom geo, Acc in, int s, int half, FixAcc* out) {
   constexpr int SF = DAG ? +1 : -1;
   int c[4];
   site_coords(geo, s, c);
   double up[3][2] = {}, give[3][2] = {}, keep[3][2] = {};
   int n;
-  n = nbr_fwd(geo, s, c, 0); split_hop64<0, SF, true>(psi, sstride, U, geo.V, n, s, half, false, up, give, keep);
-  n = nbr_bwd(geo, s, c, 0); split_hop64<0, -SF, false>(psi, sstride, U, geo.V, n, n, half, false, up, give, keep);
-  n = nbr_fwd(geo, s, c, 1); split_hop64<1, SF, true>(psi, sstride, U, geo.V, n, s, half, false, up, give, keep);
-  n = nbr_bwd(geo, s, c, 1); split_hop64<1, -SF, false>(psi, sstride, U, geo.V, n, n, half, false, up, give, keep);
-  n = nbr_fwd(geo, s, c, 2); split_hop64<2, SF, true>(psi, sstride, U, geo.V, n, s, half, false, up, give, keep);
-  n = nbr_bwd(geo, s, c, 2); split_hop64<2, -SF, false>(psi, sstride, U, geo.V, n, n, half, false, up, give, keep);
+  n = nbr_fwd(geo, s, c, 0); split_hop64<0, SF, true>(in, n, s, half, false, up, give, keep);
+  n = nbr_bwd(geo, s, c, 0); split_hop64<0, -SF, false>(in, n, n, half, false, up, give, keep);
+  n = nbr_fwd(geo, s, c, 1); split_hop64<1, SF, true>(in, n, s, half, false, up, give, keep);
+  n = nbr_bwd(geo, s, c, 1); split_hop64<1, -SF, false>(in, n, n, half, false, up, give, keep);
+  n = nbr_fwd(geo, s, c, 2); split_hop64<2, SF, true>(in, n, s, half, false, up, give, keep);
+  n = nbr_bwd(geo, s, c, 2); split_hop64<2, -SF, false>(in, n, n, half, false, up, give, keep);
   n = nbr_fwd(geo, s, c, 3);
-  split_hop64<3, SF, true>(psi, sstride, U, geo.V, n, s, half, geo.antiperiodic && c[3] == geo.L[3] - 1, up, give, keep);
+  split_hop64<3, SF, true>(in, n, s, half, geo.antiperiodic && c[3] == geo.L[3] - 1, up, give, keep);
   n = nbr_bwd(geo, s, c, 3);
-  split_hop64<3, -SF, false>(psi, sstride, U, geo.V, n, n, half, geo.antiperiodic && c[3] == 0, up, give, keep);
+  split_hop64<3, -SF, false>(in, n, n, half, geo.antiperiodic && c[3] == 0, up, give, keep);
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -244,19 +285,132 @@ __device__ __noinline__ void split_site64(Geom geo, const double2* psi, int sstr
 // Component of element k of a lane's six (spin half, then spin half + 2, colour fastest).
 __device__ __forceinline__ int fix_comp(int half, int k) { return k < 3 ? 3 * half + k : 3 * (half + 2) + (k - 3); }
 
+// The eight hops of site s (coordinates c, neighbours f, b) with common exponent E.
+template <bool DAG, class Acc>
+__device__ __forceinline__ void fix_hops(const Geom& geo, const Acc& in, int s, const int c[4], const int f[4],
+                                         const int b[4], int half, int E, FixAcc& a) {
+  constexpr int SF = DAG ? +1 : -1;
+  const int ls = -half;
+  const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
+  const int ff = (geo.antiperiodic && c[3] == geo.L[3] - 1) ? -1 : 0, fb = (geo.antiperiodic && c[3] == 0) ? -1 : 0;
+  fix_hop<0, SF, true>(in, f[0], s, half, ls, 0, e2, a);
+  fix_hop<0, -SF, false>(in, b[0], b[0], half, ls, 0, e2, a);
+  fix_hop<1, SF, true>(in, f[1], s, half, ls, 0, e2, a);
+  fix_hop<1, -SF, false>(in, b[1], b[1], half, ls, 0, e2, a);
+  fix_hop<2, SF, true>(in, f[2], s, half, ls, 0, e2, a);
+  fix_hop<2, -SF, false>(in, b[2], b[2], half, ls, 0, e2, a);
+  fix_hop<3, SF, true>(in, f[3], s, half, ls, ff, e2, a);
+  fix_hop<3, -SF, false>(in, b[3], b[3], half, ls, fb, e2, a);
+}
+
+// The same with the operands of the next hop copied to shared memory (cp.async) while a hop
+// computes: the stencil is bound by the latency of its loads at the 16 warps per SM its registers
+// allow, and the copies need none.  Per stage a block holds 21 rows of 16 bytes per site: the 9 link
+// elements (copied by both lanes of a pair, 5 and 4), then each lane's 6 spinor components; two
+// stages.  `stage` points at the pair's column of stage 0.
+constexpr int kFixRows = 21;
+constexpr size_t kFixSmem = (size_t)2 * kFixRows * (kFixBlock / 2) * sizeof(int4);
+
+__device__ __forceinline__ void fix_copy16(int4* smem, const void* gmem) {
+  const unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem) : "memory");
+}
+template <int H>
+__device__ __forceinline__ void fix_issue(const SoaAccess& in, const int f[4], const int b[4], int s, int half,
+                                          int4* stage) {
+  constexpr int MU = H >> 1;
+  constexpr bool FWD = (H & 1) == 0;
+  constexpr int P = kFixBlock / 2;
+  const int n = FWD ? f[MU] : b[MU];
+  int4* st = stage + (H & 1) * (kFixRows * P);
+  const int4* u = in.link(MU, FWD ? s : n) + (size_t)(5 * half) * in.V;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) fix_copy16(st + (5 * half + e) * P, u + (size_t)e * in.V);
+  if (half == 0) fix_copy16(st + 4 * P, u + (size_t)4 * in.V);
+  const int q = (MU <= 1) ? 3 - half : 2 + half;
+  const double2 *pa = in.site(3 * half, n), *pb = in.site(3 * q, n);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    fix_copy16(st + (9 + 6 * half + c) * P, pa + (size_t)c * in.sstride);
+    fix_copy16(st + (12 + 6 * half + c) * P, pb + (size_t)c * in.sstride);
+  }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+template <int H, bool DAG>
+__device__ __forceinline__ void fix_step(const SoaAccess& in, const int f[4], const int b[4], int s, int half, int flip,
+                                         unsigned e2, int4* stage, FixAcc& a) {
+  constexpr int MU = H >> 1, P = kFixBlock / 2;
+  constexpr bool FWD = (H & 1) == 0;
+  constexpr int S = (DAG ? +1 : -1) * (FWD ? 1 : -1);
+  if constexpr (H < 7) {
+    fix_issue<H + 1>(in, f, b, s, half, stage);
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+  } else {
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  }
+  __syncwarp();                                       // the partner's copies of the link
+  const int4* st = stage + (H & 1) * (kFixRows * P);
+  FixRaw r;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    r.x[c] = *reinterpret_cast<const double2*>(st + (9 + 6 * half + c) * P);
+    r.y[c] = *reinterpret_cast<const double2*>(st + (12 + 6 * half + c) * P);
+  }
+  int2 hr[3], hi[3];
+  fix_half<MU, S>(r, -half, flip, e2, hr, hi);
+  fix_rows<MU, S, FWD>([&](int e) { return st[e * P]; }, hr, hi, -half, a);
+  __syncwarp();                                       // the stage may be refilled
+}
+template <bool DAG>
+__device__ __forceinline__ void fix_hops_async(const Geom& geo, const SoaAccess& in, int s, const int c[4],
+                                               const int f[4], const int b[4], int half, int E, int4* stage, FixAcc& a) {
+  const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
+  const int ff = (geo.antiperiodic && c[3] == geo.L[3] - 1) ? -1 : 0, fb = (geo.antiperiodic && c[3] == 0) ? -1 : 0;
+  fix_step<0, DAG>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<1, DAG>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<2, DAG>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<3, DAG>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<4, DAG>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<5, DAG>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<6, DAG>(in, f, b, s, half, ff, e2, stage, a);
+  fix_step<7, DAG>(in, f, b, s, half, fb, e2, stage, a);
+}
+
+// The lane's two spins of M psi at site s: centre + ks * hopping sums.  Each lane completes the
+// lower spin it keeps with the partner's sums (both lanes of a pair took the same path; every lane
+// of the warp calls).  slow: the sums are FP64 bit patterns.
+template <class Acc>
+__device__ __forceinline__ void fix_finish(const Acc& in, const FixAcc& a, int s, int half, bool slow, double ks,
+                                           cplx<double> v[6]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double2 c0 = in.spin(in.site(3 * half, s), i), c1 = in.spin(in.site(3 * (half + 2), s), i);
+    double lo[2], hi[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const long long got = __shfl_xor_sync(0xffffffffu, a.give[i][q], 1);
+      hi[q] = slow ? __longlong_as_double(a.up[i][q]) : (double)a.up[i][q];
+      lo[q] = slow ? __longlong_as_double(a.keep[i][q]) + __longlong_as_double(got) : (double)(a.keep[i][q] + got);
+    }
+    v[i] = {fma(ks, hi[0], c0.x), fma(ks, hi[1], c0.y)};
+    v[3 + i] = {fma(ks, lo[0], c1.x), fma(ks, lo[1], c1.y)};
+  }
+}
+
 // Applies M (or M^dag) at the sites of pair `first`, first + stride, ... of one lattice.
 // Spinor fields are [chunk][element] with chunk stride `sstride` (V for a single lattice, the
 // batch's element count for one column of a batch) and the lattice's sites at elements
 // off .. off + V - 1; `in.norm` holds the sites' exponent words.  The epilogue gets the
 // element index.
-template <bool DAG, class Epi>
+template <bool DAG, bool ASYNC, class Epi>
 __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, const SpinorRef& in, int sstride, int off,
                                           double kappa, const Epi& epi, int first, int stride, double (&red)[1]) {
-  constexpr int SF = DAG ? +1 : -1;
-  const double2* psi = static_cast<const double2*>(in.p) + off;
+  const SoaAccess acc{static_cast<const double2*>(in.p) + off, sstride, U.fix, U.f64, geo.V};
   const int* word = reinterpret_cast<const int*>(in.norm) + off;
   const bool bad = __ldg(U.bad) != 0;
-  const int half = threadIdx.x & 1, ls = -half;
+  const int half = threadIdx.x & 1;
+  extern __shared__ int4 fix_smem[];
+  int4* stage = fix_smem + (threadIdx.x >> 1);
   const int Vr = (geo.V + 15) & ~15;                     // whole warps iterate together
   for (int s0 = first; s0 < Vr; s0 += stride) {
     const bool active = s0 < geo.V;
@@ -268,58 +422,37 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
     for (int m = 0; m < 4; ++m) {
       f[m] = nbr_fwd(geo, s, c, m);
       b[m] = nbr_bwd(geo, s, c, m);
+    }
+    if constexpr (ASYNC) fix_issue<0>(acc, f, b, s, half, stage);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
       const int wf = __ldg(word + f[m]), wb = __ldg(word + b[m]);
       any |= wf | wb;
       E = max(E, max(wf & 0x7ff, wb & 0x7ff));
     }
     const bool slow = bad || (any & kFixSlow);
     FixAcc a;
-    if (!slow) {
-      const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
-      const int ff = (geo.antiperiodic && c[3] == geo.L[3] - 1) ? -1 : 0, fb = (geo.antiperiodic && c[3] == 0) ? -1 : 0;
-      fix_clear(a);
-      fix_hop<0, SF, true>(psi, sstride, U.fix, geo.V, f[0], s, half, ls, 0, e2, a);
-      fix_hop<0, -SF, false>(psi, sstride, U.fix, geo.V, b[0], b[0], half, ls, 0, e2, a);
-      fix_hop<1, SF, true>(psi, sstride, U.fix, geo.V, f[1], s, half, ls, 0, e2, a);
-      fix_hop<1, -SF, false>(psi, sstride, U.fix, geo.V, b[1], b[1], half, ls, 0, e2, a);
-      fix_hop<2, SF, true>(psi, sstride, U.fix, geo.V, f[2], s, half, ls, 0, e2, a);
-      fix_hop<2, -SF, false>(psi, sstride, U.fix, geo.V, b[2], b[2], half, ls, 0, e2, a);
-      fix_hop<3, SF, true>(psi, sstride, U.fix, geo.V, f[3], s, half, ls, ff, e2, a);
-      fix_hop<3, -SF, false>(psi, sstride, U.fix, geo.V, b[3], b[3], half, ls, fb, e2, a);
-    } else {
+    fix_clear(a);
+    if constexpr (ASYNC) fix_hops_async<DAG>(geo, acc, s, c, f, b, half, E, stage, a);   // every lane: warp barriers
+    else if (!slow) fix_hops<DAG>(geo, acc, s, c, f, b, half, E, a);
+    if (slow) {
       FixAcc t64;
-      split_site64<DAG>(geo, psi, sstride, U.f64, s, half, &t64);
+      split_site64<DAG>(geo, acc, s, half, &t64);
       a = t64;
     }
-    // each lane completes the lower spin it keeps with the partner's sums (both lanes of a
-    // pair took the same path)
     cplx<double> v[6];
-    const double ks = slow ? -kappa : -kappa * __hiloint2double((E - 56) << 20, 0);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const double2 c0 = __ldg(psi + (size_t)fix_comp(half, i) * sstride + s);
-      const double2 c1 = __ldg(psi + (size_t)fix_comp(half, 3 + i) * sstride + s);
-      double lo[2], hi[2];
-#pragma unroll
-      for (int q2 = 0; q2 < 2; ++q2) {
-        const long long got = __shfl_xor_sync(0xffffffffu, a.give[i][q2], 1);
-        hi[q2] = slow ? __longlong_as_double(a.up[i][q2]) : (double)a.up[i][q2];
-        lo[q2] = slow ? __longlong_as_double(a.keep[i][q2]) + __longlong_as_double(got) : (double)(a.keep[i][q2] + got);
-      }
-      v[i] = {fma(ks, hi[0], c0.x), fma(ks, hi[1], c0.y)};
-      v[3 + i] = {fma(ks, lo[0], c1.x), fma(ks, lo[1], c1.y)};
-    }
+    fix_finish(acc, a, s, half, slow, slow ? -kappa : -kappa * __hiloint2double((E - 56) << 20, 0), v);
     epi.apply(sstride, off + s, half, active, v, red);
   }
 }
 
-// MINB: resident blocks per SM asked for (register cap).
+// MINB: resident blocks per SM asked for (register cap); 2: with operands copied ahead.
 template <bool DAG, class Epi, int MINB>
 __global__ void __launch_bounds__(kFixBlock, MINB)
     dslash_fix_kernel(Geom geo, FixGauge U, SpinorRef in, double kappa, Epi epi, ReduceScratch rs) {
   if (epi.halted()) return;
   double red[1] = {0.0};
-  fix_sites<DAG, Epi>(geo, U, in, geo.V, 0, kappa, epi, (blockIdx.x * blockDim.x + threadIdx.x) >> 1,
+  fix_sites<DAG, MINB == 2, Epi>(geo, U, in, geo.V, 0, kappa, epi, (blockIdx.x * blockDim.x + threadIdx.x) >> 1,
                       (gridDim.x * blockDim.x) >> 1, red);
   if constexpr (Epi::REDUCE) {
     double tot[1];
@@ -442,14 +575,34 @@ struct FixEpiResidual {
   __device__ void finalize(double (&tot)[1]) const { fin(tot[0]); }
 };
 
-// Blocks of 256
-// threads (128 sites), two per SM; measured slower: 64-site blocks at the same occupancy (286
+// Opts a kernel in to the shared memory of the copying stencil, once per device; its resident
+// blocks there.  `cache`: one slot per device, kept with the kernel's launcher.
+constexpr int kFixDevices = 64;
+inline int fix_wave(const void* kernel, std::atomic<int> (&cache)[kFixDevices]) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::atomic<int>& slot = cache[dev & (kFixDevices - 1)];
+  int wave = slot.load(std::memory_order_acquire);
+  if (wave == 0) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kFixBlock, kFixSmem);
+    wave = sm_count() * std::max(1, per_sm);
+    slot.store(wave, std::memory_order_release);
+  }
+  return wave;
+}
+
+// Blocks of 256 threads (128 sites), two per SM; measured slower: 64-site blocks at the same occupancy (286
 // against 241 us at 24^3 x 32: fewer of the x and y neighbours are in the block's own lines),
 // three blocks of 80 registers (344, spills), blocks of 4 x 4 x 4 x 2 sites (304: shorter runs per
-// load).  A lattice that leaves SMs without a block takes smaller blocks, and without the register
+// load).  Operands copied ahead (fix_hops_async): 254 instead of 300 us for CG pass 1 there, 290 instead of
+// 342 for pass 2, M^dag M at 32^3 x 64 2.68 instead of 3.6 ms.  A lattice that leaves SMs without a block takes smaller blocks, and without the register
 // cap (its warps are alone on their schedulers: 8^4 14.4 -> 10.3 us).
+// Internal linkage: every translation unit launches its own instance of the kernel and has to opt
+// that instance in (a count cached across units would leave the others at the default shared memory).
 template <bool DAG, class Epi>
-inline void launch_dslash_fix(const Geom& geo, const FixGauge& U, SpinorRef in, double kappa, const Epi& epi,
+static void launch_dslash_fix(const Geom& geo, const FixGauge& U, SpinorRef in, double kappa, const Epi& epi,
                               const ReduceScratch& rs, cudaStream_t stream) {
   static const int sms = sm_count();
   const int blocks = grid_for(2 * geo.V, kFixBlock);
@@ -459,8 +612,9 @@ inline void launch_dslash_fix(const Geom& geo, const FixGauge& U, SpinorRef in, 
     dslash_fix_kernel<DAG, Epi, 1><<<grid_for(2 * geo.V, bs), bs, 0, stream>>>(geo, U, in, kappa, epi, rs);
     return;
   }
-  static const int wave = resident_grid(reinterpret_cast<const void*>(&dslash_fix_kernel<DAG, Epi, 2>), kFixBlock);
-  dslash_fix_kernel<DAG, Epi, 2><<<std::min(blocks, wave), kFixBlock, 0, stream>>>(geo, U, in, kappa, epi, rs);
+  static std::atomic<int> waves[kFixDevices];
+  const int wave = fix_wave(reinterpret_cast<const void*>(&dslash_fix_kernel<DAG, Epi, 2>), waves);
+  dslash_fix_kernel<DAG, Epi, 2><<<std::min(blocks, wave), kFixBlock, kFixSmem, stream>>>(geo, U, in, kappa, epi, rs);
 }
 
 }  // namespace lq

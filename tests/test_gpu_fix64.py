@@ -169,3 +169,26 @@ def test_fermion_force(lq, dims, kind):
         fwd = lambda a: np.maximum(a, np.roll(a, -1, 3 - mu))   # noqa: E731
         tol = 2.0 ** -53 * 64 * 24 * 0.3 * u * (fwd(ax) * fwd(ny)).reshape(V, 1)
         assert np.all(np.abs(F[:, mu] - ref[:, mu]) <= tol), mu
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7), (16, 12, 12, 18)])
+@pytest.mark.parametrize("kind", ["gauss", "site_range", "spin_range", "point", "ones", "not_unitary", "one_bad_link"])
+def test_static_mdagm(lq, dims, kind):
+    """M^dag M on canonical buffers against the oracle; one bad link sends only the sites that read
+    it to FP64 arithmetic.  Bound per element: as above for both applications, 64 units of 2^-53 of
+    the largest component within two steps, times (1 + 8 * 0.15 * 3 max |U|)^2."""
+    U, psi = _fields(dims, "gauss" if kind == "one_bad_link" else kind)
+    lat = Lattice(dims)
+    if kind == "one_bad_link":
+        U[lat.V // 3, 2] *= 3.0
+    out = torch.empty(psi.shape, dtype=torch.complex128, device="cuda")
+    lq.lq_apply_MdagM_static(out, dev(U), dev(psi), dims, 0.15)
+    ref = apply_M(U, apply_M(U, psi, dims, 0.15), dims, 0.15, True, True)
+    near = np.abs(psi).max(axis=(1, 2)).reshape(dims[::-1])
+    for _ in range(2):
+        a = near
+        for ax in range(4):
+            near = np.maximum(near, np.maximum(np.roll(a, 1, ax), np.roll(a, -1, ax)))
+    grow = 1 + 8 * 0.15 * 3 * max(1.0, np.abs(U).max())
+    tol = 64 * 2.0 ** -53 * grow ** 2 * near.reshape(lat.V, 1, 1)
+    assert np.all(np.abs(host(out) - ref) <= tol)
