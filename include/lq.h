@@ -120,6 +120,8 @@ lq_status lq_set_stream(lq_ctx* ctx, void* cuda_stream);
  *                       replayed; 0: every kernel is launched from the host (to measure
  *                       the launch overhead the graphs remove; paper Sec. 4, Fig. 1 reads
  *                       a per-call overhead off CG time against iteration count).
+ *                       Mixed-precision solves of up to 6144 sites run the iterations
+ *                       between two reliable updates as one launch either way.
  *   LQ_OPT_DF64_UPDATES accepted (0 or 1) and without effect: every reliable update of a
  *                       mixed-precision solve recomputes the residual with the FP64 operator,
  *                       which on this part is faster than the double-float one (0.7 against

@@ -168,6 +168,10 @@ lq_status ensure_solver_fields(lq_ctx* c, int inner) {
 // precision, length and kappa); the kernels return at once after the
 // device-side halt flag is raised.
 lq_status run_chunk(lq_ctx* c, int inner, int n, double kappa) {
+  if (cluster_takes(c, inner)) {
+    LQ_CUDA(c, cg_cluster_iterations(c, inner, n, kappa, c->stream));
+    return LQ_OK;
+  }
   if (!c->use_graphs) {
     for (int i = 0; i < n; ++i) {
       if (inner == LQ_F64) cg64_iteration(c, kappa, c->stream);
@@ -259,7 +263,7 @@ lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int i
     int stagnant = 0;
     for (long guard = 0; guard < (long)maxiter + 64; ++guard) {
       LQ_TRY(run_chunk(c, inner, chunk, kappa));
-      s.kernel_launches += 3 * chunk;
+      s.kernel_launches += cluster_takes(c, inner) ? 1 : 3 * chunk;
       LQ_TRY(read_state(c));
       const SolverState& st = *c->state_host;
       if (st.breakdown) { result = fail(c, LQ_ERR_NAN, "CG breakdown (non-positive or non-finite curvature)"); break; }

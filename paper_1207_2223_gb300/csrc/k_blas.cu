@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(kBS) solver_init_kernel(int V, SpinorRef phi64
 template <SStore S>
 __global__ void __launch_bounds__(kBS) xpay_p_kernel(int V, SpinorRef r, SpinorRef p, const SolverState* st,
                                                      int forced) {
+  pdl_wait();
   if (!forced && *(volatile const int*)&st->halt) return;
   // one site per thread: a grid-stride loop over one resident wave would make
   // the empty launches after a halt cheaper, but measured slower (91% against
@@ -124,7 +125,7 @@ void launch_solver_init(const Geom& g, SpinorRef phi64, SStore sx, SpinorRef x, 
 void launch_xpay_p(const Geom& g, SStore s, SpinorRef r, SpinorRef p, SolverState* st, bool forced,
                    cudaStream_t stream) {
   const int grid = grid_for(g.V, kBS);
-  LQ_DISPATCH_S(s, (xpay_p_kernel<SS><<<grid, kBS, 0, stream>>>(g.V, r, p, st, forced ? 1 : 0)));
+  LQ_DISPATCH_S(s, (launch_pdl(&xpay_p_kernel<SS>, grid, kBS, 0, stream, g.V, r, p, st, forced ? 1 : 0)));
 }
 
 void launch_accumulate_x(const Geom& g, SStore slo, SpinorRef xlo, SpinorRef xhi, cudaStream_t stream) {

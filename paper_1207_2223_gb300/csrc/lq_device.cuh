@@ -517,6 +517,14 @@ __device__ __forceinline__ void su3_dagmul(const cplx<T> u[9], const cplx<T> h[3
   }
 }
 
+// --------------------------------------------------- programmatic dependent launch
+// Kernels of a CG iteration are launched so that the next one may be set up while its predecessor
+// finishes (launch_pdl): each waits, before it touches anything the predecessor wrote, until that
+// one has completed.  Every kernel of the chain waits, also one that then returns at once, so
+// completion stays in order along the whole chain.  No kernel asks for its successor earlier:
+// waiting blocks then take the places of blocks still to run (12^4: 20 -> 26 us per iteration).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // --------------------------------------------------- grid reductions
 // Every reducing kernel adds up to NRED doubles per thread.  Each block
 // reduces them (warp shuffles, then shared memory) and writes one partial

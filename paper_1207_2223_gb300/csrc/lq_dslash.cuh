@@ -63,7 +63,7 @@ struct SingleIndex {
 // contribution and sets acc (the first direction of the stencil).  The antiperiodic
 // sign of a hop across the time boundary is folded into the norm scale of 16-bit
 // storage, which is multiplied anyway; for the other formats it flips sign bits.
-template <int MU, bool DAG, GStore G, SStore SI, typename T, class IX = SingleIndex, bool INIT = false>
+template <int MU, bool DAG, GStore G, SStore SI, typename T, class IX = SingleIndex, bool INIT = false, int LD = 1>
 __device__ __forceinline__ void hop_dir(const Geom& geo, const GaugeRef& U, const SpinorRef& in, int s,
                                         const int c[4], cplx<T> acc[12], IX ix = IX{0}) {
   if constexpr (std::is_same<IX, SingleIndex>::value) ix.V = geo.V;
@@ -72,7 +72,7 @@ __device__ __forceinline__ void hop_dir(const Geom& geo, const GaugeRef& U, cons
   {
     const int n = nbr_fwd(geo, s, c, MU);
     cplx<T> p[12];
-    T sc = load_spinor_raw<SI, T>(in, ix.stride(), ix(n), p);
+    T sc = load_spinor_raw<SI, T, LD>(in, ix.stride(), ix(n), p);
     cplx<T> h0[3], h1[3];
     project<MU, SF>(p, h0, h1);
     const bool flip = MU == 3 && geo.antiperiodic && c[3] == geo.L[3] - 1;
@@ -96,7 +96,7 @@ __device__ __forceinline__ void hop_dir(const Geom& geo, const GaugeRef& U, cons
   {
     const int n = nbr_bwd(geo, s, c, MU);
     cplx<T> p[12];
-    T sc = load_spinor_raw<SI, T>(in, ix.stride(), ix(n), p);
+    T sc = load_spinor_raw<SI, T, LD>(in, ix.stride(), ix(n), p);
     cplx<T> h0[3], h1[3];
     project<MU, -SF>(p, h0, h1);
     const bool flip = MU == 3 && geo.antiperiodic && c[3] == 0;
@@ -148,12 +148,29 @@ __device__ __forceinline__ double site_norm2(const cplx<T> v[12]) {
   return (double)a;
 }
 
+// Launch of a kernel that begins with pdl_wait().
+template <class... KArgs, class... Args>
+inline void launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t stream, Args&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // Grid-stride: the grid is one wave of resident blocks and every thread
 // walks the lattice in steps of the grid size, so the halt check and the
 // block reduction happen once per block rather than once per 256 sites.
 template <typename T, GStore G, SStore SI, bool DAG, class Epi>
 __global__ void __launch_bounds__(DslashBlock<T>::value, (EpiMinBlocks<T, Epi>::value)) dslash_kernel(Geom geo, GaugeRef U, SpinorRef in,
                                                                         T kappa, Epi epi, ReduceScratch rs) {
+  pdl_wait();
   if (epi.halted()) return;
   double red[Epi::NRED];
 #pragma unroll
@@ -330,11 +347,11 @@ inline void launch_dslash(const Geom& geo, GaugeRef U, SpinorRef in, double kapp
   if (2 * grid_for(geo.V, bs) <= wave) {
     static const int wave_half = resident_grid(kern, bs / 2);
     const int grid = std::min(grid_for(geo.V, bs / 2), wave_half);
-    dslash_kernel<T, G, SI, DAG, Epi><<<grid, bs / 2, 0, stream>>>(geo, U, in, (T)kappa, epi, rs);
+    launch_pdl(&dslash_kernel<T, G, SI, DAG, Epi>, grid, bs / 2, 0, stream, geo, U, in, (T)kappa, epi, rs);
     return;
   }
   const int grid = std::min(grid_for(geo.V, bs), wave);
-  dslash_kernel<T, G, SI, DAG, Epi><<<grid, bs, 0, stream>>>(geo, U, in, (T)kappa, epi, rs);
+  launch_pdl(&dslash_kernel<T, G, SI, DAG, Epi>, grid, bs, 0, stream, geo, U, in, (T)kappa, epi, rs);
 }
 
 }  // namespace lq

@@ -446,13 +446,13 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
   }
 }
 
-// MINB: resident blocks per SM asked for (register cap); 2: with operands copied ahead.
-template <bool DAG, class Epi, int MINB>
-__global__ void __launch_bounds__(kFixBlock, MINB)
+template <bool DAG, class Epi>
+__global__ void __launch_bounds__(kFixBlock, 2)
     dslash_fix_kernel(Geom geo, FixGauge U, SpinorRef in, double kappa, Epi epi, ReduceScratch rs) {
+  pdl_wait();
   if (epi.halted()) return;
   double red[1] = {0.0};
-  fix_sites<DAG, MINB == 2, Epi>(geo, U, in, geo.V, 0, kappa, epi, (blockIdx.x * blockDim.x + threadIdx.x) >> 1,
+  fix_sites<DAG, true, Epi>(geo, U, in, geo.V, 0, kappa, epi, (blockIdx.x * blockDim.x + threadIdx.x) >> 1,
                       (gridDim.x * blockDim.x) >> 1, red);
   if constexpr (Epi::REDUCE) {
     double tot[1];
@@ -575,6 +575,93 @@ struct FixEpiResidual {
   __device__ void finalize(double (&tot)[1]) const { fin(tot[0]); }
 };
 
+// Small lattices, split by direction like dslash_dir_kernel: four warps share 16 sites (32 lanes), the
+// first adds the integer sums (in any order the same) and finishes the sites.  FP64 CG, us per
+// iteration, split against two threads per site: 4^4 24 / 41, 8^4 31 / 41, 8^3 x 16 34 / 40, 10^4 45 / 41.
+constexpr int kFixDirSites = 8192;
+template <bool DAG, class Epi>
+__global__ void __launch_bounds__(128, 4)
+    dslash_fix_dir_kernel(Geom geo, FixGauge U, SpinorRef in, double kappa, Epi epi, ReduceScratch rs) {
+  __shared__ long long part[3][12][32];
+  pdl_wait();
+  if (epi.halted()) return;
+  constexpr int SF = DAG ? +1 : -1;
+  const SoaAccess acc{static_cast<const double2*>(in.p), geo.V, U.fix, U.f64, geo.V};
+  const int* word = reinterpret_cast<const int*>(in.norm);
+  const bool bad = __ldg(U.bad) != 0;
+  const int lane = threadIdx.x & 31, dir = threadIdx.x >> 5, half = lane & 1, ls = -half;
+  double red[1] = {0.0};
+  for (int base = blockIdx.x * 16; base < geo.V; base += gridDim.x * 16) {
+    const bool active = base + (lane >> 1) < geo.V;
+    const int s = active ? base + (lane >> 1) : 0;
+    int c[4];
+    site_coords(geo, s, c);
+    int f[4], b[4], E = kFixMinExp, any = 0;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      f[m] = nbr_fwd(geo, s, c, m);
+      b[m] = nbr_bwd(geo, s, c, m);
+      const int wf = __ldg(word + f[m]), wb = __ldg(word + b[m]);
+      any |= wf | wb;
+      E = max(E, max(wf & 0x7ff, wb & 0x7ff));
+    }
+    const bool slow = bad || (any & kFixSlow);
+    const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
+    FixAcc a;
+    fix_clear(a);
+    if (dir == 0) {
+      fix_hop<0, SF, true>(acc, f[0], s, half, ls, 0, e2, a);
+      fix_hop<0, -SF, false>(acc, b[0], b[0], half, ls, 0, e2, a);
+    } else if (dir == 1) {
+      fix_hop<1, SF, true>(acc, f[1], s, half, ls, 0, e2, a);
+      fix_hop<1, -SF, false>(acc, b[1], b[1], half, ls, 0, e2, a);
+    } else if (dir == 2) {
+      fix_hop<2, SF, true>(acc, f[2], s, half, ls, 0, e2, a);
+      fix_hop<2, -SF, false>(acc, b[2], b[2], half, ls, 0, e2, a);
+    } else {
+      const int ff = (geo.antiperiodic && c[3] == geo.L[3] - 1) ? -1 : 0, fb = (geo.antiperiodic && c[3] == 0) ? -1 : 0;
+      fix_hop<3, SF, true>(acc, f[3], s, half, ls, ff, e2, a);
+      fix_hop<3, -SF, false>(acc, b[3], b[3], half, ls, fb, e2, a);
+    }
+    // x, y add to "give", z, t to "keep"; the start values of fix_clear (give 1; keep -1, 1) are
+    // counted once each, here in the warps of y and z
+    if (dir > 0) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          part[dir - 1][2 * i + q][lane] = a.up[i][q];
+          part[dir - 1][6 + 2 * i + q][lane] =
+              dir == 1 ? a.give[i][q] : dir == 2 ? a.keep[i][q] : a.keep[i][q] - (q ? 1 : -1);
+        }
+    }
+    __syncthreads();
+    if (dir == 0) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          a.up[i][q] += part[0][2 * i + q][lane] + part[1][2 * i + q][lane] + part[2][2 * i + q][lane];
+          a.give[i][q] += part[0][6 + 2 * i + q][lane] - 1;
+          a.keep[i][q] = part[1][6 + 2 * i + q][lane] + part[2][6 + 2 * i + q][lane];
+        }
+      if (slow) {
+        FixAcc t64;
+        split_site64<DAG>(geo, acc, s, half, &t64);
+        a = t64;
+      }
+      cplx<double> v[6];
+      fix_finish(acc, a, s, half, slow, slow ? -kappa : -kappa * __hiloint2double((E - 56) << 20, 0), v);
+      epi.apply(geo.V, s, half, active, v, red);
+    }
+    __syncthreads();
+  }
+  if constexpr (Epi::REDUCE) {
+    double tot[1];
+    if (grid_sum<1>(red, rs, tot)) epi.finalize(tot);
+  }
+}
+
 // Opts a kernel in to the shared memory of the copying stencil, once per device; its resident
 // blocks there.  `cache`: one slot per device, kept with the kernel's launcher.
 constexpr int kFixDevices = 64;
@@ -597,24 +684,23 @@ inline int fix_wave(const void* kernel, std::atomic<int> (&cache)[kFixDevices]) 
 // against 241 us at 24^3 x 32: fewer of the x and y neighbours are in the block's own lines),
 // three blocks of 80 registers (344, spills), blocks of 4 x 4 x 4 x 2 sites (304: shorter runs per
 // load).  Operands copied ahead (fix_hops_async): 254 instead of 300 us for CG pass 1 there, 290 instead of
-// 342 for pass 2, M^dag M at 32^3 x 64 2.68 instead of 3.6 ms.  A lattice that leaves SMs without a block takes smaller blocks, and without the register
-// cap (its warps are alone on their schedulers: 8^4 14.4 -> 10.3 us).
+// 342 for pass 2, M^dag M at 32^3 x 64 2.68 instead of 3.6 ms.
 // Internal linkage: every translation unit launches its own instance of the kernel and has to opt
 // that instance in (a count cached across units would leave the others at the default shared memory).
 template <bool DAG, class Epi>
 static void launch_dslash_fix(const Geom& geo, const FixGauge& U, SpinorRef in, double kappa, const Epi& epi,
                               const ReduceScratch& rs, cudaStream_t stream) {
-  static const int sms = sm_count();
   const int blocks = grid_for(2 * geo.V, kFixBlock);
-  if (blocks <= sms) {
-    int bs = kFixBlock;
-    while (bs > 32 && grid_for(2 * geo.V, bs) < sms) bs >>= 1;
-    dslash_fix_kernel<DAG, Epi, 1><<<grid_for(2 * geo.V, bs), bs, 0, stream>>>(geo, U, in, kappa, epi, rs);
+  if (geo.V <= kFixDirSites) {
+    static const int dir_wave = resident_grid(reinterpret_cast<const void*>(&dslash_fix_dir_kernel<DAG, Epi>), 128);
+    launch_pdl(&dslash_fix_dir_kernel<DAG, Epi>, std::min(grid_for(geo.V, 16), dir_wave), 128, 0, stream, geo, U, in,
+               kappa, epi, rs);
     return;
   }
   static std::atomic<int> waves[kFixDevices];
-  const int wave = fix_wave(reinterpret_cast<const void*>(&dslash_fix_kernel<DAG, Epi, 2>), waves);
-  dslash_fix_kernel<DAG, Epi, 2><<<std::min(blocks, wave), kFixBlock, kFixSmem, stream>>>(geo, U, in, kappa, epi, rs);
+  const int wave = fix_wave(reinterpret_cast<const void*>(&dslash_fix_kernel<DAG, Epi>), waves);
+  launch_pdl(&dslash_fix_kernel<DAG, Epi>, std::min(blocks, wave), kFixBlock, kFixSmem, stream, geo, U, in, kappa, epi,
+             rs);
 }
 
 }  // namespace lq

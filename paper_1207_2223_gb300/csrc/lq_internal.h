@@ -193,6 +193,14 @@ void pair_cg2(lq_ctx* c, const void* gauge, double kappa, cudaStream_t stream); 
 void cg64_iteration(lq_ctx* c, double kappa, cudaStream_t stream);
 void cg64_true_residual(lq_ctx* c, double kappa, int store_lo_prec, cudaStream_t stream);
 
+// ---- CG iterations of a small lattice inside one cluster, n of them or until halted (k_cgcluster.cu)
+// Up to this many sites 16 SMs are faster than all of them with kernel boundaries (us per iteration of
+// FP16 solves, cluster against kernels: 4^4 14.1 / 18.0, 8^4 13.9 / 17.1, 8^3 x 12 16.5 / 18.5,
+// 8^3 x 16 19.3 / 17.9).
+constexpr int kClusterMaxSites = 6144;
+bool cluster_takes(const lq_ctx* c, int prec);
+cudaError_t cg_cluster_iterations(lq_ctx* c, int prec, int n, double kappa, cudaStream_t stream);
+
 // ---- low-precision CG iteration (k_cglo.cu)
 void cglo_iteration(lq_ctx* c, int prec, double kappa, cudaStream_t stream);
 // single steps (which = 1: t = M p with |t|^2; 2: r -= alpha M^dag t, x += alpha p, |r|^2)
