@@ -43,10 +43,10 @@ __global__ void __launch_bounds__(kFixBlock, MINB)
   double red[1] = {0.0};
   if constexpr (!RESIDUAL) {
     const FixEpiStore epi{out};
-    fix_sites<false, MINB == 2>(fc.geo[k], fc.U[k], in, fc.total, fc.off[col], fc.kappa[k], epi, first, stride, red);
+    fix_sites<false, MINB == 2 ? kFixBlock : 0>(fc.geo[k], fc.U[k], in, fc.total, fc.off[col], fc.kappa[k], epi, first, stride, red);
   } else {
     const FixEpiResidual<S, true, FinBatch, false> epi{phi, SpinorRef{nullptr, nullptr}, out, FinBatch{st, col}};
-    fix_sites<true, MINB == 2>(fc.geo[k], fc.U[k], in, fc.total, fc.off[col], fc.kappa[k], epi, first, stride, red);
+    fix_sites<true, MINB == 2 ? kFixBlock : 0>(fc.geo[k], fc.U[k], in, fc.total, fc.off[col], fc.kappa[k], epi, first, stride, red);
     const ReduceScratch rs{br.partials + (size_t)col * br.max_blocks, br.ticket + col, br.max_blocks};
     double tot[1];
     if (grid_sum<1>(red, rs, tot, block, nblocks)) epi.finalize(tot);
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kFixBlock, MINB)
 template <bool RESIDUAL, SStore S>
 void launch(const Batch64Args& a, FixCols fc, SpinorRef in, SpinorRef out, cudaStream_t st) {
   static std::atomic<int> waves[kFixDevices];
-  const int wave = fix_wave(reinterpret_cast<const void*>(&batch_fix_kernel<RESIDUAL, S, 2>), waves);
+  const int wave = fix_wave(reinterpret_cast<const void*>(&batch_fix_kernel<RESIDUAL, S, 2>), kFixBlock, waves);
   long long pairs = 0;
   for (int c = 0; c < fc.ncols; ++c) pairs += fc.geo[fc.sys[c]].V;
   int bs = kFixBlock;                                   // smaller blocks when the batch leaves SMs idle
@@ -70,7 +70,7 @@ void launch(const Batch64Args& a, FixCols fc, SpinorRef in, SpinorRef out, cudaS
   }
   fc.block0[fc.ncols] = n;
   if (n <= a.sms) batch_fix_kernel<RESIDUAL, S, 1><<<n, bs, 0, st>>>(fc, in, out, a.phi, a.st, a.br);
-  else batch_fix_kernel<RESIDUAL, S, 2><<<n, bs, kFixSmem, st>>>(fc, in, out, a.phi, a.st, a.br);
+  else batch_fix_kernel<RESIDUAL, S, 2><<<n, bs, fix_smem(kFixBlock), st>>>(fc, in, out, a.phi, a.st, a.br);
 }
 
 }  // namespace

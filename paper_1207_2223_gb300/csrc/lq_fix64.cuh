@@ -309,18 +309,18 @@ __device__ __forceinline__ void fix_hops(const Geom& geo, const Acc& in, int s, 
 // elements (copied by both lanes of a pair, 5 and 4), then each lane's 6 spinor components; two
 // stages.  `stage` points at the pair's column of stage 0.
 constexpr int kFixRows = 21;
-constexpr size_t kFixSmem = (size_t)2 * kFixRows * (kFixBlock / 2) * sizeof(int4);
+constexpr size_t fix_smem(int block) { return (size_t)2 * kFixRows * (block / 2) * sizeof(int4); }
 
 __device__ __forceinline__ void fix_copy16(int4* smem, const void* gmem) {
   const unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(smem));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem) : "memory");
 }
-template <int H>
+template <int H, int BS>
 __device__ __forceinline__ void fix_issue(const SoaAccess& in, const int f[4], const int b[4], int s, int half,
                                           int4* stage) {
   constexpr int MU = H >> 1;
   constexpr bool FWD = (H & 1) == 0;
-  constexpr int P = kFixBlock / 2;
+  constexpr int P = BS / 2;
   const int n = FWD ? f[MU] : b[MU];
   int4* st = stage + (H & 1) * (kFixRows * P);
   const int4* u = in.link(MU, FWD ? s : n) + (size_t)(5 * half) * in.V;
@@ -336,14 +336,14 @@ __device__ __forceinline__ void fix_issue(const SoaAccess& in, const int f[4], c
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
-template <int H, bool DAG>
+template <int H, bool DAG, int BS>
 __device__ __forceinline__ void fix_step(const SoaAccess& in, const int f[4], const int b[4], int s, int half, int flip,
                                          unsigned e2, int4* stage, FixAcc& a) {
-  constexpr int MU = H >> 1, P = kFixBlock / 2;
+  constexpr int MU = H >> 1, P = BS / 2;
   constexpr bool FWD = (H & 1) == 0;
   constexpr int S = (DAG ? +1 : -1) * (FWD ? 1 : -1);
   if constexpr (H < 7) {
-    fix_issue<H + 1>(in, f, b, s, half, stage);
+    fix_issue<H + 1, BS>(in, f, b, s, half, stage);
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
   } else {
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -361,19 +361,19 @@ __device__ __forceinline__ void fix_step(const SoaAccess& in, const int f[4], co
   fix_rows<MU, S, FWD>([&](int e) { return st[e * P]; }, hr, hi, -half, a);
   __syncwarp();                                       // the stage may be refilled
 }
-template <bool DAG>
+template <bool DAG, int BS>
 __device__ __forceinline__ void fix_hops_async(const Geom& geo, const SoaAccess& in, int s, const int c[4],
                                                const int f[4], const int b[4], int half, int E, int4* stage, FixAcc& a) {
   const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
   const int ff = (geo.antiperiodic && c[3] == geo.L[3] - 1) ? -1 : 0, fb = (geo.antiperiodic && c[3] == 0) ? -1 : 0;
-  fix_step<0, DAG>(in, f, b, s, half, 0, e2, stage, a);
-  fix_step<1, DAG>(in, f, b, s, half, 0, e2, stage, a);
-  fix_step<2, DAG>(in, f, b, s, half, 0, e2, stage, a);
-  fix_step<3, DAG>(in, f, b, s, half, 0, e2, stage, a);
-  fix_step<4, DAG>(in, f, b, s, half, 0, e2, stage, a);
-  fix_step<5, DAG>(in, f, b, s, half, 0, e2, stage, a);
-  fix_step<6, DAG>(in, f, b, s, half, ff, e2, stage, a);
-  fix_step<7, DAG>(in, f, b, s, half, fb, e2, stage, a);
+  fix_step<0, DAG, BS>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<1, DAG, BS>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<2, DAG, BS>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<3, DAG, BS>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<4, DAG, BS>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<5, DAG, BS>(in, f, b, s, half, 0, e2, stage, a);
+  fix_step<6, DAG, BS>(in, f, b, s, half, ff, e2, stage, a);
+  fix_step<7, DAG, BS>(in, f, b, s, half, fb, e2, stage, a);
 }
 
 // The lane's two spins of M psi at site s: centre + ks * hopping sums.  Each lane completes the
@@ -401,8 +401,8 @@ __device__ __forceinline__ void fix_finish(const Acc& in, const FixAcc& a, int s
 // Spinor fields are [chunk][element] with chunk stride `sstride` (V for a single lattice, the
 // batch's element count for one column of a batch) and the lattice's sites at elements
 // off .. off + V - 1; `in.norm` holds the sites' exponent words.  The epilogue gets the
-// element index.
-template <bool DAG, bool ASYNC, class Epi>
+// element index.  ASYNC: threads per block of the copying variant, 0: loads at their use.
+template <bool DAG, int ASYNC, class Epi>
 __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, const SpinorRef& in, int sstride, int off,
                                           double kappa, const Epi& epi, int first, int stride, double (&red)[1]) {
   const SoaAccess acc{static_cast<const double2*>(in.p) + off, sstride, U.fix, U.f64, geo.V};
@@ -423,7 +423,7 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
       f[m] = nbr_fwd(geo, s, c, m);
       b[m] = nbr_bwd(geo, s, c, m);
     }
-    if constexpr (ASYNC) fix_issue<0>(acc, f, b, s, half, stage);
+    if constexpr (ASYNC) fix_issue<0, ASYNC>(acc, f, b, s, half, stage);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const int wf = __ldg(word + f[m]), wb = __ldg(word + b[m]);
@@ -433,7 +433,7 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
     const bool slow = bad || (any & kFixSlow);
     FixAcc a;
     fix_clear(a);
-    if constexpr (ASYNC) fix_hops_async<DAG>(geo, acc, s, c, f, b, half, E, stage, a);   // every lane: warp barriers
+    if constexpr (ASYNC) fix_hops_async<DAG, ASYNC>(geo, acc, s, c, f, b, half, E, stage, a);   // every lane: warp barriers
     else if (!slow) fix_hops<DAG>(geo, acc, s, c, f, b, half, E, a);
     if (slow) {
       FixAcc t64;
@@ -446,13 +446,13 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
   }
 }
 
-template <bool DAG, class Epi>
-__global__ void __launch_bounds__(kFixBlock, 2)
+template <bool DAG, class Epi, int BS>
+__global__ void __launch_bounds__(BS, 512 / BS)
     dslash_fix_kernel(Geom geo, FixGauge U, SpinorRef in, double kappa, Epi epi, ReduceScratch rs) {
   pdl_wait();
   if (epi.halted()) return;
   double red[1] = {0.0};
-  fix_sites<DAG, true, Epi>(geo, U, in, geo.V, 0, kappa, epi, (blockIdx.x * blockDim.x + threadIdx.x) >> 1,
+  fix_sites<DAG, BS, Epi>(geo, U, in, geo.V, 0, kappa, epi, (blockIdx.x * blockDim.x + threadIdx.x) >> 1,
                       (gridDim.x * blockDim.x) >> 1, red);
   if constexpr (Epi::REDUCE) {
     double tot[1];
@@ -575,9 +575,65 @@ struct FixEpiResidual {
   __device__ void finalize(double (&tot)[1]) const { fin(tot[0]); }
 };
 
-// Small lattices, split by direction like dslash_dir_kernel: four warps share 16 sites (32 lanes), the
-// first adds the integer sums (in any order the same) and finishes the sites.  FP64 CG, us per
-// iteration, split against two threads per site: 4^4 24 / 41, 8^4 31 / 41, 8^3 x 16 34 / 40, 10^4 45 / 41.
+// The lane's two spins of M psi, split by direction: four warps (dir) share 16 sites (32 lanes), the first
+// adds the integer sums (in any order the same) and finishes the sites; v is valid in its lanes.
+// Every thread of the block calls.
+template <bool DAG, class Acc>
+__device__ __forceinline__ void fix_dir_site(const Geom& geo, const Acc& acc, int s, const int c[4], const int f[4],
+                                             const int b[4], int E, bool slow, int lane, int dir, double kappa,
+                                             long long (&part)[3][12][32], cplx<double> v[6]) {
+  constexpr int SF = DAG ? +1 : -1;
+  const int half = lane & 1, ls = -half;
+  const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
+  FixAcc a;
+  fix_clear(a);
+  if (dir == 0) {
+    fix_hop<0, SF, true>(acc, f[0], s, half, ls, 0, e2, a);
+    fix_hop<0, -SF, false>(acc, b[0], b[0], half, ls, 0, e2, a);
+  } else if (dir == 1) {
+    fix_hop<1, SF, true>(acc, f[1], s, half, ls, 0, e2, a);
+    fix_hop<1, -SF, false>(acc, b[1], b[1], half, ls, 0, e2, a);
+  } else if (dir == 2) {
+    fix_hop<2, SF, true>(acc, f[2], s, half, ls, 0, e2, a);
+    fix_hop<2, -SF, false>(acc, b[2], b[2], half, ls, 0, e2, a);
+  } else {
+    const int ff = (geo.antiperiodic && c[3] == geo.L[3] - 1) ? -1 : 0, fb = (geo.antiperiodic && c[3] == 0) ? -1 : 0;
+    fix_hop<3, SF, true>(acc, f[3], s, half, ls, ff, e2, a);
+    fix_hop<3, -SF, false>(acc, b[3], b[3], half, ls, fb, e2, a);
+  }
+  // x, y add to "give", z, t to "keep"; the start values of fix_clear (give 1; keep -1, 1) are
+  // counted once each, those of the warps of y and z
+  if (dir > 0) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        part[dir - 1][2 * i + q][lane] = a.up[i][q];
+        part[dir - 1][6 + 2 * i + q][lane] =
+            dir == 1 ? a.give[i][q] : dir == 2 ? a.keep[i][q] : a.keep[i][q] - (q ? 1 : -1);
+      }
+  }
+  __syncthreads();
+  if (dir > 0) return;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      a.up[i][q] += part[0][2 * i + q][lane] + part[1][2 * i + q][lane] + part[2][2 * i + q][lane];
+      a.give[i][q] += part[0][6 + 2 * i + q][lane] - 1;
+      a.keep[i][q] = part[1][6 + 2 * i + q][lane] + part[2][6 + 2 * i + q][lane];
+    }
+  if (slow) {
+    FixAcc t64;
+    split_site64<DAG>(geo, acc, s, half, &t64);
+    a = t64;
+  }
+  fix_finish(acc, a, s, half, slow, slow ? -kappa : -kappa * __hiloint2double((E - 56) << 20, 0), v);
+}
+
+// Small lattices leave most of the chip idle, and a pass takes as long as one thread needs for its
+// eight hops: split by direction.  FP64 CG, us per iteration, split against two threads per site:
+// 4^4 24 / 41, 8^4 31 / 41, 8^3 x 16 34 / 40, 10^4 45 / 41.
 constexpr int kFixDirSites = 8192;
 template <bool DAG, class Epi>
 __global__ void __launch_bounds__(128, 4)
@@ -585,11 +641,10 @@ __global__ void __launch_bounds__(128, 4)
   __shared__ long long part[3][12][32];
   pdl_wait();
   if (epi.halted()) return;
-  constexpr int SF = DAG ? +1 : -1;
   const SoaAccess acc{static_cast<const double2*>(in.p), geo.V, U.fix, U.f64, geo.V};
   const int* word = reinterpret_cast<const int*>(in.norm);
   const bool bad = __ldg(U.bad) != 0;
-  const int lane = threadIdx.x & 31, dir = threadIdx.x >> 5, half = lane & 1, ls = -half;
+  const int lane = threadIdx.x & 31, dir = threadIdx.x >> 5;
   double red[1] = {0.0};
   for (int base = blockIdx.x * 16; base < geo.V; base += gridDim.x * 16) {
     const bool active = base + (lane >> 1) < geo.V;
@@ -606,54 +661,9 @@ __global__ void __launch_bounds__(128, 4)
       E = max(E, max(wf & 0x7ff, wb & 0x7ff));
     }
     const bool slow = bad || (any & kFixSlow);
-    const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
-    FixAcc a;
-    fix_clear(a);
-    if (dir == 0) {
-      fix_hop<0, SF, true>(acc, f[0], s, half, ls, 0, e2, a);
-      fix_hop<0, -SF, false>(acc, b[0], b[0], half, ls, 0, e2, a);
-    } else if (dir == 1) {
-      fix_hop<1, SF, true>(acc, f[1], s, half, ls, 0, e2, a);
-      fix_hop<1, -SF, false>(acc, b[1], b[1], half, ls, 0, e2, a);
-    } else if (dir == 2) {
-      fix_hop<2, SF, true>(acc, f[2], s, half, ls, 0, e2, a);
-      fix_hop<2, -SF, false>(acc, b[2], b[2], half, ls, 0, e2, a);
-    } else {
-      const int ff = (geo.antiperiodic && c[3] == geo.L[3] - 1) ? -1 : 0, fb = (geo.antiperiodic && c[3] == 0) ? -1 : 0;
-      fix_hop<3, SF, true>(acc, f[3], s, half, ls, ff, e2, a);
-      fix_hop<3, -SF, false>(acc, b[3], b[3], half, ls, fb, e2, a);
-    }
-    // x, y add to "give", z, t to "keep"; the start values of fix_clear (give 1; keep -1, 1) are
-    // counted once each, here in the warps of y and z
-    if (dir > 0) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          part[dir - 1][2 * i + q][lane] = a.up[i][q];
-          part[dir - 1][6 + 2 * i + q][lane] =
-              dir == 1 ? a.give[i][q] : dir == 2 ? a.keep[i][q] : a.keep[i][q] - (q ? 1 : -1);
-        }
-    }
-    __syncthreads();
-    if (dir == 0) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          a.up[i][q] += part[0][2 * i + q][lane] + part[1][2 * i + q][lane] + part[2][2 * i + q][lane];
-          a.give[i][q] += part[0][6 + 2 * i + q][lane] - 1;
-          a.keep[i][q] = part[1][6 + 2 * i + q][lane] + part[2][6 + 2 * i + q][lane];
-        }
-      if (slow) {
-        FixAcc t64;
-        split_site64<DAG>(geo, acc, s, half, &t64);
-        a = t64;
-      }
-      cplx<double> v[6];
-      fix_finish(acc, a, s, half, slow, slow ? -kappa : -kappa * __hiloint2double((E - 56) << 20, 0), v);
-      epi.apply(geo.V, s, half, active, v, red);
-    }
+    cplx<double> v[6];
+    fix_dir_site<DAG>(geo, acc, s, c, f, b, E, slow, lane, dir, kappa, part, v);
+    if (dir == 0) epi.apply(geo.V, s, lane & 1, active, v, red);
     __syncthreads();
   }
   if constexpr (Epi::REDUCE) {
@@ -665,15 +675,15 @@ __global__ void __launch_bounds__(128, 4)
 // Opts a kernel in to the shared memory of the copying stencil, once per device; its resident
 // blocks there.  `cache`: one slot per device, kept with the kernel's launcher.
 constexpr int kFixDevices = 64;
-inline int fix_wave(const void* kernel, std::atomic<int> (&cache)[kFixDevices]) {
+inline int fix_wave(const void* kernel, int block, std::atomic<int> (&cache)[kFixDevices]) {
   int dev = 0;
   cudaGetDevice(&dev);
   std::atomic<int>& slot = cache[dev & (kFixDevices - 1)];
   int wave = slot.load(std::memory_order_acquire);
   if (wave == 0) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFixSmem);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fix_smem(block));
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kFixBlock, kFixSmem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, fix_smem(block));
     wave = sm_count() * std::max(1, per_sm);
     slot.store(wave, std::memory_order_release);
   }
@@ -687,20 +697,39 @@ inline int fix_wave(const void* kernel, std::atomic<int> (&cache)[kFixDevices]) 
 // 342 for pass 2, M^dag M at 32^3 x 64 2.68 instead of 3.6 ms.
 // Internal linkage: every translation unit launches its own instance of the kernel and has to opt
 // that instance in (a count cached across units would leave the others at the default shared memory).
+template <bool DAG, class Epi, int BS>
+static void launch_fix_async(const Geom& geo, const FixGauge& U, SpinorRef in, double kappa, const Epi& epi,
+                             const ReduceScratch& rs, cudaStream_t stream) {
+  static std::atomic<int> waves[kFixDevices];
+  const int wave = fix_wave(reinterpret_cast<const void*>(&dslash_fix_kernel<DAG, Epi, BS>), BS, waves);
+  launch_pdl(&dslash_fix_kernel<DAG, Epi, BS>, std::min(grid_for(2 * geo.V, BS), wave), BS, fix_smem(BS), stream, geo, U, in,
+             kappa, epi, rs);
+}
+
+// Threads per block for V sites: the SM with most work has ceil(blocks / SMs) of them, which at a few
+// blocks per SM is well above the average; blocks of 128 where that SM then has at least 5% less to
+// do (12^4: 3 of 128 instead of 2 of 256, FP64 CG iteration 58 -> 50 us; 16^4: 7 instead of 4, pass 1
+// 47 -> 44 us; blocks of 64 were no better: 51 us at 12^4).
+inline int fix_block(int V) {
+  static const int sms = sm_count();
+  constexpr int half = kFixBlock / 2;
+  const long long full = 2ll * grid_for(grid_for(2 * V, kFixBlock), sms), small = grid_for(grid_for(2 * V, half), sms);
+  return 20 * small < 19 * full ? half : kFixBlock;
+}
+
 template <bool DAG, class Epi>
 static void launch_dslash_fix(const Geom& geo, const FixGauge& U, SpinorRef in, double kappa, const Epi& epi,
                               const ReduceScratch& rs, cudaStream_t stream) {
-  const int blocks = grid_for(2 * geo.V, kFixBlock);
   if (geo.V <= kFixDirSites) {
     static const int dir_wave = resident_grid(reinterpret_cast<const void*>(&dslash_fix_dir_kernel<DAG, Epi>), 128);
     launch_pdl(&dslash_fix_dir_kernel<DAG, Epi>, std::min(grid_for(geo.V, 16), dir_wave), 128, 0, stream, geo, U, in,
                kappa, epi, rs);
     return;
   }
-  static std::atomic<int> waves[kFixDevices];
-  const int wave = fix_wave(reinterpret_cast<const void*>(&dslash_fix_kernel<DAG, Epi>), waves);
-  launch_pdl(&dslash_fix_kernel<DAG, Epi>, std::min(blocks, wave), kFixBlock, kFixSmem, stream, geo, U, in, kappa, epi,
-             rs);
+  switch (fix_block(geo.V)) {
+    case 128: launch_fix_async<DAG, Epi, 128>(geo, U, in, kappa, epi, rs, stream); break;
+    default: launch_fix_async<DAG, Epi, 256>(geo, U, in, kappa, epi, rs, stream); break;
+  }
 }
 
 }  // namespace lq
