@@ -269,6 +269,7 @@ BatchDesc make_desc(lq_ctx** ctxs, int n, int R, const double* const* phi, doubl
     SysDesc& sd = bd.sys[k];
     sd.geo = ctxs[k]->geo;
     sd.gauge_lo = ctxs[k]->gauge_lo[prec];
+    sd.fix = fix_gauge_of(ctxs[k]);
     sd.kappa = kappa[k];
     sd.R = R;
     sd.off = off;
@@ -665,8 +666,7 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
   const BatchDesc bd = make_desc(ctxs, n, nrhs, phi, x, kappa, inner_prec, tu.tile, tu.rb, tu.site_major);
   batch_init(w, bdi, inner_prec, st);
   s.kernel_launches += 1;
-  Batch64Args a64{w->x64.ref(), w->tmp64.ref(), w->phi64.ref(), w->rlo.ref(), w->st, w->br, {}, w->sms};
-  for (int k = 0; k < n; ++k) a64.U[k] = fix_gauge_of(ctxs[k]);
+  const Batch64Args a64{w->x64.ref(), w->tmp64.ref(), w->phi64.ref(), w->rlo.ref(), w->st, w->br, w->sms};
 
   const int chunk = reliable_every;
   lq_status result = LQ_OK;

@@ -81,7 +81,7 @@ void batch_true_residual(const Batch64Args& a, const BatchDesc& bd, SStore s, cu
   fc.ncols = bd.ncols;
   for (int k = 0; k < bd.nsys; ++k) {
     fc.geo[k] = bd.sys[k].geo;
-    fc.U[k] = a.U[k];
+    fc.U[k] = bd.sys[k].fix;
     fc.kappa[k] = bd.sys[k].kappa;
     for (int r = 0; r < bd.sys[k].R; ++r) {
       fc.sys[bd.sys[k].col + r] = k;

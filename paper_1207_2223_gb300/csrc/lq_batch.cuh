@@ -19,6 +19,7 @@ constexpr int kMaxRB = 4;
 struct SysDesc {
   Geom geo;
   const void* gauge_lo;   // inner-format links of the system (SoA, stride V)
+  FixGauge fix;           // links of the FP64 updates
   double kappa;
   int R;                  // right-hand sides
   int off;                // first element in the batch fields
@@ -706,7 +707,6 @@ struct Batch64Args {
   SpinorRef x, tmp, phi, rlo;
   BatchState* st;
   BatchReduce br;
-  FixGauge U[kMaxSys];
   int sms;
 };
 void batch_true_residual(const Batch64Args& a, const BatchDesc& bd, SStore s, cudaStream_t st);

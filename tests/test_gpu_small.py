@@ -49,3 +49,33 @@ def test_solves_around_the_limits(lq, dims, prec):
         assert status == lq.LQ_ERR_NOT_CONVERGED and st["iterations"] == 7
     finally:
         lq.lq_destroy(ctx)
+
+
+def test_batch_with_a_context_replaced(lq):
+    """The recorded solve graph of a batch holds its systems' links: a second context destroyed and
+    created anew (at whatever addresses) between two solves is solved with its own links."""
+    import torch
+    dims, kappa = (4, 4, 4, 4), 0.15
+    lat = Lattice(dims)
+    phi = dev(source(lat, 3))
+    first = lq.lq_create(dims)
+    try:
+        lq.lq_gauge_set(first, dev(gauge_exp_iA(lat, 0.3, 21)))
+        for seed in (22, 23, 24):
+            second = lq.lq_create(dims)
+            try:
+                lq.lq_gauge_set(second, dev(gauge_exp_iA(lat, 0.3, seed)))
+                if seed == 23:              # other allocations in between
+                    lq.lq_apply_M(second, torch.empty_like(phi), phi, kappa, False, lq.LQ_DF64)
+                xs = [torch.zeros_like(phi), torch.zeros_like(phi)]
+                status, st, _, resid, _ = lq.lq_solve_batch([first, second], xs, [phi, phi], [kappa, kappa], 1, 1e-10,
+                                                            3000, lq.LQ_F16_12, 25)
+                assert status == lq.LQ_OK and np.all(resid <= 1e-10)
+                for c, x in zip((first, second), xs):
+                    r = torch.empty_like(phi)
+                    lq.lq_apply_MdagM(c, r, x, kappa, lq.LQ_F64)
+                    assert float(torch.linalg.vector_norm(phi - r) / torch.linalg.vector_norm(phi)) <= 1.01e-10
+            finally:
+                lq.lq_destroy(second)
+    finally:
+        lq.lq_destroy(first)
