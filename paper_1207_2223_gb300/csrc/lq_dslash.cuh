@@ -119,12 +119,8 @@ __device__ __forceinline__ void hop_dir(const Geom& geo, const GaugeRef& U, cons
   }
 }
 
-// Threads per block: 256 for FP32 arithmetic; 128 for FP64 and double-float,
-// whose 190-250 registers per thread would otherwise leave one block per SM
-// (the FP64 pipe, not occupancy, bounds the FP64 operator).
-template <typename T> struct DslashBlock { static constexpr int value = 256; };
-template <> struct DslashBlock<double> { static constexpr int value = 128; };
-template <> struct DslashBlock<df64> { static constexpr int value = 128; };
+// Threads per block.
+constexpr int kDslashBlock = 256;
 // Minimum resident blocks per SM requested from the compiler (register cap).
 #ifndef LQ_DSLASH_MIN_BLOCKS
 #define LQ_DSLASH_MIN_BLOCKS 2
@@ -168,7 +164,7 @@ inline void launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
 // walks the lattice in steps of the grid size, so the halt check and the
 // block reduction happen once per block rather than once per 256 sites.
 template <typename T, GStore G, SStore SI, bool DAG, class Epi>
-__global__ void __launch_bounds__(DslashBlock<T>::value, (EpiMinBlocks<T, Epi>::value)) dslash_kernel(Geom geo, GaugeRef U, SpinorRef in,
+__global__ void __launch_bounds__(kDslashBlock, (EpiMinBlocks<T, Epi>::value)) dslash_kernel(Geom geo, GaugeRef U, SpinorRef in,
                                                                         T kappa, Epi epi, ReduceScratch rs) {
   pdl_wait();
   if (epi.halted()) return;
@@ -210,20 +206,6 @@ struct EpiStore {                       // out = M psi
     store_spinor<SO, T>(out, V, s, v);
   }
   __device__ void finalize(double (&)[NRED]) const {}
-};
-
-template <SStore SO>
-struct EpiStoreNorm {                   // out = M psi, *result = |out|^2
-  static constexpr int NRED = 1;
-  static constexpr bool REDUCE = true;
-  SpinorRef out;
-  double* result;
-  __device__ bool halted() const { return false; }
-  template <typename T> __device__ void apply(int V, int s, cplx<T> v[12], double (&red)[NRED]) const {
-    store_spinor<SO, T>(out, V, s, v);
-    red[0] += site_norm2(v);
-  }
-  __device__ void finalize(double (&tot)[NRED]) const { *result = tot[0]; }
 };
 
 // CG step 1:  t = M p, tt = |t|^2, alpha = rr / tt
@@ -303,32 +285,6 @@ struct EpiCG2 {
 template <SStore S> struct EpiMinBlocks<float, EpiCG1<S>> { static constexpr int value = LQ_K1_MIN_BLOCKS; };
 template <SStore S> struct EpiMinBlocks<float, EpiStore<S>> { static constexpr int value = LQ_K1_MIN_BLOCKS; };
 
-// True residual in FP64:  v = M^dag (M x)  ->  r = phi - v, |r|^2.
-// Optionally also stores r in a low-precision field (reliable update).
-template <SStore SLO, bool STORE_LO>
-struct EpiResidual {
-  static constexpr int NRED = 1;
-  static constexpr bool REDUCE = true;
-  SpinorRef phi, r, r_lo;
-  SolverState* st;
-  __device__ bool halted() const { return false; }
-  template <typename T> __device__ void apply(int V, int s, cplx<T> v[12], double (&red)[NRED]) const {
-    cplx<double> ph[12];
-    load_spinor<SStore::F64, double>(phi, V, s, ph);
-    cplx<double> rv[12];
-    double a = 0.0;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      rv[k] = {ph[k].re - (double)v[k].re, ph[k].im - (double)v[k].im};
-      a += rv[k].re * rv[k].re + rv[k].im * rv[k].im;
-    }
-    store_spinor<SStore::F64, double>(r, V, s, rv);
-    if constexpr (STORE_LO) store_spinor<SLO, double>(r_lo, V, s, rv);
-    red[0] += a;
-  }
-  __device__ void finalize(double (&tot)[NRED]) const { st->rr_true = tot[0]; }
-};
-
 inline int grid_for(int V, int bs) { return (V + bs - 1) / bs; }
 
 // Resident blocks of one kernel on the current device (queried once per kernel).
@@ -341,7 +297,7 @@ int sm_count();                        // SMs of the current device
 template <typename T, GStore G, SStore SI, bool DAG, class Epi>
 inline void launch_dslash(const Geom& geo, GaugeRef U, SpinorRef in, double kappa, const Epi& epi,
                           const ReduceScratch& rs, cudaStream_t stream) {
-  constexpr int bs = DslashBlock<T>::value;
+  constexpr int bs = kDslashBlock;
   const void* kern = reinterpret_cast<const void*>(&dslash_kernel<T, G, SI, DAG, Epi>);
   static const int wave = resident_grid(kern, bs);
   if (2 * grid_for(geo.V, bs) <= wave) {

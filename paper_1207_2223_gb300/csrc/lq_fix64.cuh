@@ -423,7 +423,9 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
       f[m] = nbr_fwd(geo, s, c, m);
       b[m] = nbr_bwd(geo, s, c, m);
     }
-    if constexpr (ASYNC) fix_issue<0, ASYNC>(acc, f, b, s, half, stage);
+    if constexpr (ASYNC) {
+      if (!bad) fix_issue<0, ASYNC>(acc, f, b, s, half, stage);
+    }
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const int wf = __ldg(word + f[m]), wb = __ldg(word + b[m]);
@@ -433,8 +435,11 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
     const bool slow = bad || (any & kFixSlow);
     FixAcc a;
     fix_clear(a);
-    if constexpr (ASYNC) fix_hops_async<DAG, ASYNC>(geo, acc, s, c, f, b, half, E, stage, a);   // every lane: warp barriers
-    else if (!slow) fix_hops<DAG>(geo, acc, s, c, f, b, half, E, a);
+    if constexpr (ASYNC) {
+      if (!bad) fix_hops_async<DAG, ASYNC>(geo, acc, s, c, f, b, half, E, stage, a);   // every lane: warp barriers
+    } else if (!slow) {
+      fix_hops<DAG>(geo, acc, s, c, f, b, half, E, a);
+    }
     if (slow) {
       FixAcc t64;
       split_site64<DAG>(geo, acc, s, half, &t64);
