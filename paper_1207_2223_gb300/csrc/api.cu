@@ -264,17 +264,23 @@ lq_status solve_internal(lq_ctx* c, double kappa, double tol, int maxiter, int i
     for (long guard = 0; guard < (long)maxiter + 64; ++guard) {
       LQ_TRY(run_chunk(c, inner, chunk, kappa));
       s.kernel_launches += cluster_takes(c, inner) ? 1 : 3 * chunk;
-      LQ_TRY(read_state(c));
+      // a chunk of reliable_every iterations ends in a halt (an update is due at the latest), so a
+      // mixed solve goes straight to the update and waits for the device once
       const SolverState& st = *c->state_host;
-      if (st.breakdown) { result = fail(c, LQ_ERR_NAN, "CG breakdown (non-positive or non-finite curvature)"); break; }
-      if (!st.halt) continue;
+      const bool due = mixed && reliable_every > 0;
+      if (!due) {
+        LQ_TRY(read_state(c));
+        if (st.breakdown) { result = fail(c, LQ_ERR_NAN, "CG breakdown (non-positive or non-finite curvature)"); break; }
+        if (!st.halt) continue;
+      }
       // true residual; for mixed solves this is the reliable update
       if (mixed) launch_accumulate_x(g, slo, c->x_lo[k].ref(), c->x64.ref(), c->stream);
       cg64_true_residual(c, kappa, inner, c->stream);
       s.kernel_launches += mixed ? 3 : 2;
       LQ_CUDA(c, cudaGetLastError());
       LQ_TRY(read_state(c));
-      rel = std::sqrt(c->state_host->rr_true / c->state_host->phi2);
+      if (st.breakdown) { result = fail(c, LQ_ERR_NAN, "CG breakdown (non-positive or non-finite curvature)"); break; }
+      rel = std::sqrt(st.rr_true / st.phi2);
       if (mixed) s.reliable_updates++;
       const double rr_true = c->state_host->rr_true;
       if (!std::isfinite(rel)) { result = fail(c, LQ_ERR_NAN, "non-finite residual"); break; }
