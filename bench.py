@@ -715,15 +715,15 @@ def run_ours(args):
             gbs = DSLASH_BYTES[name] * V / (ms * 1e-3) / 1e9
             dsl[name] = {"ms": round(ms, 5), "GB/s": round(gbs, 1), "frac_hbm": round(gbs / hbm, 4),
                          "GFLOP/s": round(DSLASH_FLOPS * V / (ms * 1e-3) / 1e9, 1)}
-        # the FP64 operator runs on the integer pipe (lq_fix64.cuh): its rate beside the measured
-        # FP64 fused multiply-add rate of this GPU, which bounds FP64 arithmetic (frac above 1)
+        # the FP64 operator runs on the integer pipe (lq_fix64.cuh), so its rate is also given as a
+        # multiple of the measured FP64 fused multiply-add rate, which bounds FP64 arithmetic
         fma = {"f64_tflops": lq.lq_time_fma_peak(ctx, lq.LQ_F64), "f32_tflops": lq.lq_time_fma_peak(ctx, lq.LQ_F32)}
         d64 = dsl["f64"]
-        fp64_roofline = {"kernel": "dslash_fix_kernel (M, FP64 fields)", "bound": "alu",
-                         "achieved": round(d64["GFLOP/s"] / 1e3, 4), "peak": round(fma["f64_tflops"], 4),
-                         "unit": "TFLOP/s", "frac": round(d64["GFLOP/s"] / 1e3 / fma["f64_tflops"], 4),
-                         "peak_kind": "measured (lq_time_fma_peak: FP64 fused multiply-add chains)",
-                         "flop_per_site": DSLASH_FLOPS, "launch_ms": d64["ms"]}
+        fp64_roofline = {"kernel": "dslash_fix_kernel (M, FP64 fields)", "bound": "integer pipe and issue",
+                         "achieved": d64["GB/s"], "peak": hbm, "unit": "GB/s", "frac": d64["frac_hbm"],
+                         "peak_kind": peak_kind, "bytes_per_site": DSLASH_BYTES["f64"],
+                         "times_fp64_fma_rate": round(d64["GFLOP/s"] / 1e3 / fma["f64_tflops"], 4),
+                         "launch_ms": d64["ms"]}
         cg = {}
         for which in ("k1", "k2", "k3"):
             ms = lq.lq_time_cg_kernel(ctx, phid, KAPPA, int(which[1]), inner, 40)
