@@ -59,6 +59,115 @@ struct SingleIndex {
   __device__ __forceinline__ int operator()(int n) const { return n; }
 };
 
+// ------------------------------------------------ packed FP32x2 arithmetic
+// The two colour vectors h0, h1 of a hop take the same steps, so every real of the hop is held as the
+// pair (value of h0, value of h1) and one packed instruction does both: (x, y) of a float2.  That
+// takes ~40 of 180 instructions per hop away and leaves the FMA pipe as busy (a packed instruction
+// holds it for two cycles).  BF16 storage, decoded by shifts on the ALU pipe, was bound by issue and
+// gains: at 32^3 x 64 M 157 -> 144 us, CG pass 1 159 -> 144, pass 2 194 -> 183; 8^4 pass 2 7.8 -> 6.6.
+// FP16 and 16-bit fixed point, whose decoding is FMA-pipe work, lose (pass 1 154 -> 157 and 156 -> 165 us)
+// and FP32 storage, which arrives in pairs (re, im), gains nothing (162 -> 167): they stay scalar.
+__device__ __forceinline__ float2 pk(float a, float b) { return make_float2(a, b); }
+// a + (sx b.x, sy b.y), one rounding each
+template <int SX, int SY> __device__ __forceinline__ float2 add_signed(float2 a, float2 b) {
+  if constexpr (SX > 0 && SY > 0) return __fadd2_rn(a, b);
+  else return __ffma2_rn(b, pk((float)SX, (float)SY), a);
+}
+
+template <int MU, int S>
+__device__ __forceinline__ void project2(const cplx<float> p[12], float2 hr[3], float2 hi[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const cplx<float> p0 = p[c], p1 = p[3 + c], p2 = p[6 + c], p3 = p[9 + c];
+    const float2 r = pk(p0.re, p1.re), i = pk(p0.im, p1.im);
+    if constexpr (MU == 0) {
+      hr[c] = add_signed<-S, -S>(r, pk(p3.im, p2.im));
+      hi[c] = add_signed<S, S>(i, pk(p3.re, p2.re));
+    } else if constexpr (MU == 1) {
+      hr[c] = add_signed<-S, S>(r, pk(p3.re, p2.re));
+      hi[c] = add_signed<-S, S>(i, pk(p3.im, p2.im));
+    } else if constexpr (MU == 2) {
+      hr[c] = add_signed<-S, S>(r, pk(p2.im, p3.im));
+      hi[c] = add_signed<S, -S>(i, pk(p2.re, p3.re));
+    } else {
+      hr[c] = add_signed<S, S>(r, pk(p2.re, p3.re));
+      hi[c] = add_signed<S, S>(i, pk(p2.im, p3.im));
+    }
+  }
+}
+
+template <int SX, int SY, bool INIT> __device__ __forceinline__ void acc2(float& x, float& y, float2 w) {
+  if constexpr (INIT) {
+    x = SX > 0 ? w.x : -w.x;
+    y = SY > 0 ? w.y : -w.y;
+  } else {
+    const float2 r = add_signed<SX, SY>(pk(x, y), w);
+    x = r.x;
+    y = r.y;
+  }
+}
+template <int MU, int S, bool INIT>
+__device__ __forceinline__ void accumulate2(cplx<float> acc[12], const float2 wr[3], const float2 wi[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    cplx<float>&a0 = acc[c], &a1 = acc[3 + c], &a2 = acc[6 + c], &a3 = acc[9 + c];
+    acc2<1, 1, INIT>(a0.re, a1.re, wr[c]);
+    acc2<1, 1, INIT>(a0.im, a1.im, wi[c]);
+    if constexpr (MU == 0) {
+      acc2<S, S, INIT>(a3.re, a2.re, wi[c]);
+      acc2<-S, -S, INIT>(a3.im, a2.im, wr[c]);
+    } else if constexpr (MU == 1) {
+      acc2<-S, S, INIT>(a3.re, a2.re, wr[c]);
+      acc2<-S, S, INIT>(a3.im, a2.im, wi[c]);
+    } else if constexpr (MU == 2) {
+      acc2<S, -S, INIT>(a2.re, a3.re, wi[c]);
+      acc2<-S, S, INIT>(a2.im, a3.im, wr[c]);
+    } else {
+      acc2<S, S, INIT>(a2.re, a3.re, wr[c]);
+      acc2<S, S, INIT>(a2.im, a3.im, wi[c]);
+    }
+  }
+}
+
+// w = U h (DAGU: U^dag h), with n = -h.im (DAGU: -h.re)
+template <bool DAGU>
+__device__ __forceinline__ void su3_mul2(const cplx<float> u[9], const float2 hr[3], const float2 hi[3], const float2 n[3],
+                                         float2 wr[3], float2 wi[3]) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const cplx<float> e = DAGU ? u[3 * j + i] : u[3 * i + j];
+      const float2 er = pk(e.re, e.re), ei = pk(e.im, e.im);
+      wr[i] = j == 0 ? __fmul2_rn(er, hr[j]) : __ffma2_rn(er, hr[j], wr[i]);
+      wr[i] = __ffma2_rn(ei, DAGU ? hi[j] : n[j], wr[i]);
+      wi[i] = j == 0 ? __fmul2_rn(er, hi[j]) : __ffma2_rn(er, hi[j], wi[i]);
+      wi[i] = __ffma2_rn(ei, DAGU ? n[j] : hr[j], wi[i]);
+    }
+}
+
+// One hop of BF16 storage: the spinor of site n by the link at `link` (forward: U, backward: U^dag).  The
+// antiperiodic sign is folded into the norm.
+template <int MU, int S, bool FWD, GStore G, SStore SI, bool INIT, int LD, class IX>
+__device__ __forceinline__ void hop_packed(const GaugeRef& U, int V, const SpinorRef& in, int n, int link, bool flip,
+                                           cplx<float> acc[12], IX ix) {
+  cplx<float> p[12], u[9];
+  float sc = load_spinor_raw<SI, float, LD>(in, ix.stride(), ix(n), p);
+  float2 hr[3], hi[3], ng[3], wr[3], wi[3];
+  project2<MU, S>(p, hr, hi);
+  if (flip) sc = -sc;
+  const float2 s2 = pk(sc, sc), m2 = pk(-sc, -sc);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    ng[c] = __fmul2_rn(FWD ? hi[c] : hr[c], m2);
+    hr[c] = __fmul2_rn(hr[c], s2);
+    hi[c] = __fmul2_rn(hi[c], s2);
+  }
+  load_link<G, float>(U, V, MU, link, u);
+  su3_mul2<!FWD>(u, hr, hi, ng, wr, wi);
+  accumulate2<MU, S, INIT>(acc, wr, wi);
+}
+
 // Both hops of direction MU at site s.  INIT: the forward hop is the site's first
 // contribution and sets acc (the first direction of the stencil).  The antiperiodic
 // sign of a hop across the time boundary is folded into the norm scale of 16-bit
@@ -68,6 +177,12 @@ __device__ __forceinline__ void hop_dir(const Geom& geo, const GaugeRef& U, cons
                                         const int c[4], cplx<T> acc[12], IX ix = IX{0}) {
   if constexpr (std::is_same<IX, SingleIndex>::value) ix.V = geo.V;
   constexpr int SF = DAG ? +1 : -1;   // forward hop uses (1 + SF g_mu)
+  if constexpr (std::is_same<T, float>::value && SI == SStore::BF16 && G == GStore::BF16_12) {
+    const int f = nbr_fwd(geo, s, c, MU), b = nbr_bwd(geo, s, c, MU);
+    hop_packed<MU, SF, true, G, SI, INIT, LD>(U, geo.V, in, f, s, MU == 3 && geo.antiperiodic && c[3] == geo.L[3] - 1, acc, ix);
+    hop_packed<MU, -SF, false, G, SI, false, LD>(U, geo.V, in, b, b, MU == 3 && geo.antiperiodic && c[3] == 0, acc, ix);
+    return;
+  }
   constexpr bool SCALED = SI == SStore::F16 || SI == SStore::BF16 || SI == SStore::I16 || G == GStore::I16_12;
   {
     const int n = nbr_fwd(geo, s, c, MU);
