@@ -39,9 +39,12 @@ __device__ __forceinline__ unsigned cluster_size() {
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
   return r;
 }
-// All threads of the cluster; global and shared writes before it are visible after it.
+// All threads of the cluster; global and shared writes before it are visible after it (release and acquire, so
+// that plain loads of what other blocks wrote before it do not see older lines).  Not the .aligned forms: it is
+// entered after loops whose trip count differs within the last warp of a ragged lattice, and nothing
+// promises that the lanes of a warp have met again by then.
 __device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // Barrier of the cluster; f(sum of all threads' v, in a fixed order) in the first thread of every
@@ -70,6 +73,7 @@ __device__ __forceinline__ void cluster_sum(double v, double (*slots)[kMaxCluste
   __syncthreads();
 }
 
+// Load mode 0: the neighbours' elements come from other blocks of this launch, ordered by cluster_barrier.
 template <bool DAG, GStore G, SStore S>
 __device__ __forceinline__ void stencil(const Geom& geo, const GaugeRef& U, const SpinorRef& in, int s, float kappa,
                                         cplx<float> acc[12]) {

@@ -142,7 +142,8 @@ template <> struct SpinorTraits<SStore::I16> { using half_t = void; };
 // ----------------------------------------------------------- spinor I/O
 // Load path of a field:
 //   1 (true)   read-only for the whole kernel: the non-coherent read-only path
-//   0 (false)  a field the kernel also writes (each element by the thread that reads it)
+//   0 (false)  a field the kernel also writes: each element by the thread that reads it, or by other
+//              blocks before a barrier with acquire semantics (barrier.cluster) that the reader waited at
 //   2          written by other blocks of the same kernel before a device-wide barrier
 //              (persistent kernels): L2 only, never a stale L1 line
 template <int RO, typename W> __device__ __forceinline__ W ld(const W* p) {

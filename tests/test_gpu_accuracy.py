@@ -1,0 +1,104 @@
+"""FP64 entry points computed in fixed point (csrc/lq_fix64.cuh, lq_fixsu3.cuh) against extended precision,
+on the inputs where a fixed unit could cost digits that FP64 arithmetic keeps."""
+import numpy as np
+import pytest
+
+from oracle.wilson import apply_M
+from synth import Lattice, gauge_exp_iA, source
+from tests.gpu_common import require_gpu, dev, host, torch
+
+pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def lq():
+    return require_gpu()
+
+
+class _Context:
+    def __init__(self, lq, dims, U):
+        self.lq, self.dims, self.U = lq, dims, U
+
+    def __enter__(self):
+        self.ctx = self.lq.lq_create(self.dims)
+        self.lq.lq_gauge_set(self.ctx, dev(self.U))
+        return self.ctx
+
+    def __exit__(self, *exc):
+        self.lq.lq_destroy(self.ctx)
+
+
+def _M(lq, ctx, psi, kappa, dagger=False):
+    out = torch.empty(psi.shape, dtype=torch.complex128, device="cuda")
+    lq.lq_apply_M(ctx, out, dev(psi), kappa, dagger, lq.LQ_F64)
+    return host(out)
+
+
+def _gauge_force(lq, ctx, V, beta):
+    F = torch.empty((V, 4, 8), dtype=torch.float64, device="cuda")
+    lq.lq_gauge_force(ctx, F, beta)
+    return host(F)
+
+
+def _fermion_force(lq, ctx, X, kappa):
+    F = torch.empty((X.shape[0], 4, 8), dtype=torch.float64, device="cuda")
+    lq.lq_fermion_force(ctx, F, dev(X), kappa)
+    return host(F)
+
+
+# ------------------------------------------------------------ short links
+@pytest.mark.parametrize("scale", [0.3, 0.1, 1e-2, 1e-4, 1e-8])
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7)])
+def test_short_links(lq, dims, scale):
+    """Links that are a multiple of unitary ones, shorter than 1: every result to FP64 accuracy relative to
+    its own powers of the scale.  Bounds as for unitary links (128 units of 2^-53 of the largest product for
+    plaquette and gauge force, 64 for the operator, 64 * 24 for the fermion force) times those powers."""
+    from oracle.fermion import fermion_force_from_X
+    from oracle.gauge import gauge_force, plaquette
+    lat = Lattice(dims)
+    U, psi, beta = scale * gauge_exp_iA(lat, 0.3, 6), source(lat, 6), 5.6
+    kappa = 0.15 / scale
+    with _Context(lq, dims, U) as ctx:
+        P = lq.lq_plaquette(ctx)
+        F = _gauge_force(lq, ctx, lat.V, beta)
+        m = _M(lq, ctx, psi, kappa)
+        Ff = _fermion_force(lq, ctx, psi, kappa)
+    out = torch.empty(psi.shape, dtype=torch.complex128, device="cuda")
+    lq.lq_apply_MdagM_static(out, dev(U), dev(psi), dims, kappa)
+    s4 = scale ** 4
+    assert abs(P - plaquette(U, dims)) <= 128 * EPS * 3 * s4
+    assert np.abs(F - gauge_force(U, dims, beta)).max() <= 128 * EPS * beta / 3 * 18 * s4
+    top = np.abs(psi).max()
+    Y = apply_M(U, psi, dims, kappa)
+    assert np.abs(m - Y).max() <= 64 * EPS * top
+    ref = fermion_force_from_X(U, psi, dims, kappa)
+    assert np.abs(Ff - ref).max() <= 64 * 24 * EPS * 0.3 * top * np.abs(Y).max()
+    grow = 1 + 8 * 0.15 * 3
+    assert np.abs(host(out) - apply_M(U, Y, dims, kappa, True, True)).max() <= 64 * EPS * grow ** 2 * top
+
+
+def test_open_boundary_with_a_field_that_falls(lq):
+    """Temporal links of zero across the boundary and a field 1e-14 times smaller per time slice: a site next to
+    the boundary owes nothing to the large values behind the zero link.  Bound: 64 units of 2^-53 of the
+    largest component among the site and the neighbours it has a link to (all four last slices are compared)."""
+    dims = (4, 3, 4, 6)
+    lat = Lattice(dims)
+    U, psi = gauge_exp_iA(lat, 0.3, 6), source(lat, 6)
+    x = lat.coords()
+    t = x[:, 3]
+    U[t == dims[3] - 1, 3] = 0.0
+    psi = psi * (1e-14 ** t)[:, None, None]
+    with _Context(lq, dims, U) as ctx:
+        got = _M(lq, ctx, psi, 0.15)
+    out = torch.empty(psi.shape, dtype=torch.complex128, device="cuda")
+    lq.lq_apply_MdagM_static(out, dev(U), dev(psi), dims, 0.15)
+    ref = apply_M(U, psi, dims, 0.15)
+    top = np.array([np.abs(psi[t == k]).max() for k in range(dims[3])])
+    for k in range(dims[3]):
+        tol = 64 * EPS * max(top[k], top[k - 1] if k > 0 else 0.0)
+        assert np.abs(got - ref)[t == k].max() <= tol, k
+    ref = apply_M(U, ref, dims, 0.15, True, True)
+    for k in range(dims[3]):
+        tol = 64 * EPS * (1 + 8 * 0.15 * 3) ** 2 * max(top[j] for j in range(max(0, k - 2), dims[3]))
+        assert np.abs(host(out) - ref)[t == k].max() <= tol, k
