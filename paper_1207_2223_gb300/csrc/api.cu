@@ -466,9 +466,9 @@ lq_status trajectory_after_heatbath(lq_ctx* c, const lq_hmc_params* hp, double u
   lq_traj_result r{};
   const Geom& g = c->geo;
   // phi = M^dag chi; keep the start momenta and links
+  LQ_TRY(require_fix(c));
   LQ_CUDA(c, cudaMemcpyAsync(c->mom0, c->mom, sizeof(double) * 32 * (size_t)g.V, cudaMemcpyDeviceToDevice,
                              c->stream));
-  LQ_TRY(require_fix(c));
   apply_M64(c, c->chi64.ref(), c->phi64.ref(), hp->kappa, true, c->stream);
   LQ_CUDA(c, cudaMemcpyAsync(c->gauge_old, c->gauge64, gauge_bytes(GStore::F64_18, g.V), cudaMemcpyDeviceToDevice,
                              c->stream));
@@ -900,9 +900,9 @@ lq_status lq_fermion_force(lq_ctx* c, double* F, const double* X, double kappa) 
   LQ_TRY(require_gauge(c, LQ_F64));
   LQ_TRY(ensure_md_fields(c));
   const double* dX = nullptr;
+  LQ_TRY(require_fix(c));
   LQ_TRY(stage_spinor_in(c, X, &dX));
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
-  LQ_TRY(require_fix(c));
   apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
   launch_fermion_force(c->geo, fix_gauge_of(c), c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
   LQ_CUDA(c, cudaGetLastError());
@@ -916,9 +916,9 @@ lq_status lq_fermion_grad(lq_ctx* c, double* G, const double* X, double kappa) {
   LQ_TRY(require_gauge(c, LQ_F64));
   LQ_TRY(ensure_md_fields(c));
   const double* dX = nullptr;
+  LQ_TRY(require_fix(c));
   LQ_TRY(stage_spinor_in(c, X, &dX));
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
-  LQ_TRY(require_fix(c));
   apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
   const size_t bytes = sizeof(double) * 72 * (size_t)c->geo.V;
   if (is_device_ptr(G)) {
@@ -1110,9 +1110,9 @@ lq_status lq_time_fermion_force(lq_ctx* c, const double* X, double kappa, int n,
   LQ_TRY(require_gauge(c, LQ_F64));
   LQ_TRY(ensure_md_fields(c));
   const double* dX = nullptr;
+  LQ_TRY(require_fix(c));
   LQ_TRY(stage_spinor_in(c, X, &dX));
   launch_pack_spinor(c->geo, dX, SStore::F64, c->x64.ref(), c->stream);
-  LQ_TRY(require_fix(c));
   apply_M64(c, c->x64.ref(), c->y64.ref(), kappa, false, c->stream);
   launch_fermion_force(c->geo, fix_gauge_of(c), c->x64.ref(), c->y64.ref(), c->force, kappa, 0.0, false, c->stream);
   cudaEvent_t e0, e1;

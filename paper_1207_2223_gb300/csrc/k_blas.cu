@@ -47,8 +47,8 @@ __global__ void __launch_bounds__(kBS) xpay_p_kernel(int V, SpinorRef r, SpinorR
   using T = typename std::conditional<S == SStore::F64, double, float>::type;
   const T beta = (T)st->beta;
   cplx<T> rv[12], pv[12];
-  load_spinor<S, T>(r, V, s, rv);
-  load_spinor<S, T, false>(p, V, s, pv);
+  load_spinor<S, T, 0>(r, V, s, rv);
+  load_spinor<S, T, 0>(p, V, s, pv);
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     pv[k].re = fma(beta, pv[k].re, rv[k].re);

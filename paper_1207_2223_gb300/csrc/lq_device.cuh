@@ -141,7 +141,8 @@ template <> struct SpinorTraits<SStore::I16> { using half_t = void; };
 
 // ----------------------------------------------------------- spinor I/O
 // Load path of a field:
-//   1 (true)   read-only for the whole kernel: the non-coherent read-only path
+//   1 (true)   read-only for the whole kernel (one launched by launch_pdl: also not written by
+//              its predecessor): the non-coherent read-only path
 //   0 (false)  a field the kernel also writes: each element by the thread that reads it, or by other
 //              blocks before a barrier with acquire semantics (barrier.cluster) that the reader waited at
 //   2          written by other blocks of the same kernel before a device-wide barrier
@@ -524,6 +525,11 @@ __device__ __forceinline__ void su3_dagmul(const cplx<T> u[9], const cplx<T> h[3
 // one has completed.  Every kernel of the chain waits, also one that then returns at once, so
 // completion stays in order along the whole chain.  No kernel asks for its successor earlier:
 // waiting blocks then take the places of blocks still to run (12^4: 20 -> 26 us per iteration).
+// The life of such a kernel begins before the predecessor's writes are visible, so what the
+// predecessor wrote (spinors, exponent words, the solver state) is read with plain loads, which
+// neither the compiler nor the hardware takes from before the wait.  The non-coherent path (load
+// mode 1) is for what was complete before the predecessor began: links, and the flags beside them.
+// Callers convert links before the last kernel that is launched without the attribute.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // --------------------------------------------------- grid reductions

@@ -291,12 +291,12 @@ __global__ void __launch_bounds__(kDslashBlock, (EpiMinBlocks<T, Epi>::value)) d
     int c[4];
     site_coords(geo, s, c);
     cplx<T> acc[12];
-    hop_dir<0, DAG, G, SI, T, SingleIndex, true>(geo, U, in, s, c, acc);
-    hop_dir<1, DAG, G, SI, T>(geo, U, in, s, c, acc);
-    hop_dir<2, DAG, G, SI, T>(geo, U, in, s, c, acc);
-    hop_dir<3, DAG, G, SI, T>(geo, U, in, s, c, acc);
+    hop_dir<0, DAG, G, SI, T, SingleIndex, true, 0>(geo, U, in, s, c, acc);
+    hop_dir<1, DAG, G, SI, T, SingleIndex, false, 0>(geo, U, in, s, c, acc);
+    hop_dir<2, DAG, G, SI, T, SingleIndex, false, 0>(geo, U, in, s, c, acc);
+    hop_dir<3, DAG, G, SI, T, SingleIndex, false, 0>(geo, U, in, s, c, acc);
     cplx<T> ctr[12];
-    load_spinor<SI, T>(in, geo.V, s, ctr);
+    load_spinor<SI, T, 0>(in, geo.V, s, ctr);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       acc[k].re = fma(-kappa, acc[k].re, ctr[k].re);
@@ -363,7 +363,7 @@ struct EpiCG2 {
     cplx<T> rv[12], xv[12], pv[12];
     load_spinor<SR, T, false>(r, V, s, rv);
     load_spinor<SX, T, false>(x, V, s, xv);
-    load_spinor<SP, T>(p, V, s, pv);
+    load_spinor<SP, T, 0>(p, V, s, pv);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       rv[k].re = fma(-alpha, v[k].re, rv[k].re);

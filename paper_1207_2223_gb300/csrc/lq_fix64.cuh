@@ -113,7 +113,7 @@ struct SoaAccess {
   int V;
   // component `comp` of site n and the k-th after it; the link (mu, s) and its element e
   __device__ __forceinline__ const double2* site(int comp, int n) const { return psi + (size_t)comp * sstride + n; }
-  __device__ __forceinline__ double2 spin(const double2* p, int k) const { return __ldg(p + (size_t)k * sstride); }
+  __device__ __forceinline__ double2 spin(const double2* p, int k) const { return p[(size_t)k * sstride]; }
   __device__ __forceinline__ const int4* link(int mu, int s) const { return fix + (size_t)mu * 9 * V + s; }
   __device__ __forceinline__ int4 element(const int4* p, int e) const { return __ldg(p + (size_t)e * V); }
   __device__ __forceinline__ double2 element64(int mu, int e, int s) const {
@@ -445,7 +445,7 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
     }
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      const int wf = __ldg(word + f[m]), wb = __ldg(word + b[m]);
+      const int wf = word[f[m]], wb = word[b[m]];
       any |= wf | wb;
       E = max(E, max(wf & 0x7ff, wb & 0x7ff));
     }
@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(128, 4)
     for (int m = 0; m < 4; ++m) {
       f[m] = nbr_fwd(geo, s, c, m);
       b[m] = nbr_bwd(geo, s, c, m);
-      const int wf = __ldg(word + f[m]), wb = __ldg(word + b[m]);
+      const int wf = word[f[m]], wb = word[b[m]];
       any |= wf | wb;
       E = max(E, max(wf & 0x7ff, wb & 0x7ff));
     }

@@ -33,3 +33,35 @@ def test_ragged_lattices(lq, dims, prec):
     finally:
         lq.lq_destroy(ctx)
     assert np.isfinite(host(x)).all()
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (8, 8, 8, 20)])
+def test_links_replaced_before_overlapped_launches(lq, dims):
+    """New links and a call whose first stencil launch may be set up while its predecessor still runs, over and
+    over: every result is, to the bit, that of a context that only ever held those links."""
+    lat = Lattice(dims)
+    Us = [dev(gauge_exp_iA(lat, 0.3, s)) for s in (1, 2)]
+    phi = dev(source(lat, 3))
+
+    def results(ctx):
+        F = torch.empty((lat.V, 4, 8), dtype=torch.float64, device="cuda")
+        m, x = torch.empty_like(phi), torch.zeros_like(phi)
+        lq.lq_fermion_force(ctx, F, phi, 0.14)
+        lq.lq_apply_MdagM(ctx, m, phi, 0.14, lq.LQ_F64)
+        lq.lq_solve_MdagM(ctx, x, phi, 0.14, 1e-10, 60, lq.LQ_F32_12, 20)
+        return [host(v).copy() for v in (F, m, x)]
+
+    want = []
+    for U in Us:
+        ctx = lq.lq_create(dims)
+        lq.lq_gauge_set(ctx, U)
+        want.append(results(ctx))
+        lq.lq_destroy(ctx)
+    ctx = lq.lq_create(dims)
+    try:
+        for i in range(20):
+            lq.lq_gauge_set(ctx, Us[i & 1])
+            for got, ref in zip(results(ctx), want[i & 1]):
+                assert np.array_equal(got, ref)
+    finally:
+        lq.lq_destroy(ctx)
