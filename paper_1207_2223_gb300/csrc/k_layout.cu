@@ -127,8 +127,7 @@ __global__ void convert_gauge_kernel(int V, const double2* __restrict__ soa64, v
 }
 
 // FP64 links as fixed point for the operator (lq_fix64.cuh), one thread per link.  *bad is
-// set when a row or a column of a link is longer than 1 by more than 1e-3 (or not finite):
-// the bounds that keep the fixed-point sums in range assume unitary links.
+// set unless every row and column of every link is unit_length (lq_fix64.cuh).
 __global__ void __launch_bounds__(256) fix_gauge_kernel(int V, const double2* __restrict__ soa64, int4* __restrict__ out,
                                                         int* __restrict__ bad) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -147,7 +146,7 @@ __global__ void __launch_bounds__(256) fix_gauge_kernel(int V, const double2* __
   }
   bool ok = true;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 1.001f && col[k] <= 1.001f;
+  for (int k = 0; k < 3; ++k) ok = ok && unit_length(row[k]) && unit_length(col[k]);
   if (!ok) *bad = 1;
 }
 

@@ -30,7 +30,7 @@ static __device__ __align__(256) double2 g_static_scratch[(size_t)kStaticMaxSite
 // Site words of the input (ExpRange, with kBadLinks) and of M in.
 static __device__ int g_static_word[2][kStaticMaxSites];
 
-// Some link of the site is longer than a unitary one: its hops take FP64 arithmetic.
+// Some link of the site is not unitary (unit_length): its hops take FP64 arithmetic.
 constexpr int kBadLinks = 1 << 17;
 
 // The word of every site of the input and of its four links; one thread per site and link
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256) static_scan_kernel(int V, const double2* 
     }
     bool ok = true;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 1.001f && col[k] <= 1.001f;
+    for (int k = 0; k < 3; ++k) ok = ok && unit_length(row[k]) && unit_length(col[k]);
     bad = !ok;
     cplx<double> v[3];                                          // thread mu reads spin mu
 #pragma unroll

@@ -39,6 +39,12 @@ namespace lq {
 
 constexpr int kFixBlock = 256;
 
+// Whether a row or column of squared length n is that of a unitary link to 1e-3; false for NaN.  Longer
+// ones leave the range of the fixed-point sums.  Shorter ones lose digits to the fixed unit: in products
+// of links (plaquettes of links 1e-4 long 9% off), and where a link is zero, as on an open boundary,
+// because the site behind it still sets the common exponent.
+__device__ __forceinline__ bool unit_length(float n) { return n >= 0.999f && n <= 1.001f; }
+
 // round(x 2^61) of |x| < 2 as limbs (integer operations: FP64 conversions issue at 2 per clock
 // and SM; 24^3 x 32 links 166 us with them); larger or non-finite x gives some other value
 __device__ __forceinline__ int2 fix_element(double x) {
