@@ -75,7 +75,7 @@ static __device__ __noinline__ void force_link64(Geom geo, const double2* g, Spi
   im_tr_ta(Q, fa);
 }
 
-// Projection (1 + S g_mu) of the spinor of site n in fixed point with exponent word e2 (project).
+// Projection (1 + S g_mu) of the spinor of site n in fixed point with exponent word e2 (project), signed limbs.
 template <int MU, int S>
 __device__ __forceinline__ void fix_project(const double2* f, int V, int n, unsigned e2, FixRow& h0, FixRow& h1) {
   constexpr int P = S > 0 ? 0 : -1, N = ~P;
@@ -89,25 +89,25 @@ __device__ __forceinline__ void fix_project(const double2* f, int V, int n, unsi
       im[k] = fix_of(w.y, e2);
     }
     if constexpr (MU == 0) {           // p0 + S i p3, p1 + S i p2
-      h0.re[c] = fix_limbs(fix_add(re[0], 0, im[3], N));
-      h0.im[c] = fix_limbs(fix_add(im[0], 0, re[3], P));
-      h1.re[c] = fix_limbs(fix_add(re[1], 0, im[2], N));
-      h1.im[c] = fix_limbs(fix_add(im[1], 0, re[2], P));
+      h0.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[0], 0, im[3], N));
+      h0.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[0], 0, re[3], P));
+      h1.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[1], 0, im[2], N));
+      h1.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[1], 0, re[2], P));
     } else if constexpr (MU == 1) {    // p0 - S p3, p1 + S p2
-      h0.re[c] = fix_limbs(fix_add(re[0], 0, re[3], N));
-      h0.im[c] = fix_limbs(fix_add(im[0], 0, im[3], N));
-      h1.re[c] = fix_limbs(fix_add(re[1], 0, re[2], P));
-      h1.im[c] = fix_limbs(fix_add(im[1], 0, im[2], P));
+      h0.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[0], 0, re[3], N));
+      h0.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[0], 0, im[3], N));
+      h1.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[1], 0, re[2], P));
+      h1.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[1], 0, im[2], P));
     } else if constexpr (MU == 2) {    // p0 + S i p2, p1 - S i p3
-      h0.re[c] = fix_limbs(fix_add(re[0], 0, im[2], N));
-      h0.im[c] = fix_limbs(fix_add(im[0], 0, re[2], P));
-      h1.re[c] = fix_limbs(fix_add(re[1], 0, im[3], P));
-      h1.im[c] = fix_limbs(fix_add(im[1], 0, re[3], N));
+      h0.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[0], 0, im[2], N));
+      h0.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[0], 0, re[2], P));
+      h1.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[1], 0, im[3], P));
+      h1.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[1], 0, re[3], N));
     } else {                           // p0 + S p2, p1 + S p3
-      h0.re[c] = fix_limbs(fix_add(re[0], 0, re[2], P));
-      h0.im[c] = fix_limbs(fix_add(im[0], 0, im[2], P));
-      h1.re[c] = fix_limbs(fix_add(re[1], 0, re[3], P));
-      h1.im[c] = fix_limbs(fix_add(im[1], 0, im[3], P));
+      h0.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[0], 0, re[2], P));
+      h0.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[0], 0, im[2], P));
+      h1.re[c] = fix_limbs_signed(fix_add<kLimbBias>(re[1], 0, re[3], P));
+      h1.im[c] = fix_limbs_signed(fix_add<kLimbBias>(im[1], 0, im[3], P));
     }
   }
 }
@@ -116,31 +116,33 @@ __device__ __forceinline__ void fix_project(const double2* f, int V, int n, unsi
 struct ForceSums {
   long long pair[3][2], diag[3];
 };
-// + a b^dag, in units of 2^62 of the product of the operands' units
+// + a b^dag, in units of 2^60 of the product of the operands' units: two bits finer than the first
+// column, so that the four roundings of a sum are a quarter of what FP64 products cost
+__device__ __forceinline__ long long force_join(long long h, long long m) { return (h << 2) + (m >> 29); }
 __device__ __forceinline__ void force_outer(const FixRow& a, const FixRow& b, ForceSums& f) {
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const int i = q == 2 ? 1 : 0, j = q == 0 ? 1 : 2;
-    long long h = 0, m = 1 << 30;       // Im T_ij + Im T_ji, T_ij = a_i conj(b_j)
+    long long h = 0, m = 1 << 28;       // Im T_ij + Im T_ji, T_ij = a_i conj(b_j)
     fix_mac(h, m, a.im[i].x, a.im[i].y, b.re[j]);
     fix_mac(h, m, -a.re[i].x, -a.re[i].y, b.im[j]);
     fix_mac(h, m, a.im[j].x, a.im[j].y, b.re[i]);
     fix_mac(h, m, -a.re[j].x, -a.re[j].y, b.im[i]);
-    f.pair[q][0] += h + (m >> 31);
+    f.pair[q][0] += force_join(h, m);
     h = 0;
-    m = 1 << 30;                        // Re T_ij - Re T_ji
+    m = 1 << 28;                        // Re T_ij - Re T_ji
     fix_mac(h, m, a.re[i].x, a.re[i].y, b.re[j]);
     fix_mac(h, m, a.im[i].x, a.im[i].y, b.im[j]);
     fix_mac(h, m, -a.re[j].x, -a.re[j].y, b.re[i]);
     fix_mac(h, m, -a.im[j].x, -a.im[j].y, b.im[i]);
-    f.pair[q][1] += h + (m >> 31);
+    f.pair[q][1] += force_join(h, m);
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    long long h = 0, m = 1 << 30;
+    long long h = 0, m = 1 << 28;
     fix_mac(h, m, a.im[i].x, a.im[i].y, b.re[i]);
     fix_mac(h, m, -a.re[i].x, -a.re[i].y, b.im[i]);
-    f.diag[i] += h + (m >> 31);
+    f.diag[i] += force_join(h, m);
   }
 }
 // U h in half the unit of h, NEG: - U h
@@ -149,7 +151,7 @@ __device__ __forceinline__ FixRow fix_matvec(const Fix3& u, const FixRow& h) {
   FixRow r;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    long long rh = 0, rm = 1 << 30, ih = 0, im = 1 << 30;
+    long long rh = kLimbBias, rm = 1 << 30, ih = kLimbBias, im = 1 << 30;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const int4 e = u.m[3 * i + j];
@@ -158,27 +160,30 @@ __device__ __forceinline__ FixRow fix_matvec(const Fix3& u, const FixRow& h) {
       fix_mac(ih, im, e.x, e.y, h.im[j]);
       fix_mac(ih, im, e.z, e.w, h.re[j]);
     }
-    const long long wr = rh + (rm >> 31), wi = ih + (im >> 31);
-    r.re[i] = fix_limbs(NEG ? -wr : wr);
-    r.im[i] = fix_limbs(NEG ? -wi : wi);
+    r.re[i] = fix_limbs_signed(rh + (rm >> 31));
+    r.im[i] = fix_limbs_signed(ih + (im >> 31));
+    if constexpr (NEG) {
+      r.re[i] = neg2(r.re[i]);
+      r.im[i] = neg2(r.im[i]);
+    }
   }
   return r;
 }
 
 template <int MU>
 __device__ __forceinline__ void force_sums(const double2* X, const double2* Y, const int4* g, int V, int s, int xf,
-                                           unsigned ex, unsigned ey, ForceSums& f) {
+                                           unsigned ex, unsigned exf, unsigned ey, unsigned eyf, ForceSums& f) {
   const Fix3 U = load_fix3(g, V, MU, s);
   FixRow a0, a1, b0, b1;
   // - (U h(X(x+mu))) h(Y(x))^dag with (1 - g_mu)
-  fix_project<MU, -1>(X, V, xf, ex, a0, a1);
+  fix_project<MU, -1>(X, V, xf, exf, a0, a1);
   a0 = fix_matvec<true>(U, a0);
   a1 = fix_matvec<true>(U, a1);
   fix_project<MU, -1>(Y, V, s, ey, b0, b1);
   force_outer(a0, b0, f);
   force_outer(a1, b1, f);
   // + h(X(x)) (U h(Y(x+mu)))^dag with (1 + g_mu)
-  fix_project<MU, +1>(Y, V, xf, ey, b0, b1);
+  fix_project<MU, +1>(Y, V, xf, eyf, b0, b1);
   b0 = fix_matvec<false>(U, b0);
   b1 = fix_matvec<false>(U, b1);
   fix_project<MU, +1>(X, V, s, ex, a0, a1);
@@ -186,11 +191,16 @@ __device__ __forceinline__ void force_sums(const double2* X, const double2* Y, c
   force_outer(a1, b1, f);
 }
 
-// One thread per link, fixed point (lq_fix64.cuh) with one exponent for the two spinors of X and one
-// for those of Y; links whose spinors or matrix do not fit take FP64 arithmetic.  Only the sums the
-// generators ask for are formed (30 of the 36 real products of an outer product).  |h| < 2^59 and
-// |U h| < 2^59.3: four products of a sum stay below 2^62.3 in the middle column.
-// FP64 arithmetic took 212 clocks per link and SM (24^3 x 32: 1.27 ms); 0.53 ms here.
+// One thread per link, fixed point (lq_fix64.cuh) with an exponent for each of its four spinors.  The two
+// terms X(x+mu) Y(x) and X(x) Y(x+mu) need a common unit: the one with the smaller exponent sum takes
+// its X in a larger unit, which drops only bits below the other term's last.  (One exponent for both X
+// and one for both Y lost the square of the ratio where a field falls from site to site: 1.7e-15 at an
+// eighth.)  Links whose spinors or matrix do not fit take FP64 arithmetic.  Only the sums the generators
+// ask for are formed (30 of the 36 real products of an outer product).
+// |h| < 2^60.3 and |U h| < 2^59.3 as vectors: a sum of four products is below 2^57.6 in the first column,
+// the four of them 2^61.6 in units of 2^60; 2^61.3 in the middle column.
+// FP64 arithmetic took 212 clocks per link and SM (24^3 x 32: 1.27 ms); 0.54 ms here.  Error against extended
+// precision (2-norm of a link): 0.9e-16, FP64 arithmetic 1.8e-16, at any fall from site to site.
 template <bool UPDATE>
 __global__ void __launch_bounds__(128, 2) fermion_force_kernel(Geom geo, FixGauge G, SpinorRef X, SpinorRef Y, double* f,
                                                                double kappa, double eps) {
@@ -207,25 +217,33 @@ __global__ void __launch_bounds__(128, 2) fermion_force_kernel(Geom geo, FixGaug
   if (__ldg(G.bad) || ((x0 | x1 | y0 | y1) & kFixSlow)) {
     force_link64(geo, G.f64, X, Y, mu, s, xf, fa);
   } else {
-    const int EX = max(kFixMinExp, max(x0, x1)), EY = max(kFixMinExp, max(y0, y1));
-    const unsigned ex = (unsigned)EX << 21 | 0x1fffffu, ey = (unsigned)EY << 21 | 0x1fffffu;
+    // exponents of X(x+mu), Y(x) and X(x), Y(x+mu); 60 places up nothing of a term is left.  A word holds
+    // exponents to 2047: what X cannot take goes to Y.
+    int e[4] = {max(kFixMinExp, x1), max(kFixMinExp, y0), max(kFixMinExp, x0), max(kFixMinExp, y1)};
+    const int d = e[0] + e[1] - e[2] - e[3], up = min(abs(d), 60);
+    const int EX = d > 0 ? e[0] : e[2], EY = d > 0 ? e[1] : e[3];
+    const int dx = min(up, 2047 - (d > 0 ? e[2] : e[0]));
+    if (d > 0) { e[2] += dx; e[3] += up - dx; }
+    else { e[0] += dx; e[1] += up - dx; }
+    auto word = [](int E) { return (unsigned)E << 21 | 0x1fffffu; };
+    const unsigned exf = word(e[0]), ey = word(e[1]), ex = word(e[2]), eyf = word(e[3]);
     const double2 *px = static_cast<const double2*>(X.p), *py = static_cast<const double2*>(Y.p);
     ForceSums q{};
     switch (mu) {
-      case 0: force_sums<0>(px, py, G.fix, geo.V, s, xf, ex, ey, q); break;
-      case 1: force_sums<1>(px, py, G.fix, geo.V, s, xf, ex, ey, q); break;
-      case 2: force_sums<2>(px, py, G.fix, geo.V, s, xf, ex, ey, q); break;
-      default: force_sums<3>(px, py, G.fix, geo.V, s, xf, ex, ey, q); break;
+      case 0: force_sums<0>(px, py, G.fix, geo.V, s, xf, ex, exf, ey, eyf, q); break;
+      case 1: force_sums<1>(px, py, G.fix, geo.V, s, xf, ex, exf, ey, eyf, q); break;
+      case 2: force_sums<2>(px, py, G.fix, geo.V, s, xf, ex, exf, ey, eyf, q); break;
+      default: force_sums<3>(px, py, G.fix, geo.V, s, xf, ex, exf, ey, eyf, q); break;
     }
-    // unit of the sums: 2^62 * 2 * 2^(EX - 1080) * 2^(EY - 1080), in two factors that do not underflow
-    const double ux = __hiloint2double((EX - 25) << 20, 0), uy = __hiloint2double((EY - 26) << 20, 0);
+    // unit of the sums: 2^60 * 2 * 2^(EX - 1080) * 2^(EY - 1080), in two factors that do not underflow
+    const double ux = __hiloint2double((EX - 26) << 20, 0), uy = __hiloint2double((EY - 27) << 20, 0);
     const double r2 = 0.70710678118654752440 * ux, r6 = 0.40824829046386301637 * ux;
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
       for (int t = 0; t < 2; ++t) fa[(p == 0 ? 0 : p == 1 ? 3 : 5) + t] = r2 * (double)q.pair[p][t] * uy;
     fa[2] = r2 * (double)(q.diag[0] - q.diag[1]) * uy;
-    fa[7] = r6 * (double)(q.diag[0] + q.diag[1] - 2 * q.diag[2]) * uy;
+    fa[7] = r6 * ((double)(q.diag[0] - q.diag[2]) + (double)(q.diag[1] - q.diag[2])) * uy;
   }
   const double sc = 2.0 * kappa * sign;
 #pragma unroll

@@ -94,11 +94,12 @@ __device__ __forceinline__ FixTerm fix_of(double x, unsigned e2) {
   t.s = hi >> 31;
   return t;
 }
-// a + b, each negated where its mask is -1: complements, and the ones they lack in one small term
+// a + b + BIAS, a and b negated where their masks are -1: complements, and the ones they lack in one small term
+template <int BIAS = 0>
 __device__ __forceinline__ long long fix_add(FixTerm a, int ma, FixTerm b, int mb) {
   const int sa = a.s ^ ma, sb = b.s ^ mb;
   return (long long)(a.v ^ (unsigned long long)(long long)sa) + (long long)(b.v ^ (unsigned long long)(long long)sb) +
-         (long long)(unsigned)(-sa - sb);
+         (long long)(unsigned)(BIAS - sa - sb);
 }
 
 // acc += a b in the two columns: (hi, lo) limbs of a and b
@@ -108,6 +109,12 @@ __device__ __forceinline__ void fix_mac(long long& hh, long long& mm, int ah, in
   mm = mad_wide(al, b.x, mm);
 }
 __device__ __forceinline__ int2 fix_limbs(long long h) { return make_int2((int)(h >> 31), (int)h & 0x7fffffff); }
+// The limbs of h - kLimbBias with a signed low one, as the links have: a product of two numbers that both
+// come from fix_limbs drops low limbs of one sign, up to a last place each.
+constexpr int kLimbBias = 1 << 30;
+__device__ __forceinline__ int2 fix_limbs_signed(long long h) {
+  return make_int2((int)(h >> 31), ((int)h & 0x7fffffff) - kLimbBias);
+}
 
 // Where the operator reads: [chunk][element] fields with fixed-point links (V: the lattice's
 // volume, sstride: the chunk stride of the spinor field, psi its first element).

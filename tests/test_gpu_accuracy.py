@@ -102,3 +102,84 @@ def test_open_boundary_with_a_field_that_falls(lq):
     for k in range(dims[3]):
         tol = 64 * EPS * (1 + 8 * 0.15 * 3) ** 2 * max(top[j] for j in range(max(0, k - 2), dims[3]))
         assert np.abs(host(out) - ref)[t == k].max() <= tol, k
+
+
+# ------------------------------------------------------------ extended precision
+# numpy's long double (64 bits of mantissa or more on the machines this runs on); matrices by explicit sums.
+LD, CLD = np.longdouble, np.clongdouble
+
+
+def _generators():
+    T = np.zeros((8, 3, 3), CLD)
+    for a, (i, j) in ((0, (0, 1)), (3, (0, 2)), (5, (1, 2))):
+        T[a, i, j] = T[a, j, i] = 1
+        T[a + 1, i, j], T[a + 1, j, i] = -1j, 1j
+    T[2, 0, 0], T[2, 1, 1] = 1, -1
+    T[7] = np.diag([1, 1, -2]).astype(CLD) / np.sqrt(LD(3))
+    return T / np.sqrt(LD(2))
+
+
+def _mm(a, b):
+    return (a[..., :, :, None] * b[..., None, :, :]).sum(-2)
+
+
+def _dag(a):
+    return a.conj().swapaxes(-1, -2)
+
+
+def _rms_rel(F, ref):
+    """Root mean square over the links of |F - ref| / |ref| (2-norms of the eight components)."""
+    d = np.sqrt(((F.astype(LD) - ref) ** 2).sum(-1) / (ref ** 2).sum(-1))
+    return float(np.sqrt((d ** 2).mean()))
+
+
+def _ld_M(U, psi, dims, kappa):
+    from oracle.conventions import GAMMA, neighbours
+    fwd, bwd, sf, sb = neighbours(dims)
+    out = psi.copy()
+    for mu in range(4):
+        g = GAMMA[mu].astype(CLD)
+        for f, n, u, sg in ((sf, fwd, U[:, mu], -1), (sb, bwd, _dag(U[bwd[mu], mu]), 1)):
+            p = psi[n[mu]]
+            p = p + sg * _mm(np.broadcast_to(g, (len(p), 4, 4)), p)
+            out = out - LD(kappa) * f[mu][:, None, None] * _mm(p, u.swapaxes(-1, -2))
+    return out
+
+
+def _ld_fermion_force(U, X, dims, kappa):
+    """F_a = 2 kappa s Re[i Y(x)^dag (1 - g) t_a U X(x+mu) - i Y(x+mu)^dag (1 + g) U^dag t_a X(x)]."""
+    from oracle.conventions import GAMMA, neighbours
+    fwd, _, sf, _ = neighbours(dims)
+    U, X, T = U.astype(CLD), X.astype(CLD), _generators()
+    Y = _ld_M(U, X, dims, kappa)
+    F = np.zeros((len(X), 4, 8), LD)
+    for mu in range(4):
+        g = np.broadcast_to(GAMMA[mu].astype(CLD), (len(X), 4, 4))
+        Xf, Yf = X[fwd[mu]], Y[fwd[mu]]
+        a = _mm(Xf, U[:, mu].swapaxes(-1, -2))                         # U X(x+mu)
+        b = _mm(Yf + _mm(g, Yf), U[:, mu].swapaxes(-1, -2))            # U (1 + g) Y(x+mu)
+        C = _mm(a.swapaxes(-1, -2), (Y - _mm(g, Y)).conj()) - _mm(X.swapaxes(-1, -2), b.conj())
+        tr = (T[None] * C[:, None].swapaxes(-1, -2)).sum((-1, -2))     # sum_ij T_ij C_ji
+        F[:, mu] = LD(2) * LD(kappa) * sf[mu][:, None] * (1j * tr).real
+    return F
+
+
+@pytest.mark.parametrize("fall", [1.0, 2.0, 8.0, 1024.0])
+@pytest.mark.parametrize("dims", [(4, 4, 4, 6), (3, 5, 2, 7)])
+def test_fermion_force_of_a_falling_field(lq, dims, fall):
+    """X a factor smaller on every time slice (a propagator away from its source): no link's force is further
+    from extended precision than FP64 arithmetic in the order of the oracle, root mean square over the
+    links of each direction.  (Temporal links into and across the boundary, and those of the steepest fall, are
+    left out: there Y comes from one large neighbour whose part the projection takes away again, and what
+    is left are the roundings of Y to FP64, the same in any arithmetic.)"""
+    from oracle.fermion import fermion_force_from_X
+    lat = Lattice(dims)
+    U, X = gauge_exp_iA(lat, 0.3, 6), source(lat, 6)
+    X = X * (fall ** -lat.coords()[:, 3].astype(float))[:, None, None]
+    ref = _ld_fermion_force(U, X, dims, 0.15)
+    plain = fermion_force_from_X(U, X, dims, 0.15)
+    with _Context(lq, dims, U) as ctx:
+        F = _fermion_force(lq, ctx, X, 0.15)
+    for mu in range(4 if fall < 100 else 3):
+        sel = lat.coords()[:, 3] < dims[3] - 2 * (mu == 3)
+        assert _rms_rel(F[sel, mu], ref[sel, mu]) <= _rms_rel(plain[sel, mu], ref[sel, mu]), mu
