@@ -66,7 +66,13 @@ typedef enum {
 } lq_status;
 
 /* Storage / arithmetic precision of the operator and of the inner solver.
- *   LQ_F64      FP64 links (18 reals) and spinors, FP64 arithmetic
+ *   LQ_F64      FP64 links (18 reals) and spinors.  Where the links are unitary to 1e-3 the
+ *               operator adds its eight hops exactly in 64-bit fixed point, with one exponent
+ *               for the eight neighbours of a site: a component of the hopping sum is off by
+ *               a few 2^-58 of their largest component (closer than FP64 arithmetic in norm;
+ *               a component far smaller than that, say of a colour that links next to
+ *               diagonal ones hardly mix, does not keep digits of its own).  Other links,
+ *               and sites with a non-zero spin 2^6 below the largest, FP64 arithmetic.
  *   LQ_F32      FP32 links (18 reals) and spinors, FP32 arithmetic
  *   LQ_F32_12   FP32 links stored as 12 reals (row 3 rebuilt), FP32 spinors
  *   LQ_F16_12   FP16 links (12 reals), FP16 spinors scaled by a per-site FP32 norm,

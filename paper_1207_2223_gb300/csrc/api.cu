@@ -611,7 +611,7 @@ lq_status lq_destroy(lq_ctx* c) {
     if (e) cudaEventDestroy(e);
   if (c->gauge64) cudaFree(c->gauge64);
   if (c->gauge_fix) cudaFree(c->gauge_fix);
-  if (c->fix_bad) cudaFree(c->fix_bad);
+  if (c->fix_flags) cudaFree(c->fix_flags);
   for (int p = 0; p < kNumPrec; ++p)
     if (c->gauge_lo[p]) cudaFree(c->gauge_lo[p]);
   if (c->stage_in) cudaFree(c->stage_in);

@@ -24,15 +24,15 @@ static void apply_one(const Geom& g, const void* gauge, SpinorRef in, SpinorRef 
 }
 
 FixGauge fix_gauge_of(const lq_ctx* c) {
-  return FixGauge{static_cast<const int4*>(c->gauge_fix), static_cast<const double2*>(c->gauge64), c->fix_bad};
+  return FixGauge{static_cast<const int4*>(c->gauge_fix), static_cast<const double2*>(c->gauge64), c->fix_flags};
 }
 
 cudaError_t ensure_fix_gauge(lq_ctx* c, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   if (!c->gauge_fix) e = cudaMalloc(&c->gauge_fix, gauge_bytes(GStore::F64_18, c->geo.V));
-  if (e == cudaSuccess && !c->fix_bad) e = cudaMalloc(&c->fix_bad, sizeof(int));
+  if (e == cudaSuccess && !c->fix_flags) e = cudaMalloc(&c->fix_flags, kFixFlags * sizeof(int));
   if (e != cudaSuccess || c->gauge_fix_valid) return e;
-  launch_fix_gauge(c->geo, c->gauge64, c->gauge_fix, c->fix_bad, st);
+  launch_fix_gauge(c->geo, c->gauge64, c->gauge_fix, c->fix_flags, st);
   e = cudaGetLastError();
   c->gauge_fix_valid = e == cudaSuccess;
   return e;

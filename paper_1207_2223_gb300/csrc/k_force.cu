@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(128, 2) fermion_force_kernel(Geom geo, FixGaug
   const int *wx = reinterpret_cast<const int*>(X.norm), *wy = reinterpret_cast<const int*>(Y.norm);
   const int x0 = __ldg(wx + s), x1 = __ldg(wx + xf), y0 = __ldg(wy + s), y1 = __ldg(wy + xf);
   double fa[8];
-  if (__ldg(G.bad) || ((x0 | x1 | y0 | y1) & kFixSlow)) {
+  if (__ldg(G.flags + kFixBad) || ((x0 | x1 | y0 | y1) & kFixSlow)) {
     force_link64(geo, G.f64, X, Y, mu, s, xf, fa);
   } else {
     // exponents of X(x+mu), Y(x) and X(x), Y(x+mu); 60 places up nothing of a term is left.  A word holds

@@ -3,7 +3,7 @@
 // the momentum update, the link update U <- exp(i eps p) U with
 // reunitarisation, and the kinetic-energy difference.  All FP64; plaquettes and
 // staples multiply links in fixed point (lq_fixsu3.cuh), and in FP64 arithmetic
-// when some link is not unitary.
+// when some link is not unitary (staples also where the field is smooth).
 //
 // Momenta and forces are stored site-major as double [32][V], entry
 // (4 mu + ... ) -> index (8 mu + a) * V + site, for su(3) coefficient a.
@@ -93,23 +93,40 @@ __global__ void __launch_bounds__(kBS) plaquette_kernel(Geom geo, const double2*
   if (grid_sum<2>(red, rs, tot)) { out[0] = tot[0]; out[1] = tot[1]; }
 }
 
-// F_a(x, mu) = (beta/3) Im tr(t_a U_mu(x) Sigma_mu(x)), Sigma the six staples.
-// UPDATE: p -= eps F, otherwise F is stored.
-//
-// Fixed point, one thread per link.  The rows of a staple are independent chains of two
-// row-vector products, so one plane needs two links in registers (72) and one row at a time of
-// the third; the staple sum is 18 64-bit integers.  Units: staples 2^-59, their sum 2^-58 after a
-// shift, W = U Sigma 2^-57; |Sigma| <= 6 keeps every sum in 63 bits.  1404 real products per link
-// took 770 clocks per link and SM on the FP64 pipe (24^3 x 32: 4.65 ms); 1.28 ms here, now bound by
-// load latency at 8 warps per SM (168 registers for 12 warps spill: 1.36 ms; 128: 1.51 ms).
-template <bool UPDATE>
-__global__ void __launch_bounds__(128, 2) gauge_force_fix_kernel(Geom geo, const int4* __restrict__ g,
-                                                                 const int* __restrict__ bad, double* f, double beta,
-                                                                 double eps) {
-  if (__ldg(bad)) return;                              // gauge_force_kernel computes it
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 4 * geo.V) return;
-  const int mu = idx / geo.V, s = idx - mu * geo.V;
+// Im tr(t_a U_mu(x) Sigma_mu(x)) in FP64 arithmetic, Sigma the six staples.
+static __device__ __noinline__ void gauge_link64(Geom geo, const double2* g, int mu, int s, double* fa) {
+  int c[4];
+  site_coords(geo, s, c);
+  const int xm = nbr_fwd(geo, s, c, mu);
+  int cm[4] = {c[0], c[1], c[2], c[3]};
+  cm[mu] = (c[mu] + 1) % geo.L[mu];
+  M3 S;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) S.m[k] = {0.0, 0.0};
+#pragma unroll 1
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu == mu) continue;
+    const int xn = nbr_fwd(geo, s, c, nu);
+    const int xmn = nbr_bwd(geo, s, c, nu);          // x - nu
+    const int xpm_mn = nbr_bwd(geo, xm, cm, nu);     // x + mu - nu
+    // upper: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
+    M3 up = mul_dag(load_m3(g, geo.V, nu, xm), load_m3(g, geo.V, mu, xn));
+    up = mul_dag(up, load_m3(g, geo.V, nu, s));
+    add_to(S, up);
+    // lower: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu) = (U_mu(x-nu) U_nu(x+mu-nu))^dag U_nu(x-nu)
+    M3 lo = mul(load_m3(g, geo.V, mu, xmn), load_m3(g, geo.V, nu, xpm_mn));
+    lo = dag_mul(lo, load_m3(g, geo.V, nu, xmn));
+    add_to(S, lo);
+  }
+  im_tr_ta(mul(load_m3(g, geo.V, mu, s), S), fa);
+}
+
+// The same in fixed point, q_a 2^-57 without the generators' norms.  The rows of a staple are independent
+// chains of two row-vector products, so one plane needs two links in registers (72) and one row at a time
+// of the third; the staple sum is 18 64-bit integers.  Units: staples 2^-59, their sum 2^-58 after a
+// shift, W = U Sigma 2^-57; |Sigma| <= 6 keeps every sum in 63 bits.
+__device__ __forceinline__ void gauge_link_fix(const Geom& geo, const int4* __restrict__ g, int mu, int s,
+                                               long long (&q)[8]) {
   int c[4];
   site_coords(geo, s, c);
   const int xm = nbr_fwd(geo, s, c, mu);
@@ -172,55 +189,54 @@ __global__ void __launch_bounds__(128, 2) gauge_force_fix_kernel(Geom geo, const
       W[i][j][1] = ih + (im >> 31);
     }
   }
-  // f_a = Im tr(t_a W) (im_tr_ta), the sums of matrix elements exact
-  const double r2 = 0.70710678118654752440 * 0x1p-57 * (beta / 3.0), r6 = 0.40824829046386301637 * 0x1p-57 * (beta / 3.0);
-  const double fa[8] = {r2 * (double)(W[0][1][1] + W[1][0][1]), r2 * (double)(W[0][1][0] - W[1][0][0]),
-                        r2 * (double)(W[0][0][1] - W[1][1][1]), r2 * (double)(W[0][2][1] + W[2][0][1]),
-                        r2 * (double)(W[0][2][0] - W[2][0][0]), r2 * (double)(W[1][2][1] + W[2][1][1]),
-                        r2 * (double)(W[1][2][0] - W[2][1][0]),
-                        r6 * (double)(W[0][0][1] + W[1][1][1] - 2 * W[2][2][1])};
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    double* q = f + ((size_t)mu * 8 + a) * geo.V + s;
-    if (UPDATE) *q -= eps * fa[a];
-    else *q = fa[a];
-  }
+  // Im tr(t_a W) (im_tr_ta), the sums of matrix elements exact
+  q[0] = W[0][1][1] + W[1][0][1];
+  q[1] = W[0][1][0] - W[1][0][0];
+  q[2] = W[0][0][1] - W[1][1][1];
+  q[3] = W[0][2][1] + W[2][0][1];
+  q[4] = W[0][2][0] - W[2][0][0];
+  q[5] = W[1][2][1] + W[2][1][1];
+  q[6] = W[1][2][0] - W[2][1][0];
+  q[7] = W[0][0][1] + W[1][1][1] - 2 * W[2][2][1];
 }
 
-// The same in FP64 arithmetic, for links that are not unitary (*bad set).
+// F_a(x, mu) = (beta/3) Im tr(t_a U_mu(x) Sigma_mu(x)).  UPDATE: p -= eps F, otherwise F is stored.
+//
+// One thread per link, in fixed point: 1404 real products per link took 770 clocks per link and SM on the
+// FP64 pipe (24^3 x 32: 4.65 ms); 1.28 ms here, now bound by load latency at 8 warps per SM
+// (168 registers for 12 warps spill: 1.36 ms; 128: 1.51 ms).
+//
+// FP64 arithmetic where fixed point would know less than it.  Links that are not unitary (kFixBad).  Links of a
+// smooth field: an absolute error of 4e-18 in each q is 1.5e-16 of the force, as much as FP64 products
+// leave, where the largest q is 2^-3, and only near real diagonal links do FP64 products get better than
+// that, because their small imaginary parts keep their own digits.  So a link goes to FP64 arithmetic
+// with q below 2^-3 and its matrix within 2^-5 of real diagonal, and without trying fixed point
+// when every link of the lattice is that close (no kFixRough).  Error against extended precision, fixed / FP64:
+// roughness 0.3 2.9e-18 / 1.7e-16, 0.01 4.5e-17 / 1.5e-16, 0.003 1.5e-16 / 1.5e-16, 1e-4 4.5e-15 /
+// 1.5e-16.  The check of q costs nothing measurable; one of the matrix before the staples cost 26%.
 template <bool UPDATE>
-__global__ void __launch_bounds__(kBS) gauge_force_kernel(Geom geo, const double2* g, const int* bad, double* f,
-                                                          double beta, double eps) {
-  if (!__ldg(bad)) return;
+__global__ void __launch_bounds__(128, 2) gauge_force_kernel(Geom geo, FixGauge U, double* f, double beta, double eps) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= 4 * geo.V) return;
   const int mu = idx / geo.V, s = idx - mu * geo.V;
-  int c[4];
-  site_coords(geo, s, c);
-  const int xm = nbr_fwd(geo, s, c, mu);
-  int cm[4] = {c[0], c[1], c[2], c[3]};
-  cm[mu] = (c[mu] + 1) % geo.L[mu];
-  M3 S;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) S.m[k] = {0.0, 0.0};
-#pragma unroll 1
-  for (int nu = 0; nu < 4; ++nu) {
-    if (nu == mu) continue;
-    const int xn = nbr_fwd(geo, s, c, nu);
-    const int xmn = nbr_bwd(geo, s, c, nu);          // x - nu
-    const int xpm_mn = nbr_bwd(geo, xm, cm, nu);     // x + mu - nu
-    // upper: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-    M3 up = mul_dag(load_m3(g, geo.V, nu, xm), load_m3(g, geo.V, mu, xn));
-    up = mul_dag(up, load_m3(g, geo.V, nu, s));
-    add_to(S, up);
-    // lower: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu) = (U_mu(x-nu) U_nu(x+mu-nu))^dag U_nu(x-nu)
-    M3 lo = mul(load_m3(g, geo.V, mu, xmn), load_m3(g, geo.V, nu, xpm_mn));
-    lo = dag_mul(lo, load_m3(g, geo.V, nu, xmn));
-    add_to(S, lo);
-  }
-  const M3 W = mul(load_m3(g, geo.V, mu, s), S);
   double fa[8];
-  im_tr_ta(W, fa);
+  bool fp64 = __ldg(U.flags + kFixBad) || !__ldg(U.flags + kFixRough);
+  if (!fp64) {
+    long long q[8], top = 0;
+    gauge_link_fix(geo, U.fix, mu, s, q);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) top = max(top, llabs(q[a]));
+    const double r2 = 0.70710678118654752440 * 0x1p-57, r6 = 0.40824829046386301637 * 0x1p-57;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) fa[a] = (a == 7 ? r6 : r2) * (double)q[a];
+    if (top < 1ll << 54) {
+      int far = 0;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) far = max(far, fix_far(__ldg(U.fix + ((size_t)mu * 9 + k) * geo.V + s), k));
+      fp64 = far < kFixSmooth;
+    }
+  }
+  if (fp64) gauge_link64(geo, U.f64, mu, s, fa);
   const double sc = beta / 3.0;
 #pragma unroll
   for (int a = 0; a < 8; ++a) {
@@ -317,18 +333,14 @@ void launch_plaquette_diff(const Geom& g, const void* ga, const void* gb, const 
                                                        static_cast<const double2*>(gb), nullptr, rs, out);
 }
 void launch_plaquette(const Geom& g, const FixGauge& U, const ReduceScratch& rs, double* out, cudaStream_t st) {
-  plaquette_fix_kernel<<<grid_for(g.V, kFixBlock), kFixBlock, 0, st>>>(g, U.fix, U.bad, rs, out);
-  plaquette_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g, U.f64, nullptr, U.bad, rs, out);
-}
-template <bool UPDATE>
-static void gauge_force(const Geom& g, const FixGauge& U, double* f, double beta, double eps, cudaStream_t st) {
-  gauge_force_fix_kernel<UPDATE><<<grid_for(4 * g.V, 128), 128, 0, st>>>(g, U.fix, U.bad, f, beta, eps);
-  gauge_force_kernel<UPDATE><<<grid_for(4 * g.V, kBS), kBS, 0, st>>>(g, U.f64, U.bad, f, beta, eps);
+  plaquette_fix_kernel<<<grid_for(g.V, kFixBlock), kFixBlock, 0, st>>>(g, U.fix, U.flags + kFixBad, rs, out);
+  plaquette_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g, U.f64, nullptr, U.flags + kFixBad, rs, out);
 }
 void launch_gauge_force(const Geom& g, const FixGauge& U, double* f, double beta, double eps, bool update,
                         cudaStream_t st) {
-  if (update) gauge_force<true>(g, U, f, beta, eps, st);
-  else gauge_force<false>(g, U, f, beta, eps, st);
+  const int grid = grid_for(4 * g.V, 128);
+  if (update) gauge_force_kernel<true><<<grid, 128, 0, st>>>(g, U, f, beta, eps);
+  else gauge_force_kernel<false><<<grid, 128, 0, st>>>(g, U, f, beta, eps);
 }
 void launch_link_update(const Geom& g, void* gauge, const double* p, double eps, cudaStream_t st) {
   link_update_kernel<<<grid_for(4 * g.V, kBS), kBS, 0, st>>>(g, static_cast<double2*>(gauge), p, eps);

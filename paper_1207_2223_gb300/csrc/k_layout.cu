@@ -126,28 +126,37 @@ __global__ void convert_gauge_kernel(int V, const double2* __restrict__ soa64, v
   }
 }
 
-// FP64 links as fixed point for the operator (lq_fix64.cuh), one thread per link.  *bad is
-// set unless every row and column of every link is unit_length (lq_fix64.cuh).
+// FP64 links as fixed point for the operator (lq_fix64.cuh), one thread per link, and the lattice's flags
+// (FixGauge): kFixBad unless every row and column is unit_length, kFixRough if some element is not smooth.
+// One store per block and flag: one per warp to a single address would take as long as the links.
 __global__ void __launch_bounds__(256) fix_gauge_kernel(int V, const double2* __restrict__ soa64, int4* __restrict__ out,
-                                                        int* __restrict__ bad) {
+                                                        int* __restrict__ flags) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 4 * V) return;
-  const int mu = idx / V, s = idx - mu * V;
-  const double2* p = soa64 + (size_t)mu * 9 * V + s;
-  int4* o = out + (size_t)mu * 9 * V + s;
-  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    const double2 u = p[(size_t)k * V];
-    const float a = (float)u.x, b = (float)u.y, n = a * a + b * b;
-    row[k / 3] += n;
-    col[k % 3] += n;
-    o[(size_t)k * V] = fix_link(u);
-  }
   bool ok = true;
+  int far = 0;
+  if (idx < 4 * V) {
+    const int mu = idx / V, s = idx - mu * V;
+    const double2* p = soa64 + (size_t)mu * 9 * V + s;
+    int4* o = out + (size_t)mu * 9 * V + s;
+    float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && unit_length(row[k]) && unit_length(col[k]);
-  if (!ok) *bad = 1;
+    for (int k = 0; k < 9; ++k) {
+      const double2 u = p[(size_t)k * V];
+      const float a = (float)u.x, b = (float)u.y, n = a * a + b * b;
+      const int4 w = fix_link(u);
+      row[k / 3] += n;
+      col[k % 3] += n;
+      far = max(far, fix_far(w, k));
+      o[(size_t)k * V] = w;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ok = ok && unit_length(row[k]) && unit_length(col[k]);
+  }
+  const bool bad = __syncthreads_or(!ok), rough = __syncthreads_or(far >= kFixSmooth);
+  if (threadIdx.x == 0) {
+    if (bad) flags[kFixBad] = 1;
+    if (rough) flags[kFixRough] = 1;
+  }
 }
 
 template <SStore S>
@@ -194,10 +203,10 @@ void launch_pack_gauge64(const Geom& g, const double* canon, void* soa, cudaStre
   pack_gauge64_kernel<<<grid_for(g.V, kGaugeTile), 256, 0, st>>>(g.V, reinterpret_cast<const double2*>(canon),
                                                                   static_cast<double2*>(soa));
 }
-void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* bad, cudaStream_t st) {
-  cudaMemsetAsync(bad, 0, sizeof(int), st);
+void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* flags, cudaStream_t st) {
+  cudaMemsetAsync(flags, 0, kFixFlags * sizeof(int), st);
   fix_gauge_kernel<<<grid_for(4 * g.V, 256), 256, 0, st>>>(g.V, static_cast<const double2*>(soa64),
-                                                            static_cast<int4*>(fix), bad);
+                                                            static_cast<int4*>(fix), flags);
 }
 void launch_unpack_gauge64(const Geom& g, const void* soa, double* canon, cudaStream_t st) {
   unpack_gauge64_kernel<<<grid_for(g.V, kGaugeTile), 256, 0, st>>>(g.V, static_cast<const double2*>(soa),

@@ -45,6 +45,11 @@ constexpr int kFixBlock = 256;
 // because the site behind it still sets the common exponent.
 __device__ __forceinline__ bool unit_length(float n) { return n >= 0.999f && n <= 1.001f; }
 
+// How far element k of a link is from that of a real diagonal matrix, in units of 2^-30; all elements of a
+// "smooth" link are below kFixSmooth (k_gauge.cu).
+constexpr int kFixSmooth = 1 << 25;
+__device__ __forceinline__ int fix_far(int4 u, int k) { return k % 4 ? max(abs(u.x), abs(u.z)) : abs(u.z); }
+
 // round(x 2^61) of |x| < 2 as limbs (integer operations: FP64 conversions issue at 2 per clock
 // and SM; 24^3 x 32 links 166 us with them); larger or non-finite x gives some other value
 __device__ __forceinline__ int2 fix_element(double x) {
@@ -437,7 +442,7 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
                                           double kappa, const Epi& epi, int first, int stride, double (&red)[1]) {
   const SoaAccess acc{static_cast<const double2*>(in.p) + off, sstride, U.fix, U.f64, geo.V};
   const int* word = reinterpret_cast<const int*>(in.norm) + off;
-  const bool bad = __ldg(U.bad) != 0;
+  const bool bad = __ldg(U.flags + kFixBad) != 0;
   const int half = threadIdx.x & 1;
   extern __shared__ int4 fix_smem[];
   int4* stage = fix_smem + (threadIdx.x >> 1);
@@ -678,7 +683,7 @@ __global__ void __launch_bounds__(128, 4)
   if (epi.halted()) return;
   const SoaAccess acc{static_cast<const double2*>(in.p), geo.V, U.fix, U.f64, geo.V};
   const int* word = reinterpret_cast<const int*>(in.norm);
-  const bool bad = __ldg(U.bad) != 0;
+  const bool bad = __ldg(U.flags + kFixBad) != 0;
   const int lane = threadIdx.x & 31, dir = threadIdx.x >> 5;
   double red[1] = {0.0};
   for (int base = blockIdx.x * 16; base < geo.V; base += gridDim.x * 16) {

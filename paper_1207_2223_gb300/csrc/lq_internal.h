@@ -63,11 +63,12 @@ struct GraphEntry {
 
 // Links of one lattice as the fixed-point kernels read them (lq_fix64.cuh): int4 [4][9][V]
 // (re.hi, re.lo, im.hi, im.lo), the FP64 links for what takes FP64 arithmetic, and the device
-// flag "some link is not unitary".
+// flags: [kFixBad] some link is not unitary, [kFixRough] some link is not close to a real diagonal one.
+constexpr int kFixBad = 0, kFixRough = 1, kFixFlags = 2;
 struct FixGauge {
   const int4* fix;
   const double2* f64;
-  const int* bad;
+  const int* flags;
 };
 
 }  // namespace lq
@@ -86,7 +87,7 @@ struct lq_ctx {
   bool gauge_lo_valid[lq::kNumPrec] = {};
   bool gauge_set = false;
   void* gauge_fix = nullptr;             // fixed-point links of the FP64 operator (lq_fix64.cuh), built lazily
-  int* fix_bad = nullptr;                // device flag: some link is not unitary
+  int* fix_flags = nullptr;               // device flags of the links (FixGauge)
   bool gauge_fix_valid = false;
 
   // canonical-layout staging buffers (device)
@@ -146,7 +147,7 @@ void destroy_batch_work(void* w);
 // ---- layout (k_layout.cu)
 void launch_pack_gauge64(const Geom& g, const double* canon, void* soa, cudaStream_t st);
 void launch_unpack_gauge64(const Geom& g, const void* soa, double* canon, cudaStream_t st);
-void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* bad, cudaStream_t st);
+void launch_fix_gauge(const Geom& g, const void* soa64, void* fix, int* flags, cudaStream_t st);
 // the context's fixed-point links, built on `st` unless they are current
 cudaError_t ensure_fix_gauge(lq_ctx* c, cudaStream_t st);
 FixGauge fix_gauge_of(const lq_ctx* c);

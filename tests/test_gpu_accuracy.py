@@ -183,3 +183,43 @@ def test_fermion_force_of_a_falling_field(lq, dims, fall):
     for mu in range(4 if fall < 100 else 3):
         sel = lat.coords()[:, 3] < dims[3] - 2 * (mu == 3)
         assert _rms_rel(F[sel, mu], ref[sel, mu]) <= _rms_rel(plain[sel, mu], ref[sel, mu]), mu
+
+
+def _ld_gauge_force(U, dims, beta):
+    from oracle.conventions import neighbours
+    fwd, bwd, _, _ = neighbours(dims, False)
+    U = U.astype(CLD)
+    T, F = _generators(), np.zeros((len(U), 4, 8), LD)
+    for mu in range(4):
+        S = np.zeros((len(U), 3, 3), CLD)
+        for nu in range(4):
+            if nu != mu:
+                xm, xn, xb = fwd[mu], fwd[nu], bwd[nu]
+                S += _mm(_mm(U[xm, nu], _dag(U[xn, mu])), _dag(U[:, nu]))
+                S += _mm(_mm(_dag(U[xb[xm], nu]), _dag(U[xb, mu])), U[xb, nu])
+        W = _mm(U[:, mu], S)
+        F[:, mu] = LD(beta) / 3 * (T[None] * W[:, None].swapaxes(-1, -2)).sum((-1, -2)).imag
+    return F
+
+
+@pytest.mark.parametrize("rough", [0.3, 0.05, 1e-2, 3e-3, 1e-3, 1e-4, 1e-6, "half"])
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7)])
+def test_gauge_force_of_smooth_links(lq, dims, rough):
+    """Links close to 1, where the force is as small as their roughness and FP64 products keep its relative
+    accuracy: no further from extended precision than FP64 arithmetic in the order of the oracle (root mean
+    square over the links; 1.25: the spread of that figure over some hundred links).  "half": smooth on one
+    half of the time slices, rough on the other, each half of the links compared by itself."""
+    from oracle.gauge import gauge_force
+    lat = Lattice(dims)
+    U = gauge_exp_iA(lat, 0.3 if rough == "half" else rough, 6)
+    part = np.zeros(lat.V, bool)
+    if rough == "half":
+        t = lat.coords()[:, 3]
+        U[t < dims[3] // 2] = gauge_exp_iA(lat, 1e-5, 7)[t < dims[3] // 2]
+        part = (t > 0) & (t < dims[3] // 2 - 1)
+    ref, plain = _ld_gauge_force(U, dims, 5.6), gauge_force(U, dims, 5.6)
+    with _Context(lq, dims, U) as ctx:
+        F = _gauge_force(lq, ctx, lat.V, 5.6)
+    for sel in (part, ~part):
+        if sel.any():
+            assert _rms_rel(F[sel], ref[sel]) <= 1.25 * _rms_rel(plain[sel], ref[sel])
