@@ -242,21 +242,23 @@ __device__ __forceinline__ T load_spinor_raw(const SpinorRef& f, int V, int s, c
 // Exponent word of a site of an FP64 field: what the fixed-point operator (lq_fix64.cuh)
 // has to know of a neighbour before it reads it.  Bits 0-10: the largest biased exponent of
 // the site's components (0 for a zero site); kFixSlow: the site needs FP64 arithmetic
-// (non-finite values, values below 2^-953, or a spin more than 2^6 below the largest, whose
-// last bits one scale for the site would cost).
+// (non-finite values, values below 2^-953, or a non-zero spin more than 2^6 below the largest,
+// whose last bits one scale for the site would cost; a spin that is zero, as in a chirally
+// projected field, has none to lose).
 constexpr int kFixMinExp = 70;
 constexpr int kFixSlow = 1 << 16;
 struct ExpRange {
-  int mx = 0, mn = 0x7fffffff, lo = 0;     // largest and smallest spin (high words), all low words or-ed
+  int mx = 0, mn = 0x7fffffff, lo = 0;     // largest and smallest non-zero spin (high words), all low words or-ed
   __device__ __forceinline__ void spin(const cplx<double> v[3]) {
-    int m = 0;
+    int m = 0, l = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       m = max(m, max(__double2hiint(v[c].re) & 0x7fffffff, __double2hiint(v[c].im) & 0x7fffffff));
-      lo |= __double2loint(v[c].re) | __double2loint(v[c].im);
+      l |= __double2loint(v[c].re) | __double2loint(v[c].im);
     }
     mx = max(mx, m);
-    mn = min(mn, m);
+    lo |= l;
+    if (m | l) mn = min(mn, m);
   }
   __device__ __forceinline__ int word() const {
     const int E = mx >> 20, e = mn >> 20;

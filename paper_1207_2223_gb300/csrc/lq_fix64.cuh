@@ -24,6 +24,7 @@
 // What does not fit goes, site by site, through the same stencil in FP64
 // arithmetic: sites with a neighbour marked kFixSlow, and every site when
 // some link is not unitary to 1e-3 (a flag set when the links are converted).
+// A warp whose sites all go there skips the integer hops.
 //
 // Two threads per site, as in lq_dfsplit.cuh: lane 0 of a pair computes what
 // comes from the first projected colour vector of each hop, lane 1 from the
@@ -447,6 +448,9 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
   extern __shared__ int4 fix_smem[];
   int4* stage = fix_smem + (threadIdx.x >> 1);
   const int Vr = (geo.V + 15) & ~15;                     // whole warps iterate together
+  // A warp whose sites all took FP64 arithmetic looks at the next sites' words before it copies anything; the
+  // others copy first (a vote before the hops would make those wait for the words: 2 to 4% of M).
+  bool look = bad;
   for (int s0 = first; s0 < Vr; s0 += stride) {
     const bool active = s0 < geo.V;
     const int s = active ? s0 : 0;
@@ -459,7 +463,7 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
       b[m] = nbr_bwd(geo, s, c, m);
     }
     if constexpr (ASYNC) {
-      if (!bad) fix_issue<0, ASYNC>(acc, f, b, s, half, stage);
+      if (!look) fix_issue<0, ASYNC>(acc, f, b, s, half, stage);
     }
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -471,7 +475,11 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
     FixAcc a;
     fix_clear(a);
     if constexpr (ASYNC) {
-      if (!bad) fix_hops_async<DAG, ASYNC>(geo, acc, s, c, f, b, half, E, stage, a);   // every lane: warp barriers
+      if (look && !bad && !__all_sync(0xffffffffu, slow)) {
+        fix_issue<0, ASYNC>(acc, f, b, s, half, stage);
+        look = false;
+      }
+      if (!look) fix_hops_async<DAG, ASYNC>(geo, acc, s, c, f, b, half, E, stage, a);   // every lane: warp barriers
     } else if (!slow) {
       fix_hops<DAG>(geo, acc, s, c, f, b, half, E, a);
     }
@@ -480,6 +488,7 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
       split_site64<DAG>(geo, acc, s, half, &t64);
       a = t64;
     }
+    if constexpr (ASYNC) look = bad || __all_sync(0xffffffffu, slow);
     cplx<double> v[6];
     fix_finish(acc, a, s, half, slow, slow ? -kappa : -kappa * __hiloint2double((E - 56) << 20, 0), v);
     epi.apply(sstride, off + s, half, active, v, red);
@@ -627,7 +636,9 @@ __device__ __forceinline__ void fix_dir_site(const Geom& geo, const Acc& acc, in
   const unsigned e2 = (unsigned)E << 21 | 0x1fffffu;
   FixAcc a;
   fix_clear(a);
-  if (dir == 0) {
+  if (__all_sync(0xffffffffu, slow)) {
+    // the four warps hold the same 16 sites, so all of them skip the hops
+  } else if (dir == 0) {
     fix_hop<0, SF, true>(acc, f[0], s, half, ls, 0, e2, a);
     fix_hop<0, -SF, false>(acc, b[0], b[0], half, ls, 0, e2, a);
   } else if (dir == 1) {
