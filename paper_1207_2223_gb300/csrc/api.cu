@@ -60,10 +60,16 @@ void* host_direct(const lq_ctx* c, const void* p) {
 
 lq_status alloc_field(lq_ctx* c, Field& f, SStore s) {
   if (f.data) return LQ_OK;
+  void *data = nullptr, *norm = nullptr;
+  LQ_CUDA(c, cudaMalloc(&data, spinor_bytes(s, c->geo.V)));
+  if (s == SStore::F16 || s == SStore::BF16 || s == SStore::I16 || s == SStore::F64) {
+    const cudaError_t e = cudaMalloc(&norm, sizeof(float) * c->geo.V);     // norms; FP64: exponent words
+    if (e != cudaSuccess) cudaFree(data);       // a field is there with both or not at all
+    LQ_CUDA(c, e);
+  }
   f.store = s;
-  LQ_CUDA(c, cudaMalloc(&f.data, spinor_bytes(s, c->geo.V)));
-  if (s == SStore::F16 || s == SStore::BF16 || s == SStore::I16 || s == SStore::F64)
-    LQ_CUDA(c, cudaMalloc(&f.norm, sizeof(float) * c->geo.V));     // norms; FP64: exponent words
+  f.data = data;
+  f.norm = static_cast<float*>(norm);
   return LQ_OK;
 }
 
