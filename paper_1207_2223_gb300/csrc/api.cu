@@ -65,7 +65,7 @@ lq_status alloc_field(lq_ctx* c, Field& f, SStore s) {
   if (s == SStore::F16 || s == SStore::BF16 || s == SStore::I16 || s == SStore::F64) {
     const cudaError_t e = cudaMalloc(&norm, sizeof(float) * c->geo.V);     // norms; FP64: exponent words
     if (e != cudaSuccess) cudaFree(data);       // a field is there with both or not at all
-    LQ_CUDA(c, e);
+    LQ_TRY(cuda_check(c, e, "cudaMalloc of norms"));
   }
   f.store = s;
   f.data = data;
@@ -594,6 +594,7 @@ lq_status lq_create(lq_ctx** out, const int dims[4], int t_antiperiodic, void* c
   chk(cudaMalloc(&c->rs.partials, sizeof(double) * 4 * c->rs.max_blocks), "cudaMalloc partials");
   chk(cudaMalloc(&c->rs.ticket, sizeof(unsigned int) * 4), "cudaMalloc ticket");
   if (st == LQ_OK) chk(cudaMemset(c->rs.ticket, 0, sizeof(unsigned int) * 4), "cudaMemset");
+  chk(cudaMalloc(&c->fix_flags, sizeof(int) * kFixFlags), "cudaMalloc flags");
   chk(cudaMalloc(&c->state, sizeof(SolverState)), "cudaMalloc state");
   chk(cudaMallocHost(&c->state_host, sizeof(SolverState)), "cudaMallocHost");
   chk(cudaMalloc(&c->dscalar, sizeof(double) * 8), "cudaMalloc scalars");

@@ -27,13 +27,22 @@ FixGauge fix_gauge_of(const lq_ctx* c) {
   return FixGauge{static_cast<const int4*>(c->gauge_fix), static_cast<const double2*>(c->gauge64), c->fix_flags};
 }
 
+// A lattice whose second copy of the links does not fit into device memory (576 bytes a site) is marked
+// as not unitary for the life of the context: every kernel then reads the FP64 links alone.
 cudaError_t ensure_fix_gauge(lq_ctx* c, cudaStream_t st) {
-  cudaError_t e = cudaSuccess;
-  if (!c->gauge_fix) e = cudaMalloc(&c->gauge_fix, gauge_bytes(GStore::F64_18, c->geo.V));
-  if (e == cudaSuccess && !c->fix_flags) e = cudaMalloc(&c->fix_flags, kFixFlags * sizeof(int));
-  if (e != cudaSuccess || c->gauge_fix_valid) return e;
+  if (!c->gauge_fix && !c->gauge_fix_refused) {
+    const cudaError_t e = cudaMalloc(&c->gauge_fix, gauge_bytes(GStore::F64_18, c->geo.V));
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      c->gauge_fix = nullptr;
+      c->gauge_fix_refused = true;
+      return cudaMemsetAsync(c->fix_flags, 0xff, kFixFlags * sizeof(int), st);
+    }
+    if (e != cudaSuccess) return e;
+  }
+  if (c->gauge_fix_valid || c->gauge_fix_refused) return cudaSuccess;
   launch_fix_gauge(c->geo, c->gauge64, c->gauge_fix, c->fix_flags, st);
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   c->gauge_fix_valid = e == cudaSuccess;
   return e;
 }
