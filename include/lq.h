@@ -94,7 +94,7 @@ typedef struct {
   int converged;            /* 1 when true_rel_resid <= tol */
   double true_rel_resid;    /* ||phi - M^dag M x|| / ||phi||, recomputed in FP64 */
   double seconds;           /* host wall-clock of the call, from entry to the final synchronisation */
-  int64_t kernel_launches;  /* kernels this call launched (every node of a CUDA graph counts once) */
+  int64_t kernel_launches;  /* kernels this call launched (every node of a CUDA graph counts once; link conversions too) */
   int escalations;          /* times the inner precision was raised to FP32 because it stagnated */
   /* lq_solve_MdagM only (0 elsewhere): time on the context's stream (CUDA events) of staging
    * the right-hand side (host-to-device copy and packing), of the solve, and of delivering
@@ -413,19 +413,19 @@ lq_status lq_time_dslash(lq_ctx* ctx, const double* in, double kappa, int dagger
  * dims and t_antiperiodic as in lq_create, and the work is issued on
  * `cuda_stream` (a cudaStream_t) without synchronising.  out may equal in.
  *
- * The intermediate field M in is kept in one array compiled into the
- * library (12 MiB, held on every GPU that loads the library until the
- * process exits), so the lattice may have at most 65,536 sites (e.g. 16^4);
- * larger lattices return LQ_ERR_SHAPE.  All calls share that array: two
+ * The intermediate field M in and two words per site are kept in arrays compiled
+ * into the library (12.5 MiB in all, held on every GPU that loads the library
+ * until the process exits), so the lattice may have at most 65,536 sites (e.g.
+ * 16^4); larger lattices return LQ_ERR_SHAPE.  All calls share those arrays: two
  * calls whose work overlaps on the GPU (different streams, or different
  * host threads without ordering) race and give wrong results; calls on the
  * same stream are ordered and safe.  Every call overwrites the whole part
- * of the array it uses before reading it, so no state carries over.
- * The first call on each device looks up the array's device address (one
- * cudaGetSymbolAddress with that device current) and keeps it for the life
+ * of the arrays it uses before reading it, so no state carries over.
+ * The first call on each device looks up the arrays' device addresses (one
+ * cudaGetSymbolAddress each with that device current) and keeps them for the life
  * of the process; make that first call before capturing the stream into a
  * CUDA graph.  Calls after a device reset (cudaDeviceReset, or a reset of
- * the primary context) are not supported: the address kept belongs to the
+ * the primary context) are not supported: the addresses kept belong to the
  * module instance the reset unloaded.
  * Errors: LQ_ERR_ARG (null or misaligned buffer, or a buffer that is not
  * device memory: host buffers are refused, never read by a kernel),

@@ -87,6 +87,7 @@ lq_status require_gauge(lq_ctx* c, int prec) {
   if (!c->gauge_lo_valid[prec]) {
     launch_convert_gauge(c->geo, c->gauge64, gauge_store_of(prec), c->gauge_lo[prec], c->stream);
     LQ_CUDA(c, cudaGetLastError());
+    c->conversions++;
     c->gauge_lo_valid[prec] = true;
   }
   return LQ_OK;
@@ -471,6 +472,7 @@ lq_status trajectory_after_heatbath(lq_ctx* c, const lq_hmc_params* hp, double u
                                     std::chrono::steady_clock::time_point t0, int heatbath_launches) {
   lq_traj_result r{};
   const Geom& g = c->geo;
+  const int64_t converted = c->conversions;
   // phi = M^dag chi; keep the start momenta and links
   LQ_TRY(require_fix(c));
   LQ_CUDA(c, cudaMemcpyAsync(c->mom0, c->mom, sizeof(double) * 32 * (size_t)g.V, cudaMemcpyDeviceToDevice,
@@ -534,7 +536,7 @@ lq_status trajectory_after_heatbath(lq_ctx* c, const lq_hmc_params* hp, double u
   }
   LQ_TRY(require_fix(c));
   launch_plaquette(g, fix_gauge_of(c), c->rs, c->dscalar + 4, c->stream);
-  r.kernel_launches += 1;
+  r.kernel_launches += 1 + c->conversions - converted;
   LQ_TRY(read_scalars(c));
   r.plaquette = c->dscalar_host[4] / (18.0 * g.V);
   if (p) LQ_TRY(deliver_mom(c, c->mom, p));
@@ -786,9 +788,10 @@ lq_status lq_solve_MdagM(lq_ctx* c, double* x, const double* phi, double kappa, 
   launch_pack_spinor(c->geo, dphi, SStore::F64, c->phi64.ref(), c->stream);
   cudaEventRecord(c->phase_ev[1], c->stream);
   lq_solve_stats s{};
+  const int64_t converted = c->conversions;
   lq_status result = solve_internal(c, kappa, tol, maxiter, inner, reliable_every, hist_dev, hist_len, &s);
   cudaEventRecord(c->phase_ev[2], c->stream);
-  s.kernel_launches += 1;
+  s.kernel_launches += 1 + c->conversions - converted;
   bool delivered = false;
   if (result == LQ_OK || result == LQ_ERR_NOT_CONVERGED) {
     lq_status d = deliver_spinor(c, c->x64, x);

@@ -42,6 +42,7 @@ cudaError_t ensure_fix_gauge(lq_ctx* c, cudaStream_t st) {
   }
   if (c->gauge_fix_valid || c->gauge_fix_refused) return cudaSuccess;
   launch_fix_gauge(c->geo, c->gauge64, c->gauge_fix, c->fix_flags, st);
+  c->conversions++;
   const cudaError_t e = cudaGetLastError();
   c->gauge_fix_valid = e == cudaSuccess;
   return e;

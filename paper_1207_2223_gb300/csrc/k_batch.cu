@@ -507,21 +507,25 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
     if (elements > (long long)(INT_MAX / 2)) return fail(LQ_ERR_SHAPE, "batch too large for 32-bit element indices");
   }
   cudaStream_t st = c->stream;
+  int64_t converted = 0;
   // every system's links in the inner format and in fixed point (FP64 updates), converted on
   // the caller's stream
   for (int k = 0; k < n; ++k) {
     lq_ctx* ck = ctxs[k];
+    const int64_t before = ck->conversions;
     void*& lo = ck->gauge_lo[inner_prec];
     if (!lo && cudaMalloc(&lo, gauge_bytes(gauge_store_of(inner_prec), ck->geo.V)) != cudaSuccess)
       return fail(LQ_ERR_CUDA, "cudaMalloc");
     if (!ck->gauge_lo_valid[inner_prec]) {
       launch_convert_gauge(ck->geo, ck->gauge64, gauge_store_of(inner_prec), lo, st);
+      ck->conversions++;
       ck->gauge_lo_valid[inner_prec] = true;
     }
     if (ensure_fix_gauge(ck, st) != cudaSuccess) {
       cudaGetLastError();
       return fail(LQ_ERR_CUDA, "fixed-point links");
     }
+    converted += ck->conversions - before;
   }
   // workspace owned by the first context, rebuilt when the batch changes shape
   std::vector<int> key{n, nrhs, inner_prec};
@@ -584,6 +588,7 @@ extern "C" lq_status lq_solve_batch(lq_ctx** ctxs, int n, double** x, const doub
   *w->st_host = h;
   cudaMemcpyAsync(w->st, w->st_host, sizeof(BatchState), cudaMemcpyHostToDevice, st);
   lq_solve_stats s{};
+  s.kernel_launches = converted;
 
   // the initialisation (|phi|^2 per column) in one fixed launch shape, so that the sums do
   // not depend on the shape the tuner picks

@@ -33,16 +33,24 @@ __device__ __forceinline__ double site_plaquettes(const double2* g, const Geom& 
   return sum;
 }
 
+static __device__ __noinline__ double site_plaquettes64(const double2* g, Geom geo, int s) {
+  int c[4];
+  site_coords(geo, s, c);
+  return site_plaquettes(g, geo, s, c);
+}
+
 // out[0] = sum_x sum_{mu<nu} Re tr U_P with fixed-point links: per site the two-link products of
-// both paths row by row and their scalar product, summed exactly in units of 2^-58.  24^3 x 32: 1.19 ms
-// in FP64 arithmetic (1400 multiply-adds per site at 2 per clock and SM), 0.31 ms here.
-__global__ void __launch_bounds__(kFixBlock, 2) plaquette_fix_kernel(Geom geo, const int4* __restrict__ g,
-                                                                     const int* __restrict__ bad, ReduceScratch rs,
+// both paths row by row and their scalar product, summed exactly in units of 2^-58; links that are not unitary
+// in FP64 arithmetic.  24^3 x 32: 1.19 ms in FP64 arithmetic (1400 multiply-adds per site at 2 per clock and
+// SM), 0.31 ms in fixed point.
+__global__ void __launch_bounds__(kFixBlock, 2) plaquette_kernel(Geom geo, FixGauge U, ReduceScratch rs,
                                                                      double* out) {
-  if (__ldg(bad)) return;                              // plaquette_kernel computes it
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int4* __restrict__ g = U.fix;
   double red[1] = {0.0};
-  if (s < geo.V) {
+  if (__ldg(U.flags + kFixBad)) {
+    if (s < geo.V) red[0] = site_plaquettes64(U.f64, geo, s);
+  } else if (s < geo.V) {
     int c[4];
     site_coords(geo, s, c);
     long long sum = 0;
@@ -58,7 +66,7 @@ __global__ void __launch_bounds__(kFixBlock, 2) plaquette_fix_kernel(Geom geo, c
           long long a[3][2], b[3][2];
           fix_vecmat<false>(fix_row(g, geo.V, mu, s, i), p, a);
           fix_vecmat<false>(fix_row(g, geo.V, nu, s, i), q, b);
-          const FixRow x = fix_split(a), y = fix_split(b);
+          const FixRow x = fix_split_signed(a), y = fix_split(b);
           long long h = 0, m = 1 << 30;
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
@@ -75,11 +83,9 @@ __global__ void __launch_bounds__(kFixBlock, 2) plaquette_fix_kernel(Geom geo, c
   if (grid_sum<1>(red, rs, tot)) out[0] = tot[0];
 }
 
-// red[0] = sum_x sum_{mu<nu} Re tr U_P (gauge a);  red[1] = same minus for gauge b (when given).
-// only_bad, when not null: runs only if it points to a non-zero flag (links that are not unitary).
-__global__ void __launch_bounds__(kBS) plaquette_kernel(Geom geo, const double2* ga, const double2* gb,
-                                                        const int* only_bad, ReduceScratch rs, double* out) {
-  if (only_bad && !__ldg(only_bad)) return;
+// out[0] = sum_x sum_{mu<nu} Re tr U_P (gauge a), out[1] = the same minus that of gauge b, site by site; FP64.
+__global__ void __launch_bounds__(kBS) plaquette_diff_kernel(Geom geo, const double2* ga, const double2* gb,
+                                                             ReduceScratch rs, double* out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   double red[2] = {0.0, 0.0};
   if (s < geo.V) {
@@ -87,7 +93,7 @@ __global__ void __launch_bounds__(kBS) plaquette_kernel(Geom geo, const double2*
     site_coords(geo, s, c);
     const double pa = site_plaquettes(ga, geo, s, c);
     red[0] = pa;
-    if (gb) red[1] = pa - site_plaquettes(gb, geo, s, c);
+    red[1] = pa - site_plaquettes(gb, geo, s, c);
   }
   double tot[2];
   if (grid_sum<2>(red, rs, tot)) { out[0] = tot[0]; out[1] = tot[1]; }
@@ -329,12 +335,11 @@ __global__ void __launch_bounds__(kBS) kinetic_diff_kernel(int V, const double* 
 
 void launch_plaquette_diff(const Geom& g, const void* ga, const void* gb, const ReduceScratch& rs, double* out,
                            cudaStream_t st) {
-  plaquette_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g, static_cast<const double2*>(ga),
-                                                       static_cast<const double2*>(gb), nullptr, rs, out);
+  plaquette_diff_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g, static_cast<const double2*>(ga),
+                                                            static_cast<const double2*>(gb), rs, out);
 }
 void launch_plaquette(const Geom& g, const FixGauge& U, const ReduceScratch& rs, double* out, cudaStream_t st) {
-  plaquette_fix_kernel<<<grid_for(g.V, kFixBlock), kFixBlock, 0, st>>>(g, U.fix, U.flags + kFixBad, rs, out);
-  plaquette_kernel<<<grid_for(g.V, kBS), kBS, 0, st>>>(g, U.f64, nullptr, U.flags + kFixBad, rs, out);
+  plaquette_kernel<<<grid_for(g.V, kFixBlock), kFixBlock, 0, st>>>(g, U, rs, out);
 }
 void launch_gauge_force(const Geom& g, const FixGauge& U, double* f, double beta, double eps, bool update,
                         cudaStream_t st) {

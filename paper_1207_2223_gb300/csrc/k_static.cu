@@ -21,8 +21,8 @@
 namespace lq {
 
 // Largest lattice the array holds: 65,536 sites (for example 16^4), one FP64
-// spinor of 12 complex numbers per site = 12 MiB.  Every GPU that loads the
-// library holds this array until the process exits.
+// spinor of 12 complex numbers per site = 12 MiB, and two words per site = 0.5 MiB.
+// Every GPU that loads the library holds these arrays until the process exits.
 constexpr int kStaticMaxSites = 65536;
 
 static __device__ __align__(256) double2 g_static_scratch[(size_t)kStaticMaxSites * 12];

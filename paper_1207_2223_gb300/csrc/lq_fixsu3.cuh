@@ -2,8 +2,8 @@
 // two limbs of 31 bits) multiplied row by row with 32 x 32 + 64 bit integer
 // multiply-adds, 32 times the rate of the FP64 pipe.  A row-vector times a link
 // keeps its unit: with the vector's unit 2^-q the product is exact in units of
-// 2^-(q - 1) up to the dropped product of the low limbs (mean zero, a quarter of
-// the last place) and one rounding.  Elements of products of unitary matrices
+// 2^-(q - 1) up to the dropped product of the low limbs (mean zero, as one of the
+// two has signed low limbs, and at most half a last place) and one rounding.  Elements of products of unitary matrices
 // are at most 1, so a chain of two products starting from a link stays at 59
 // fractional bits, 2^-6 of the last place of FP64.
 #pragma once
@@ -78,6 +78,17 @@ __device__ __forceinline__ FixRow fix_split(const long long (&w)[3][2]) {
   for (int k = 0; k < 3; ++k) {
     r.re[k] = fix_limbs(w[k][0]);
     r.im[k] = fix_limbs(w[k][1]);
+  }
+  return r;
+}
+
+// the same with signed low limbs, for an operand whose partner comes from fix_split
+__device__ __forceinline__ FixRow fix_split_signed(const long long (&w)[3][2]) {
+  FixRow r;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    r.re[k] = fix_limbs_signed(w[k][0] + kLimbBias);
+    r.im[k] = fix_limbs_signed(w[k][1] + kLimbBias);
   }
   return r;
 }

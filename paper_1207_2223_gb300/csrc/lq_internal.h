@@ -89,6 +89,7 @@ struct lq_ctx {
   void* gauge_fix = nullptr;             // fixed-point links of the FP64 operator (lq_fix64.cuh), built lazily
   int* fix_flags = nullptr;               // device flags of the links (FixGauge)
   bool gauge_fix_valid = false;
+  int64_t conversions = 0;               // link conversions launched so far (kernel_launches of the calls)
   bool gauge_fix_refused = false;        // no memory for them: FP64 arithmetic throughout
 
   // canonical-layout staging buffers (device)
