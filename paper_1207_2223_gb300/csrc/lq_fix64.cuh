@@ -683,8 +683,11 @@ __device__ __forceinline__ void fix_dir_site(const Geom& geo, const Acc& acc, in
 }
 
 // Small lattices leave most of the chip idle, and a pass takes as long as one thread needs for its
-// eight hops: split by direction.  FP64 CG, us per iteration, split against two threads per site:
-// 4^4 24 / 41, 8^4 31 / 41, 8^3 x 16 34 / 40, 10^4 45 / 41.
+// eight hops: split by direction.  Split against two threads per site, us: M 4^4 5.2 / 9.7, 8^4 8.6 / 9.9,
+// 8^3 x 16 9.1 / 10.1, 8^2 x 12^2 9.2 / 10.2, 8 x 12^3 16.3 / 13.3; static M^dag M 4^4 22.8 / 51.8, 8^4 34.9 / 51.3,
+// 8^3 x 16 34.9 / 52.0, 8^2 x 12^2 34.9 / 51.9, 8 x 12^3 58.9 / 53.3; an FP64 CG iteration, whose reductions want
+// few blocks, 4^4 24.0 / 32.6, 8^4 31.6 / 32.4, 8^3 x 12 33.7 / 33.5, 8^3 x 16 34.3 / 32.9.  One line for all
+// three, at a size where it costs the iteration 4% and saves the others 10 and 33%.
 constexpr int kFixDirSites = 8192;
 template <bool DAG, class Epi>
 __global__ void __launch_bounds__(128, 4)

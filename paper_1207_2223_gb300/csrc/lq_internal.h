@@ -197,9 +197,13 @@ void cg64_iteration(lq_ctx* c, double kappa, cudaStream_t stream);
 void cg64_true_residual(lq_ctx* c, double kappa, int store_lo_prec, cudaStream_t stream);
 
 // ---- CG iterations of a small lattice inside one cluster, n of them or until halted (k_cgcluster.cu)
-// Up to this many sites 16 SMs are faster than all of them with kernel boundaries (us per iteration of
-// FP16 solves, cluster against kernels: 4^4 14.1 / 18.0, 8^4 13.9 / 17.1, 8^3 x 12 16.5 / 18.5,
-// 8^3 x 16 19.3 / 17.9).
+// Up to this many sites 16 SMs are faster than all of them with kernel boundaries, in every format (us per
+// iteration of a solve, cluster against kernels):
+//              F32          F32-12       F16          BF16         I16
+//   4^4        11.9 / 18.9  12.4 / 18.8  13.1 / 19.4  13.5 / 23.1  13.2 / 20.2
+//   8^4        14.5 / 18.0  14.3 / 17.9  13.8 / 17.6  14.4 / 19.3  13.9 / 18.3
+//   8^3 x 12   17.0 / 17.8  16.6 / 17.6  16.2 / 18.1  16.1 / 18.3  16.6 / 18.7
+//   8^3 x 16   19.8 / 17.4  19.2 / 17.2  19.1 / 17.4  18.8 / 17.2  19.8 / 18.0
 constexpr int kClusterMaxSites = 6144;
 bool cluster_takes(const lq_ctx* c, int prec);
 cudaError_t cg_cluster_iterations(lq_ctx* c, int prec, int n, double kappa, cudaStream_t stream);
