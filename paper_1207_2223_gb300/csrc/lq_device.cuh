@@ -417,13 +417,9 @@ __device__ __forceinline__ void load_link_q16(const GaugeRef& g, int V, int mu, 
   }
 }
 
-// -x by flipping the sign bit (an integer operation: exact, and off the FP64 pipe for doubles)
-__device__ __forceinline__ double flip_sign(double x) {
-  return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
-}
+// -x by flipping the sign bit (an integer operation: exact)
 __device__ __forceinline__ float flip_sign(float x) { return __int_as_float(__float_as_int(x) ^ (int)0x80000000); }
-__device__ __forceinline__ df64 flip_sign(df64 x) { return df64(flip_sign(x.hi), flip_sign(x.lo)); }
-template <typename T> __device__ __forceinline__ void negate3(cplx<T> h[3]) {
+__device__ __forceinline__ void negate3(cplx<float> h[3]) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) h[k] = {flip_sign(h[k].re), flip_sign(h[k].im)};
 }
