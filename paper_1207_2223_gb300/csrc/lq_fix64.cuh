@@ -409,27 +409,40 @@ __device__ __forceinline__ void fix_hops_async(const Geom& geo, const SoaAccess&
 
 // The lane's two spins of M psi at site s: centre + ks * hopping sums.  Each lane completes the
 // lower spin it keeps with the partner's sums (both lanes of a pair took the same path; every lane
-// of the warp calls).  slow: the sums are FP64 bit patterns.
+// of the warp calls).  slow: the sums are FP64 bit patterns.  One branch around the twelve values, not one
+// around each: those became selections, and the conversions of the integer side took 24 of 902 places on
+// the FP64 pipe that bounds slow sites (24^3 x 32 705 -> 684 us, 16^4 125 -> 121).
 template <class Acc>
 __device__ __forceinline__ void fix_finish(const Acc& in, const FixAcc& a, int s, int half, bool slow, double ks,
                                            cplx<double> v[6]) {
+  long long got[3][2];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) got[i][q] = __shfl_xor_sync(0xffffffffu, a.give[i][q], 1);
+  double up[3][2], lo[3][2];
+  if (slow) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        up[i][q] = __longlong_as_double(a.up[i][q]);
+        lo[i][q] = __longlong_as_double(a.keep[i][q]) + __longlong_as_double(got[i][q]);
+      }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        up[i][q] = (double)a.up[i][q];
+        lo[i][q] = (double)(a.keep[i][q] + got[i][q]);
+      }
+  }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const double2 c0 = in.spin(in.site(3 * half, s), i), c1 = in.spin(in.site(3 * (half + 2), s), i);
-    double lo[2], hi[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const long long got = __shfl_xor_sync(0xffffffffu, a.give[i][q], 1);
-      if (slow) {
-        hi[q] = __longlong_as_double(a.up[i][q]);
-        lo[q] = __longlong_as_double(a.keep[i][q]) + __longlong_as_double(got);
-      } else {
-        hi[q] = (double)a.up[i][q];
-        lo[q] = (double)(a.keep[i][q] + got);
-      }
-    }
-    v[i] = {fma(ks, hi[0], c0.x), fma(ks, hi[1], c0.y)};
-    v[3 + i] = {fma(ks, lo[0], c1.x), fma(ks, lo[1], c1.y)};
+    v[i] = {fma(ks, up[i][0], c0.x), fma(ks, up[i][1], c0.y)};
+    v[3 + i] = {fma(ks, lo[i][0], c1.x), fma(ks, lo[i][1], c1.y)};
   }
 }
 
