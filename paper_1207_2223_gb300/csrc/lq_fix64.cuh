@@ -458,8 +458,8 @@ __device__ __forceinline__ void fix_sites(const Geom& geo, const FixGauge& U, co
   const int* word = reinterpret_cast<const int*>(in.norm) + off;
   const bool bad = __ldg(U.flags + kFixBad) != 0;
   const int half = threadIdx.x & 1;
-  extern __shared__ int4 fix_smem[];
-  int4* stage = fix_smem + (threadIdx.x >> 1);
+  extern __shared__ int4 fix_stages[];
+  int4* stage = fix_stages + (threadIdx.x >> 1);
   const int Vr = (geo.V + 15) & ~15;                     // whole warps iterate together
   // A warp whose sites all took FP64 arithmetic looks at the next sites' words before it copies anything; the
   // others copy first (a vote before the hops would make those wait for the words: 2 to 4% of M).
