@@ -165,7 +165,7 @@ def _ld_fermion_force(U, X, dims, kappa):
 
 
 @pytest.mark.parametrize("fall", [1.0, 2.0, 8.0, 1024.0])
-@pytest.mark.parametrize("dims", [(4, 4, 4, 6), (3, 5, 2, 7)])
+@pytest.mark.parametrize("dims", [(4, 4, 4, 6), (3, 5, 2, 7), (8, 6, 5, 9)])
 def test_fermion_force_of_a_falling_field(lq, dims, fall):
     """X a factor smaller on every time slice (a propagator away from its source): no link's force is further
     from extended precision than FP64 arithmetic in the order of the oracle, root mean square over the
@@ -203,7 +203,7 @@ def _ld_gauge_force(U, dims, beta):
 
 
 @pytest.mark.parametrize("rough", [0.3, 0.05, 1e-2, 3e-3, 1e-3, 1e-4, 1e-6, "half"])
-@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7)])
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (3, 5, 2, 7), (8, 6, 5, 9)])
 def test_gauge_force_of_smooth_links(lq, dims, rough):
     """Links close to 1, where the force is as small as their roughness and FP64 products keep its relative
     accuracy: no further from extended precision than FP64 arithmetic in the order of the oracle (root mean
