@@ -130,8 +130,8 @@ lq_status lq_set_stream(lq_ctx* ctx, void* cuda_stream);
  *                       between two reliable updates as one launch either way.
  *   LQ_OPT_DF64_UPDATES accepted (0 or 1) and without effect: every reliable update of a
  *                       mixed-precision solve recomputes the residual with the FP64 operator,
- *                       which on this part is faster than the double-float one (0.7 against
- *                       0.85 ns per site) and certifies the solution by itself.
+ *                       which on this part is faster than the double-float one (M 0.56 against
+ *                       0.71 ns per site) and certifies the solution by itself.
  *   LQ_OPT_PAIR_SITES   0 (default): one site per thread; 1: with LQ_I16_12 and an even
  *                       L_t, the operator and the CG passes apply the stencil at two sites
  *                       per thread (x and x + L_t/2 in time) with packed FP32x2 arithmetic.

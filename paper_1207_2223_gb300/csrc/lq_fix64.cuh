@@ -12,7 +12,7 @@
 //   spinor   P = p 2^(1080 - E) truncated  = ph 2^31 + pl   (0 <= pl < 2^31)
 // with E the largest biased exponent among the eight neighbour sites (written per site with
 // the field, ExpRange).  A product is three multiply-adds, uh ph 2^62 + (uh pl + ul ph) 2^31;
-// the dropped ul pl has mean zero and is at most a quarter of the last place kept.  A row is
+// the dropped ul pl has mean zero and is at most half of the last place kept.  A row is
 // rounded once, the eight hops add exactly, the result is converted to FP64 once, and kappa
 // and the centre enter in FP64.  Against a computation in extended precision the result is
 // 1.6 times closer than that of FP64 arithmetic (2-norm 5.4e-17 against 9.1e-17 at 8^4).
